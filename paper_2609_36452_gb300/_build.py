@@ -16,7 +16,7 @@ LIB = os.path.join(HERE, "librpd.so")
 # the checked build (-DRPD_CHECKS: device-side bounds checks latch RPD_ERR_CHECK), for tests
 CHECKED_BUILD = os.path.join(HERE, "_build_checked")
 CHECKED_LIB = os.path.join(HERE, "librpd_checked.so")
-SOURCES = ["rpd_host.cu", "k_gather_norm.cu", "k_head_stats.cu", "k_merge_commit.cu",
+SOURCES = ["rpd_host.cu", "k_compact.cu", "k_head_stats.cu", "k_merge_commit.cu",
            "rpd_noalloc.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

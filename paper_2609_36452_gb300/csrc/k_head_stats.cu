@@ -29,6 +29,8 @@
 
 #include "ptx.cuh"
 #include "rpd_internal.h"
+#include "step_epilogue.cuh"
+#include "step_prologue.cuh"
 
 namespace rpd {
 namespace {
@@ -48,8 +50,7 @@ struct TileWalk {
         num_n = (V + kTileN - 1) / kTileN;
         splits = g;
         units = num_m * splits;
-        const long long tile_bytes = static_cast<long long>(tile_rows) * d * 2;
-        band = static_cast<int>(kBandBytes / tile_bytes);
+        band = static_cast<int>(kBandBytes / 2) / tile_rows / d;
         band = max(1, min(num_m, band));
     }
     __device__ __forceinline__ void unit(int u, int &m, int &g, int &n0, int &n1) const {
@@ -60,8 +61,9 @@ struct TileWalk {
         const int in_band = min(band, num_m - m0);
         m = m0 + r % in_band;
         g = r / in_band;
-        n0 = static_cast<int>((static_cast<long long>(g) * num_n) / splits);
-        n1 = static_cast<int>((static_cast<long long>(g + 1) * num_n) / splits);
+        // at most a few hundred splits of at most 2^23 tiles: the products fit 32 bits
+        n0 = static_cast<int>(static_cast<unsigned>(g) * num_n / splits);
+        n1 = static_cast<int>(static_cast<unsigned>(g + 1) * num_n / splits);
     }
 };
 
@@ -153,6 +155,7 @@ struct HeadSmem {
     uint32_t *tmem_slot;
     volatile int *abort_flag;
     volatile int *unit_ring;  // [kUnitRing] claimed unit indices
+    MaskMap map;              // the compaction (and the pass) of this CTA
 };
 
 __device__ __forceinline__ HeadSmem carve_smem(uint8_t *raw) {
@@ -173,12 +176,196 @@ __device__ __forceinline__ HeadSmem carve_smem(uint8_t *raw) {
     s.tmem_slot = reinterpret_cast<uint32_t *>(s.chunk_free + kTmemCols / 32);
     s.abort_flag = reinterpret_cast<volatile int *>(s.tmem_slot + 1);
     s.unit_ring = s.abort_flag + 1;
+    s.map.words = reinterpret_cast<uint32_t *>(base + kHeadRegionBytes + kHeadBarrierBytes);
+    s.map.before = reinterpret_cast<uint16_t *>(s.map.words + kMaskWords);
+    s.map.pass = reinterpret_cast<PassInfo *>(s.map.before + kMaskWords + 8);
     return s;
 }
 
 static_assert((2 * kSwapMaxStages + 6 + 2 * kUnitRing + kTmemCols / 32) * 8 + 8 + 4 * kUnitRing <=
                   kHeadBarrierBytes,
               "barrier region");
+
+// Barriers and tensor memory of a CTA, the same for both tilings so that neither depends on the
+// pass.  full[s] lives in the even CTA and receives both CTAs' TMA completions; empty[s],
+// acc_full[a] and drain receive multicast commits from the MMA issuer in both CTAs; acc_empty[a]
+// lives in the even CTA and counts the 8 epilogue warps of both CTAs (with pair tiles half of
+// the warps work and each arrives twice); unit_empty[i] also counts the even CTA's MMA issuer and
+// the odd CTA's producer.
+__device__ __forceinline__ void init_barriers(const HeadSmem &sm) {
+    for (int i = 0; i < kSwapMaxStages; ++i) {
+        mbar_init(&sm.full[i], 1);
+        mbar_init(&sm.empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+        mbar_init(&sm.acc_full[i], 1);
+        mbar_init(&sm.acc_empty[i], 2 * kSwapEpiWarps);
+    }
+    for (int i = 0; i < kUnitRing; ++i) {
+        mbar_init(&sm.unit_full[i], 1);
+        mbar_init(&sm.unit_empty[i], 2 + 2 * kSwapEpiWarps);
+    }
+    // ring tiles: a chunk is read by one warp per TMEM sub-partition in each CTA
+    for (uint32_t i = 0; i < kTmemCols / 32; ++i) mbar_init(&sm.chunk_free[i], 8);
+    mbar_init(sm.epi, 32 * kSwapEpiWarps);
+    mbar_init(sm.drain, 1);
+    *sm.abort_flag = 0;
+    fence_mbar_init();
+}
+
+// An epilogue warp's acquire of the other CTAs' inv_rms, long before its first tile is done.
+__device__ __forceinline__ bool wait_for_rows(const HeadParams &p, const HeadSmem &sm, int rows) {
+    return counter_wait(&p.meta[kMetaRowsDone], rows, sm.abort_flag, p.wait_limit_ns, 500);
+}
+
+// The TMA producer's claim of the next work unit (-1: none left): the even CTA takes it from the
+// pass's counter - its first claim was made before the pass was known - and hands it to both
+// CTAs' rings.  Returns false if a wait gave up.
+__device__ __forceinline__ bool claim_unit(const HeadParams &p, const HeadSmem &sm, uint32_t rank,
+                                           int units, UnitCursor &uc, int &first, int &u) {
+    volatile int *unit_ring = sm.unit_ring;
+    if (rank == 0) {
+        const uint32_t unit_full1 = mapa_shared(smem_u32(&sm.unit_full[0]), 1);
+        const uint32_t unit_ring1 = mapa_shared(smem_u32(const_cast<int *>(&unit_ring[0])), 1);
+        if (!mbar_wait_bounded_cluster(&sm.unit_empty[uc.slot], uc.phase ^ 1u, sm.abort_flag, p.wait_limit_ns))
+            return false;
+        const int claimed = first >= 0 ? first : atomicAdd(&p.meta[kMetaUnitNext], 1);
+        first = -1;
+        u = claimed < units ? claimed : -1;
+        unit_ring[uc.slot] = u;
+        st_shared_cluster(unit_ring1 + static_cast<uint32_t>(uc.slot * sizeof(int)), u);
+        mbar_arrive(&sm.unit_full[uc.slot]);
+        mbar_arrive_cluster(unit_full1 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
+    } else {
+        const uint32_t unit_empty0 = mapa_shared(smem_u32(&sm.unit_empty[0]), 0);
+        if (!mbar_wait_bounded_cluster(&sm.unit_full[uc.slot], uc.phase, sm.abort_flag, p.wait_limit_ns))
+            return false;
+        u = unit_ring[uc.slot];
+        mbar_arrive_cluster(unit_empty0 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
+    }
+    uc.advance();
+    return true;
+}
+
+// What one CTA's TMA producer copies: per stage 128 head rows x 64 columns (w_off bytes into the
+// stage) and this CTA's rows of u x 64 columns (u_off), u_rows * m + u_row0 on for row tile m.
+struct Copies {
+    const CUtensorMap *w, *u;
+    int stages, stage_bytes, w_off, u_off, u_rows, u_row0;
+};
+
+// One tile's K-steps kb0 .. num_kb - 1; returns how many were issued (fewer if a wait gave up).
+// The loop is kept as tight as it gets: the same copies issued
+// from a loop with a few more branches and address computations in it made whole first-step and
+// mid-decode passes 1.5 to 3 % slower.  kOnce: drop the head tile from L2 first (see produce).
+template <bool kOnce>
+__device__ __forceinline__ int copy_tile(const HeadParams &p, const HeadSmem &sm, const Copies &c,
+                                          uint32_t rank, uint32_t full0, uint64_t evict_first, int n,
+                                          int u_row, int kb0, int num_kb, int &stage, uint32_t &phase) {
+    // block (2n + rank, kb) of the tiled copy (128 contiguous rows of 64), or the same rows and
+    // columns of W in place
+    const int block = 2 * n + static_cast<int>(rank);
+    const int dx = p.w_tiled ? 0 : kTileK, dy = p.w_tiled ? kPairHalfRows : 0;
+    int x = kb0 * dx;
+    int y = (p.w_tiled ? block * num_kb + kb0 : block) * kPairHalfRows;
+    int kb = kb0;
+    for (; kb < num_kb; ++kb, x += dx, y += dy) {
+        if (!mbar_wait_bounded(&sm.empty[stage], phase ^ 1u, sm.abort_flag, p.wait_limit_ns)) break;
+        if (rank == 0) mbar_arrive_expect_tx(&sm.full[stage], 2 * c.stage_bytes);
+        const uint32_t bar = full0 + static_cast<uint32_t>(stage * sizeof(uint64_t));
+        uint8_t *st = sm.ring + stage * c.stage_bytes;
+        tma_load_2d_pair(st + c.u_off, c.u, bar, kb * kTileK, u_row);
+        if (kOnce)
+            tma_load_2d_pair_hint(st + c.w_off, c.w, bar, x, y, evict_first);
+        else
+            tma_load_2d_pair(st + c.w_off, c.w, bar, x, y);
+        if (++stage == c.stages) {
+            stage = 0;
+            phase ^= 1u;
+        }
+    }
+    return kb - kb0;
+}
+
+// The first stages of a CTA's first tile, while the ring is empty and the rows of u are still
+// being gathered: the head tiles at once, the rows once all of them are counted.  Returns the
+// K-steps issued, or -1 if the wait gave up.
+__device__ __forceinline__ int copy_ahead(const HeadParams &p, const HeadSmem &sm, const Copies &c,
+                                          uint32_t rank, uint32_t full0, bool once, uint64_t evict_first,
+                                          int n, int u_row, int rows, int num_kb) {
+    const int ahead = min(c.stages, num_kb);
+    const int block = 2 * n + static_cast<int>(rank);
+    for (int s = 0; s < ahead; ++s) {
+        if (rank == 0) mbar_arrive_expect_tx(&sm.full[s], 2 * c.stage_bytes);
+        const uint32_t bar = full0 + static_cast<uint32_t>(s * sizeof(uint64_t));
+        uint8_t *dst = sm.ring + s * c.stage_bytes + c.w_off;
+        const int x = p.w_tiled ? 0 : s * kTileK;
+        const int y = (p.w_tiled ? block * num_kb + s : block) * kPairHalfRows;
+        if (once)
+            tma_load_2d_pair_hint(dst, c.w, bar, x, y, evict_first);
+        else
+            tma_load_2d_pair(dst, c.w, bar, x, y);
+    }
+    if (!counter_wait(&p.meta[kMetaRowsDone], rows, sm.abort_flag, p.wait_limit_ns)) return -1;
+    proxy_fence();
+    for (int s = 0; s < ahead; ++s)
+        tma_load_2d_pair(sm.ring + s * c.stage_bytes + c.u_off, c.u,
+                         full0 + static_cast<uint32_t>(s * sizeof(uint64_t)), s * kTileK, u_row);
+    return ahead;
+}
+
+// The TMA producer of one CTA (one thread); returns the units it has taken.
+//
+// With a single row tile every head tile is read once and is dropped from L2 first, which keeps
+// the hidden rows, the partials and the code of the step's other phases there from one step to
+// the next: 171.5 -> 166.4 us at 20 rows (LLaDA head), of which 3 us after the last tile.  Several
+// row tiles re-read a head tile at slightly different times: with that policy, and with an
+// explicit normal one instead of none, first-step and serving passes were 1.5 % slower.
+__device__ __forceinline__ int produce(const HeadParams &p, const HeadSmem &sm, const Copies &c,
+                                       uint32_t rank, const TileWalk &tw, int rows, int num_kb, int first) {
+    const uint32_t full0 = mapa_shared(smem_u32(&sm.full[0]), 0);
+    const uint64_t evict_first = l2_evict_first();
+    const bool once = tw.num_m == 1;
+    int taken = 0;
+    int stage = 0;
+    uint32_t phase = 0;
+    long long fills = 0;
+    bool ok = true;
+    UnitCursor uc;
+    proxy_fence();  // the compaction's scratch lay in the ring
+    while (ok) {
+        int u;
+        if (!claim_unit(p, sm, rank, tw.units, uc, first, u) || u < 0) break;
+        int m, g, n0, n1;
+        tw.unit(u, m, g, n0, n1);
+        const int u_row = m * c.u_rows + c.u_row0;
+        int kb0 = 0;
+        if (taken++ == 0) {
+            kb0 = copy_ahead(p, sm, c, rank, full0, once, evict_first, n0, u_row, rows, num_kb);
+            fills = kb0 < 0 ? min(c.stages, num_kb) : kb0;
+            if (kb0 < 0) break;
+            if (kb0 == c.stages)
+                phase = 1u;
+            else
+                stage = kb0;
+        }
+        for (int n = n0; ok && n < n1; ++n, kb0 = 0) {
+            const int issued =
+                once ? copy_tile<true>(p, sm, c, rank, full0, evict_first, n, u_row, kb0, num_kb, stage, phase)
+                     : copy_tile<false>(p, sm, c, rank, full0, evict_first, n, u_row, kb0, num_kb, stage, phase);
+            fills += issued;
+            ok = issued == num_kb - kb0;
+        }
+    }
+    // Drain: a stage's copies have landed once the MMAs that read it have completed, which the
+    // multicast commit on empty[s] reports in this CTA.
+    for (int s = 0; s < c.stages; ++s) {
+        const long long n_s = fills / c.stages + (s < fills % c.stages ? 1 : 0);
+        if (n_s > 0)
+            mbar_wait_drain(&sm.empty[s], static_cast<uint32_t>((n_s - 1) & 1), p.wait_limit_ns / 8);
+    }
+    return taken;
+}
 
 // ------------------------------------------------------------------------------------------
 // Tiling 1: CTA pairs, rows on M (tcgen05 cta_group::2).  A pair (cluster of 2 CTAs) computes a tile of
@@ -192,9 +379,9 @@ static_assert((2 * kSwapMaxStages + 6 + 2 * kUnitRing + kTmemCols / 32) * 8 + 8 
 // 64 KB per stage); empty[s], acc_full[a] and drain receive multicast commits from the MMA
 // thread in both CTAs; acc_empty[a] lives in the even CTA and counts the 4 epilogue warps
 // of both CTAs (8 arrivals).
-__device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensorMap *tmW,
+__device__ __forceinline__ int head_pair(const CUtensorMap *tmU, const CUtensorMap *tmW,
                                           const HeadParams &p, const HeadSmem &sm, int rows,
-                                          int splits) {
+                                          int splits, int first_unit, uint32_t tmem_base) {
     constexpr int kStageBytes = kPairStageBytesA + kPairStageBytesB;
     uint64_t *full = sm.full, *empty = sm.empty, *acc_full = sm.acc_full,
              *acc_empty = sm.acc_empty, *unit_full = sm.unit_full, *unit_empty = sm.unit_empty;
@@ -204,105 +391,17 @@ __device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensor
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();  // 0 = even CTA (issues the MMAs), 1 = odd
 
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < kPairStages; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
-        }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&acc_full[i], 1);
-            mbar_init(&acc_empty[i], 8);
-        }
-        for (int i = 0; i < kUnitRing; ++i) {
-            mbar_init(&unit_full[i], 1);
-            // even CTA: its MMA issuer and 4 epilogue warps, the odd producer and 4 epilogue warps
-            mbar_init(&unit_empty[i], 10);
-        }
-        mbar_init(sm.drain, 1);
-        *abort_flag = 0;
-        fence_mbar_init();
-        tma_prefetch_desc(tmU);
-        tma_prefetch_desc(tmW);
-    }
-    if (warp == 1) tmem_alloc_pair(sm.tmem_slot, kTmemCols);
-    tc_fence_before_sync();
-    __syncthreads();
-    cluster_sync();  // both CTAs' barriers initialised before any cross-CTA signal
-    tc_fence_after_sync();
-    const uint32_t tmem_base = *sm.tmem_slot;
-
     TileWalk tw;
     tw.init(rows, kPairTileM, p.V, p.d, splits);
     const int num_kb = (p.d + kTileK - 1) / kTileK;
+    int taken = 0;
 
     if (warp == 0) {
         if (lane == 0 && !p.stall) {
             // ------------------------------------------------------- TMA producer (both CTAs)
-            const uint32_t full0 = mapa_shared(smem_u32(&full[0]), 0);
-            const uint32_t unit_full1 = mapa_shared(smem_u32(&unit_full[0]), 1);
-            const uint32_t unit_ring1 = mapa_shared(smem_u32(const_cast<int *>(&unit_ring[0])), 1);
-            const uint32_t unit_empty0 = mapa_shared(smem_u32(&unit_empty[0]), 0);
-            int stage = 0;
-            uint32_t phase = 0;
-            long long fills = 0;
-            bool ok = true;
-            UnitCursor uc;
-            while (ok) {
-                int u;
-                if (rank == 0) {
-                    // claim the next unit and hand it to both CTAs
-                    if (!mbar_wait_bounded_cluster(&unit_empty[uc.slot], uc.phase ^ 1u, abort_flag,
-                                                   p.wait_limit_ns))
-                        break;
-                    const int claimed = atomicAdd(&p.meta[kMetaUnitNext], 1);
-                    u = claimed < tw.units ? claimed : -1;
-                    unit_ring[uc.slot] = u;
-                    st_shared_cluster(unit_ring1 + static_cast<uint32_t>(uc.slot * sizeof(int)), u);
-                    mbar_arrive(&unit_full[uc.slot]);
-                    mbar_arrive_cluster(unit_full1 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
-                } else {
-                    if (!mbar_wait_bounded_cluster(&unit_full[uc.slot], uc.phase, abort_flag,
-                                                   p.wait_limit_ns))
-                        break;
-                    u = unit_ring[uc.slot];
-                    mbar_arrive_cluster(unit_empty0 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
-                }
-                uc.advance();
-                if (u < 0) break;
-                int m, g, n0, n1;
-                tw.unit(u, m, g, n0, n1);
-                for (int n = n0; ok && n < n1; ++n) {
-                    for (int kb = 0; kb < num_kb; ++kb) {
-                        if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, abort_flag, p.wait_limit_ns)) {
-                            ok = false;
-                            break;
-                        }
-                        if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * kStageBytes);
-                        const uint32_t fb = full0 + static_cast<uint32_t>(stage * sizeof(uint64_t));
-                        uint8_t *st = sm.ring + stage * kStageBytes;
-                        tma_load_2d_pair(st, tmU, fb, kb * kTileK,
-                                         m * kPairTileM + static_cast<int>(rank) * kPairHalfRows);
-                        if (p.w_tiled)  // block (2n + rank, kb): 128 contiguous rows of 64
-                            tma_load_2d_pair(st + kPairStageBytesA, tmW, fb, 0,
-                                             ((2 * n + static_cast<int>(rank)) * num_kb + kb) * kPairHalfRows);
-                        else
-                            tma_load_2d_pair(st + kPairStageBytesA, tmW, fb, kb * kTileK,
-                                             n * kTileN + static_cast<int>(rank) * kPairHalfRows);
-                        ++fills;
-                        if (++stage == kPairStages) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
-                    }
-                }
-            }
-            // Drain: a stage's copy has landed once the MMAs that read it have completed, which
-            // the multicast commit on empty[s] reports in this CTA.
-            for (int s = 0; s < kPairStages; ++s) {
-                const long long n_s = fills / kPairStages + (s < fills % kPairStages ? 1 : 0);
-                if (n_s > 0)
-                    mbar_wait_drain(&empty[s], static_cast<uint32_t>((n_s - 1) & 1), p.wait_limit_ns / 8);
-            }
+            const Copies copies{tmW, tmU, kPairStages, kStageBytes, kPairStageBytesA, 0, kPairTileM,
+                                static_cast<int>(rank) * kPairHalfRows};
+            taken = produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
         }
     } else if (warp == 1) {
         if (rank == 0) {
@@ -371,14 +470,14 @@ __device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensor
         const uint32_t acc_empty0 = mapa_shared(smem_u32(&acc_empty[0]), 0);
         const uint32_t unit_empty0 = mapa_shared(smem_u32(&unit_empty[0]), 0);
         uint32_t tile_iter = 0;
-        bool ok = true;
+        bool ok = wait_for_rows(p, sm, rows);
         UnitCursor uc;
         while (ok) {
             if (!mbar_wait_bounded_cluster(&unit_full[uc.slot], uc.phase, abort_flag, p.wait_limit_ns))
                 break;
             const int u = unit_ring[uc.slot];
             __syncwarp();
-            if (lane == 0)
+            if (lane < 2)  // half of the warps work: each arrives twice
                 mbar_arrive_cluster(unit_empty0 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
             uc.advance();
             if (u < 0) break;
@@ -386,7 +485,7 @@ __device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensor
             tw.unit(u, m, g, n0, n1);
             const int r = m * kPairTileM + row_in_tile;
             const bool valid = r < rows;
-            const float scale = valid ? p.inv_rms[r] * kLog2e : 0.f;
+            const float scale = valid ? p.norm.inv_rms[r] * kLog2e : 0.f;
             float run_m = -INFINITY, run_s = 0.f, run_t = 0.f;
             int run_a = 0;
             for (int n = n0; n < n1; ++n, ++tile_iter) {
@@ -410,7 +509,7 @@ __device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensor
                 }
                 tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) mbar_arrive_cluster(acc_empty0 + acc * static_cast<uint32_t>(sizeof(uint64_t)));
+                if (lane < 2) mbar_arrive_cluster(acc_empty0 + acc * static_cast<uint32_t>(sizeof(uint64_t)));
             }
             if (!ok) break;
             if (valid && rpd_check(g < p.max_splits, p.meta + kMetaStatus)) {
@@ -419,17 +518,7 @@ __device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensor
             }
         }
     }
-
-    __syncwarp();
-    tc_fence_before_sync();
-    __syncthreads();
-    cluster_sync();  // no signal may still be in flight to a CTA that is about to exit
-    tc_fence_after_sync();
-    if (*abort_flag && threadIdx.x == 0) atomicExch(&p.meta[kMetaStatus], RPD_ERR_TIMEOUT);
-    if (warp == 1) {
-        __syncwarp();
-        tmem_dealloc_pair(tmem_base, kTmemCols);
-    }
+    return taken;
 }
 
 // Barrier of the rows-on-N epilogue's threads: every thread arrives (release) and waits
@@ -521,10 +610,10 @@ __device__ __forceinline__ SwapSegs swap_segments(int c0, int ng) {
     return g;
 }
 
-__device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps] */,
+__device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] */,
                                           const CUtensorMap *tmW,
                                           const HeadParams &p, const HeadSmem &sm, int rows,
-                                          int splits, int ng) {
+                                          int splits, int ng, int first_unit, uint32_t tmem_base) {
     uint64_t *full = sm.full, *empty = sm.empty, *acc_full = sm.acc_full,
              *acc_empty = sm.acc_empty, *unit_full = sm.unit_full, *unit_empty = sm.unit_empty,
              *chunk_free = sm.chunk_free;
@@ -544,117 +633,31 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
     const bool ring = 2 * nch > kChunks && !single;
     const int stage_b = (ng / 2) * kTileK * 2;
     const int stage_bytes = kSwapStageBytesA + stage_b;
-    // region: operand ring (as many stages as fit), transpose blocks, statistics [4][ng]
-    int stages = (kHeadRegionBytes - kSwapXposeBytes - 4 * ng * 16) / stage_bytes;
+    // region: operand ring (as many stages as fit), transpose blocks, statistics [4][ng], RMS
+    // factors [ng]
+    int stages = (kHeadRegionBytes - kSwapXposeBytes - ng * kSwapRowBytes) / stage_bytes;
     stages = stages < kSwapMaxStages ? stages : kSwapMaxStages;
     float *xpose = reinterpret_cast<float *>(sm.ring + stages * stage_bytes);
     float4 *stats = reinterpret_cast<float4 *>(sm.ring + stages * stage_bytes + kSwapXposeBytes);
+    float *scales = reinterpret_cast<float *>(stats + 4 * ng);
     constexpr int kEpiThreads = 32 * kSwapEpiWarps;
-
-    if (threadIdx.x == 0) {
-        for (int i = 0; i < stages; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
-        }
-        for (int i = 0; i < 2; ++i) {
-            mbar_init(&acc_full[i], 1);
-            mbar_init(&acc_empty[i], 2 * kSwapEpiWarps);
-        }
-        for (int i = 0; i < kUnitRing; ++i) {
-            mbar_init(&unit_full[i], 1);
-            // even CTA: its MMA issuer and epilogue warps; odd CTA: its producer and epilogue warps
-            mbar_init(&unit_empty[i], 2 + 2 * kSwapEpiWarps);
-        }
-        // ring tiles: a chunk is read by one warp per TMEM sub-partition in each CTA
-        for (uint32_t i = 0; i < kChunks; ++i) mbar_init(&chunk_free[i], 8);
-        mbar_init(sm.epi, kEpiThreads);
-        mbar_init(sm.drain, 1);
-        *abort_flag = 0;
-        fence_mbar_init();
-        tma_prefetch_desc(&tmUrows[(ng / 2) / kUBoxRows - 1]);
-        tma_prefetch_desc(tmW);
-    }
-    if (warp == 1) tmem_alloc_pair(sm.tmem_slot, kTmemCols);
-    tc_fence_before_sync();
-    __syncthreads();
-    cluster_sync();
-    tc_fence_after_sync();
-    const uint32_t tmem_base = *sm.tmem_slot;
 
     TileWalk tw;
     tw.init(rows, ng, p.V, p.d, splits);
     const int num_kb = (p.d + kTileK - 1) / kTileK;
+    int taken = 0;
 
     if (warp == 0) {
         if (lane == 0 && !p.stall) {
             // ------------------------------------------------------- TMA producer (both CTAs)
-            const uint32_t full0 = mapa_shared(smem_u32(&full[0]), 0);
-            const uint32_t unit_full1 = mapa_shared(smem_u32(&unit_full[0]), 1);
-            const uint32_t unit_ring1 = mapa_shared(smem_u32(const_cast<int *>(&unit_ring[0])), 1);
-            const uint32_t unit_empty0 = mapa_shared(smem_u32(&unit_empty[0]), 0);
             // this CTA's half of the group's rows, one copy: the map whose box is that many rows
             // high (rows [rank * half, +half) of the group; see the epilogue's row order)
             const int half = ng / 2;
             const CUtensorMap *umap = &tmUrows[half / kUBoxRows - 1];
-            int stage = 0;
-            uint32_t phase = 0;
-            long long fills = 0;
-            bool ok = true;
-            UnitCursor uc;
-            while (ok) {
-                int u;
-                if (rank == 0) {
-                    if (!mbar_wait_bounded_cluster(&unit_empty[uc.slot], uc.phase ^ 1u, abort_flag,
-                                                   p.wait_limit_ns))
-                        break;
-                    const int claimed = atomicAdd(&p.meta[kMetaUnitNext], 1);
-                    u = claimed < tw.units ? claimed : -1;
-                    unit_ring[uc.slot] = u;
-                    st_shared_cluster(unit_ring1 + static_cast<uint32_t>(uc.slot * sizeof(int)), u);
-                    mbar_arrive(&unit_full[uc.slot]);
-                    mbar_arrive_cluster(unit_full1 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
-                } else {
-                    if (!mbar_wait_bounded_cluster(&unit_full[uc.slot], uc.phase, abort_flag,
-                                                   p.wait_limit_ns))
-                        break;
-                    u = unit_ring[uc.slot];
-                    mbar_arrive_cluster(unit_empty0 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
-                }
-                uc.advance();
-                if (u < 0) break;
-                int m, g, v0, v1;
-                tw.unit(u, m, g, v0, v1);
-                const int urow = m * ng + static_cast<int>(rank) * half;
-                const int w_off = static_cast<int>(rank) * kPairHalfRows;
-                for (int n = v0; ok && n < v1; ++n) {
-                    for (int kb = 0; kb < num_kb; ++kb) {
-                        if (!mbar_wait_bounded(&empty[stage], phase ^ 1u, abort_flag, p.wait_limit_ns)) {
-                            ok = false;
-                            break;
-                        }
-                        if (rank == 0) mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
-                        const uint32_t fb = full0 + static_cast<uint32_t>(stage * sizeof(uint64_t));
-                        uint8_t *st = sm.ring + stage * stage_bytes;
-                        const int x = kb * kTileK;
-                        if (p.w_tiled)  // block (2n + rank, kb): 128 contiguous rows of 64
-                            tma_load_2d_pair(st, tmW, fb, 0,
-                                             ((2 * n + static_cast<int>(rank)) * num_kb + kb) * kPairHalfRows);
-                        else
-                            tma_load_2d_pair(st, tmW, fb, x, n * kTileN + w_off);
-                        tma_load_2d_pair(st + kSwapStageBytesA, umap, fb, x, urow);
-                        ++fills;
-                        if (++stage == stages) {
-                            stage = 0;
-                            phase ^= 1u;
-                        }
-                    }
-                }
-            }
-            for (int s = 0; s < stages; ++s) {
-                const long long n_s = fills / stages + (s < fills % stages ? 1 : 0);
-                if (n_s > 0)
-                    mbar_wait_drain(&empty[s], static_cast<uint32_t>((n_s - 1) & 1), p.wait_limit_ns / 8);
-            }
+            tma_prefetch_desc(umap);
+            const Copies copies{tmW, umap, stages, stage_bytes, 0, kSwapStageBytesA, ng,
+                                static_cast<int>(rank) * half};
+            taken = produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
         }
     } else if (warp == 1) {
         if (rank == 0) {
@@ -739,7 +742,7 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
         for (int i = etid; i < 4 * ng; i += kEpiThreads) stats[i] = kEmpty;
         uint32_t epi_phase = 0;
         uint32_t tile_iter = 0;
-        bool ok = epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns);
+        bool ok = epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns) && wait_for_rows(p, sm, rows);
         UnitCursor uc;
         while (ok) {
             if (!mbar_wait_bounded_cluster(&unit_full[uc.slot], uc.phase, abort_flag, p.wait_limit_ns))
@@ -752,6 +755,11 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
             if (u < 0) break;
             int m, g, v0, v1;
             tw.unit(u, m, g, v0, v1);
+            // the group's RMS factors, once per unit (read from global memory for every chunk of
+            // every tile, steps of two 320-row groups were 0.6 % slower)
+            for (int rl = etid; rl < ng; rl += kEpiThreads)
+                scales[rl] = m * ng + rl < rows ? p.norm.inv_rms[m * ng + rl] * kLog2e : 0.f;
+            if (!epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns)) break;
             for (int n = v0; n < v1; ++n, ++tile_iter) {
                 const uint32_t acc = single ? 0u : (tile_iter & 1u);
                 const uint32_t acc_phase = (single ? tile_iter : (tile_iter >> 1)) & 1u;
@@ -794,8 +802,7 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
                     const int nj = col < x1 ? sg.n0 : (col < x2 ? sg.n1 : sg.n2);
                     const int x = col - xj;
                     const int rl = xj / 2 + (x < nj / 2 ? x : ng / 2 + (x - nj / 2));
-                    const int r = m * ng + rl;
-                    const float scale = r < rows ? __ldg(p.inv_rms + r) * kLog2e : 0.f;
+                    const float scale = scales[rl];
                     float4 st = stats[sub * ng + rl];
                     int a = __float_as_int(st.w);
                     if (full_tile)
@@ -830,34 +837,200 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
             if (!epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns)) break;
         }
     }
+    return taken;
+}
+
+// After the contraction: this CTA's `taken` work units are counted, blocks of rows are claimed and
+// merged once every unit of the pass is, and the CTA that completes the merge scores the canvas.
+// Only running CTAs hold units, so the wait ends whatever part of the grid is resident.  It also
+// ends when another CTA has given up (the step's outputs are then meaningless) and, for a CTA
+// that came so late that the canvas was already being scored (`stale`), it is not begun.
+__device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem &sm,
+                                            const PassInfo &pass, int taken, bool stale) {
+    int32_t *meta = p.meta;
+    volatile int *share = reinterpret_cast<volatile int *>(sm.ring + kHeadRegionBytes - 16);
+    const int gs = merge_lanes(pass.splits);
+    const int per_block = kHeadKernelThreads / gs;
+    const int blocks = (pass.rows + per_block - 1) / per_block;
+    if (threadIdx.x == 0) {
+        int block = blocks;
+        if (taken > 0) counter_add_release(&meta[kMetaUnitsDone], taken);
+        if (blocks > 0 && !stale) {
+            block = atomicAdd(&meta[kMetaMergeNext], 1);
+            const int units = pass.mode == kHeadModePair
+                                  ? (pass.rows + kPairTileM - 1) / kPairTileM * pass.splits
+                                  : (pass.rows + pass.swap_rows - 1) / pass.swap_rows * (pass.splits / 2);
+            const uint64_t t0 = globaltimer_ns();
+            while (block < blocks && ld_acquire(&meta[kMetaUnitsDone]) < 2 * units) {
+                if (ld_acquire(&meta[kMetaStatus]) != RPD_OK) break;
+                if (globaltimer_ns() - t0 > 2 * p.wait_limit_ns) {
+                    atomicExch(&meta[kMetaStatus], RPD_ERR_TIMEOUT);
+                    break;
+                }
+            }
+        }
+        share[0] = block;
+        // nothing to merge: the first CTA scores
+        share[1] = blocks == 0 && blockIdx.x == 0 && !stale;
+    }
+    __syncthreads();
+    const int num_words = p.from_mask ? (p.compact.B * p.compact.N + 31) >> 5 : 0;
+    for (int block = share[0]; block < blocks; block = share[0]) {
+        merge_block(p.merge, pass, p.norm.sel_list, block, gs, meta + kMetaStatus,
+                    [&](int q) { return sm.map.position(q, num_words); });
+        __threadfence();  // this CTA's merged rows are visible before they are counted
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            share[1] = atomicAdd(&meta[kMetaMergeDone], 1) == blocks - 1;
+            share[0] = atomicAdd(&meta[kMetaMergeNext], 1);
+            __threadfence();
+        }
+        __syncthreads();
+    }
+    if (!p.score_canvas || !share[1]) return;
+    int status = RPD_OK, rows_total = pass.rows;
+    if (threadIdx.x == 0) {
+        atomicExch(&meta[kMetaClosed], 1);
+        __threadfence();  // before any mask byte changes
+        status = ld_acquire(&meta[kMetaStatus]);
+        if (!p.from_mask) rows_total = meta[kMetaRowsTotal];
+    }
+    score_canvas(p.score, 0, p.score.tau, p.score.budget, pass, status, rows_total,
+                 carve_score(sm.ring, p.score.N), [&](int i, bool masked) {
+                     if (p.from_mask) return sm.map.scored(i) ? sm.map.rank(i) : -1;
+                     const int q = p.score.q_of_pos[i];
+                     return masked ? q : -1;
+                 });
+}
+
+// The head kernel: one launch per projection pass, clusters of two CTAs, one CTA per SM.  It
+// compacts the mask (or reads the pass from the meta words), gathers and normalises the pass's
+// rows, contracts them with the head, merges the splits' statistics and scores a single canvas.
+__global__ void __launch_bounds__(kHeadKernelThreads, 1)
+    k_head(const __grid_constant__ HeadMaps maps, const __grid_constant__ HeadParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    const HeadSmem sm = carve_smem(smem_raw);
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_ctarank();
+    pdl_trigger();  // successors may launch now; they wait for this grid before reading
+    for (int i = threadIdx.x * 64; i < p.d; i += blockDim.x * 64)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"(p.norm.gain + i));
+    if (threadIdx.x == 0) {
+        init_barriers(sm);
+        tma_prefetch_desc(&maps.w128);
+        tma_prefetch_desc(&maps.u);
+    }
+    if (warp == 1) tmem_alloc_pair(sm.tmem_slot, kTmemCols);
+    tc_fence_before_sync();
+    __syncthreads();
+    cluster_sync();  // both CTAs' barriers initialised before any cross-CTA signal
+    tc_fence_after_sync();
+    const uint32_t tmem_base = *sm.tmem_slot;
+    pdl_wait();  // mask, hidden states and meta words come from preceding work of the stream
+
+    // The first claims need nothing of the pass, and return while it is worked out.
+    int first_unit = -1, first_row = 0;
+    if (threadIdx.x == 0 && rank == 0) first_unit = atomicAdd(&p.meta[kMetaUnitNext], 1);
+    if (warp >= 2 && lane == 0) first_row = atomicAdd(&p.meta[kMetaRowNext], 1);
+
+    PassInfo pass;
+    int num_words = 0;
+    bool stale = false;
+    if (p.from_mask) {
+        const int masked = compact_mask(p.compact, sm.map, reinterpret_cast<int *>(sm.ring));
+        num_words = (p.compact.B * p.compact.N + 31) >> 5;
+        if (threadIdx.x == 0 && p.score_canvas) {  // read after the mask
+            __threadfence();
+            stale = ld_acquire(&p.meta[kMetaClosed]) != 0;
+        }
+        int lazy = 0;
+        if (p.compact.lazy) {  // which rows there are may depend on the plan
+            if (warp == 0) {
+                lazy = choose_lazy(p.compact, masked);
+                if (lane == 0) sm.map.pass->lazy = lazy;
+            }
+            __syncthreads();
+            lazy = sm.map.pass->lazy;
+        }
+        pass.masked = masked;
+        pass.lazy = lazy;
+        pass.sel = masked;
+        pass.layer0 = lazy ? p.compact.K - 1 : 0;
+        pass.rows = lazy ? masked : p.compact.K * masked;
+        if (warp == 0) {
+            const HeadPlan hp = lookup_plan(pass.rows, p.compact.plan, p.compact.plan_rows, p.compact.plan_in);
+            pass.mode = hp.mode;
+            pass.splits = hp.splits;
+            pass.swap_rows = hp.swap_rows;
+            if (lane == 0) *sm.map.pass = pass;
+        }
+    } else {
+        pass.rows = p.meta[kMetaRows];
+        pass.masked = p.meta[kMetaMasked];
+        pass.lazy = p.meta[kMetaLazy];
+        pass.sel = p.meta[kMetaSel];
+        pass.layer0 = p.meta[kMetaLayer0];
+        pass.mode = p.meta[kMetaHeadMode];
+        pass.splits = p.meta[kMetaSplits];
+        pass.swap_rows = p.meta[kMetaSwapRows];
+    }
+
+    if (warp >= 2) {
+        first_row = __shfl_sync(0xffffffffu, first_row, 0);
+        gather_rows(p.norm, sm.map, num_words, pass.rows, pass.sel, pass.layer0, first_row,
+                    rows_per_claim(pass.rows, gridDim.x * kSwapEpiWarps), p.meta, lane);
+    }
+    if (p.from_mask) {  // the plan, from warp 0, which does not wait for the others
+        if (warp == 0) {
+            __syncwarp();
+            asm volatile("bar.arrive 1, %0;" ::"n"(kHeadKernelThreads) : "memory");
+        } else {
+            asm volatile("bar.sync 1, %0;" ::"n"(kHeadKernelThreads) : "memory");
+            pass = *sm.map.pass;
+            // for the kernels after this one, by the warp that gathered row 0 (or, without rows,
+            // one of the first CTA)
+            if (!p.score_canvas && warp >= 2 && (pass.rows > 0 ? first_row == 0 : blockIdx.x == 0 && warp == 2))
+                publish_pass(p.compact, sm.map, lane);
+        }
+    }
+
+    int taken = 0;
+    if (pass.rows > 0) {
+        if (pass.mode == kHeadModePair)
+            taken = head_pair(&maps.u, &maps.w128, p, sm, pass.rows, pass.splits, first_unit, tmem_base);
+        else if (pass.mode == kHeadModeRowsN)
+            taken = head_swap(maps.u_rows, &maps.w128, p, sm, pass.rows, pass.splits / 2,
+                              pass.swap_rows, first_unit, tmem_base);
+    }
 
     __syncwarp();
     tc_fence_before_sync();
     __syncthreads();
-    cluster_sync();
+    cluster_sync();  // no signal may still be in flight to a CTA that is about to exit
     tc_fence_after_sync();
-    if (*abort_flag && threadIdx.x == 0) atomicExch(&p.meta[kMetaStatus], RPD_ERR_TIMEOUT);
+    if (*sm.abort_flag && threadIdx.x == 0) atomicExch(&p.meta[kMetaStatus], RPD_ERR_TIMEOUT);
     if (warp == 1) {
         __syncwarp();
         tmem_dealloc_pair(tmem_base, kTmemCols);
     }
-}
-
-// The head kernel: one launch per projection pass, clusters of two CTAs, one CTA per SM.
-__global__ void __launch_bounds__(kHeadKernelThreads, 1)
-    k_head(const __grid_constant__ HeadMaps maps, HeadParams p) {
-    pdl_trigger();  // successors may launch now; they wait for this grid before reading
-    pdl_wait();     // row count, tiling, u and inv_rms come from the preceding kernels
-    const int rows = p.meta[kMetaRows];
-    if (rows == 0) return;  // uniform over the grid: no cluster-wide barrier is left waiting
-    const int mode = p.meta[kMetaHeadMode];
-    const int splits = p.meta[kMetaSplits];
-    extern __shared__ uint8_t smem_raw[];
-    const HeadSmem sm = carve_smem(smem_raw);
-    if (mode == kHeadModePair)
-        head_pair(&maps.u, &maps.w128, p, sm, rows, splits);
-    else if (mode == kHeadModeRowsN)
-        head_swap(maps.u_rows, &maps.w128, p, sm, rows, splits / 2, p.meta[kMetaSwapRows]);
+    finish_pass(p, sm, pass, taken, stale);
+    // The last CTA of the grid leaves the counters at zero for the next pass.
+    if (threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(&p.meta[kMetaExit], 1) == static_cast<int>(gridDim.x) - 1) {
+            __threadfence();
+            p.meta[kMetaUnitNext] = 0;
+            p.meta[kMetaRowNext] = 0;
+            p.meta[kMetaMergeNext] = 0;
+            p.meta[kMetaMergeDone] = 0;
+            p.meta[kMetaRowsDone] = 0;
+            p.meta[kMetaUnitsDone] = 0;
+            p.meta[kMetaClosed] = 0;
+            p.meta[kMetaExit] = 0;
+            if (p.last_pass) p.meta[kMetaStepStatus] = atomicExch(&p.meta[kMetaStatus], RPD_OK);
+        }
+    }
 }
 
 // The tiled copy of the head: thread i writes 16-byte vector i of Wt, which is vector k8 of

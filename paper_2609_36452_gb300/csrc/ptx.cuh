@@ -135,6 +135,39 @@ __device__ __forceinline__ bool mbar_wait_drain(uint64_t *bar, uint32_t parity, 
     return true;
 }
 
+// ------------------------------------------------------- counters in global memory
+// Work of one grid that its CTAs hand to one another through global memory: a writer finishes
+// its stores with counter_add_release, a reader polls with counter_wait until the count is
+// reached.  proxy_fence orders these generic accesses with TMA copies of the same data.
+
+__device__ __forceinline__ int ld_acquire(const int *p) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void counter_add_release(int *p, int n) {
+    asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(n) : "memory");
+}
+
+__device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;" ::: "memory"); }
+
+// Bounded and abort aware like the mbarrier waits; `sleep_ns` between polls.
+__device__ __forceinline__ bool counter_wait(const int *p, int target, volatile int *abort,
+                                             uint64_t limit_ns, unsigned sleep_ns = 0) {
+    if (ld_acquire(p) >= target) return true;
+    const uint64_t t0 = globaltimer_ns();
+    while (true) {
+        if (sleep_ns) __nanosleep(sleep_ns);
+        if (ld_acquire(p) >= target) return true;
+        if (*abort) return false;
+        if (globaltimer_ns() - t0 > limit_ns) {
+            *abort = 1;
+            return false;
+        }
+    }
+}
+
 // ------------------------------------------------------------------------------ clusters
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -179,6 +212,24 @@ __device__ __forceinline__ void tma_load_2d_pair(void *smem_dst, const CUtensorM
         " [%0], [%1, {%2, %3}], [%4];" ::"r"(smem_u32(smem_dst)),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster_addr)
         : "memory");
+}
+
+// The same load with an L2 eviction policy (l2_evict_first).
+__device__ __forceinline__ void tma_load_2d_pair_hint(void *smem_dst, const CUtensorMap *map,
+                                                      uint32_t bar_cluster_addr, int32_t x, int32_t y,
+                                                      uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes"
+        ".L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(smem_u32(smem_dst)),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar_cluster_addr), "l"(policy)
+        : "memory");
+}
+
+// Policy for data that is streamed through L2: its lines go before any others.
+__device__ __forceinline__ uint64_t l2_evict_first() {
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    return policy;
 }
 
 __device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *map) {

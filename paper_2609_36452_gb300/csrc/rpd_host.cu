@@ -1,9 +1,10 @@
 // rpd_host.cu - the C ABI of include/rpd.h: context, argument checks, scratch, TMA
 // descriptors and the launch sequence of one commit step.
 //
-// Step = k_compact -> k_gather_norm -> k_head_stats -> k_merge -> k_score_commit, all on
-// the context's stream, sized from device-resident counts (nothing is read back
-// mid-step).  Scratch is owned by the context and sized for the largest B*N seen.
+// Step = k_head (compaction, gather, contraction, merge and, for a single canvas, score and
+// commit), sized from device-resident counts (nothing is read back mid-step).  Several canvases
+// are scored by k_score_commit; batches of more than kFusedMaxPositions positions are compacted
+// by k_compact first; lazy projection runs k_band and a second k_head.  Scratch is owned by the context and sized for the largest B*N seen.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -319,13 +320,13 @@ int check_call(const rpd_ctx *c, float tau, float budget) {
     return RPD_OK;
 }
 
+// Scoring of a canvas, with the thresholds of the first (or only) one.
 ScoreParams score_params(const rpd_ctx *c, uint8_t *mask, int B, int N, const float *tau,
                          const float *budget, uint8_t *out_commit, int32_t *out_token,
-                         rpd_stats *out_stats, bool lazy) {
+                         rpd_stats *out_stats) {
     ScoreParams sp{};
     sp.mask = mask;
     sp.q_of_pos = c->q_of_pos;
-    sp.canvas_off = c->canvas_off;
     sp.meta = c->meta;
     sp.row_arg = c->row_arg;
     sp.row_pmax = c->row_pmax;
@@ -343,12 +344,49 @@ ScoreParams score_params(const rpd_ctx *c, uint8_t *mask, int B, int N, const fl
     sp.k_max = c->rule.k_max;
     sp.window = c->rule.window;
     sp.block = c->rule.block;
-    sp.lazy = lazy ? 1 : 0;
-    for (int b = 0; b < B; ++b) {
-        sp.tau[b] = tau[b];
-        sp.budget[b] = budget[b];
-    }
+    sp.tau = tau[0];
+    sp.budget = budget[0];
     return sp;
+}
+
+// The same for B canvases, each with its own thresholds.
+BatchScoreParams batch_score_params(const ScoreParams &sp, const float *tau, const float *budget) {
+    BatchScoreParams bp{};
+    bp.canvas = sp;
+    for (int b = 0; b < sp.B; ++b) {
+        bp.tau[b] = tau[b];
+        bp.budget[b] = budget[b];
+    }
+    return bp;
+}
+
+// The compaction of a step's mask; `lazy` as in CompactParams.
+CompactParams compact_params(const rpd_ctx *c, const uint8_t *mask, int B, int N, int lazy) {
+    return CompactParams{mask, c->q_of_pos, c->pos_of_q, c->canvas_off, c->meta, B, N, c->K,
+                         plan_inputs(c), c->plan, c->plan_rows, c->rule.block, lazy};
+}
+
+// One launch of the head kernel: the pass over the mask's positions (from_mask) or over those the
+// meta words and sel_list describe.
+HeadParams head_params(const rpd_ctx *c, const CompactParams &cp, const void *hidden,
+                       const int32_t *sel_list, bool from_mask, bool last_pass, const MergeArgs &mg) {
+    HeadParams hp{};
+    hp.compact = cp;
+    hp.norm = NormParams{static_cast<const __nv_bfloat16 *>(hidden),
+                         static_cast<const __nv_bfloat16 *>(c->g), c->pos_of_q, sel_list, c->meta,
+                         c->u, c->inv_rms, cp.B * cp.N, c->d, c->eps};
+    hp.merge = mg;
+    hp.partials = c->partials;
+    hp.meta = c->meta;
+    hp.from_mask = from_mask ? 1 : 0;
+    hp.last_pass = last_pass ? 1 : 0;
+    hp.V = c->V;
+    hp.d = c->d;
+    hp.max_splits = c->max_splits;
+    hp.wait_limit_ns = c->wait_limit_ns;
+    hp.stall = c->stall_next ? 1 : 0;
+    hp.w_tiled = c->W_tiled != nullptr ? 1 : 0;
+    return hp;
 }
 
 // Arguments every single-canvas step checks before it touches the GPU.
@@ -391,56 +429,35 @@ int run_step(rpd_ctx *c, const void *hidden, uint8_t *mask, int B, int N, const 
     if (rc) return rc;
 
     const int bn = B * N;
-    const int num_n = (c->V + kTileN - 1) / kTileN;
-    const HeadPlanInputs plan_in = plan_inputs(c);
     // Lazy projection (forced, or chosen on the device per step): a second pass over the band.
     // It is not launched when even the largest possible row count keeps a single pass cheaper.
     const bool lazy = c->projection == RPD_PROJECT_LAZY ||
                       (c->projection == RPD_PROJECT_AUTO && c->K > 1 &&
                        static_cast<long long>(c->K) * bn > 2LL * kTileM);
-    cudaError_t e;
-    {
+    cudaError_t e = cudaSuccess;
+    const CompactParams cp = compact_params(
+        c, mask, B, N, c->projection == RPD_PROJECT_LAZY ? 1 : (lazy ? 2 : 0));
+    const bool from_mask = bn <= kFusedMaxPositions;
+    if (!from_mask) {
         KernelTimer t(c, 0);
-        CompactParams cp{mask, c->q_of_pos, c->pos_of_q, c->canvas_off, c->meta, B, N, c->K,
-                         plan_in, c->plan, c->plan_rows, c->rule.block,
-                         c->projection == RPD_PROJECT_LAZY ? 1 : (lazy ? 2 : 0)};
         e = launch_compact(cp, c->stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "compaction launch");
 
-    // Scoring, scan and commit of every canvas (k_score_commit, or the last merge's grid).
-    const ScoreParams sp = score_params(c, mask, B, N, tau, budget, out_commit, out_token,
-                                        out_stats, lazy);
-    const bool fuse_score = B == 1 && N <= kFuseScoreMaxN;
+    // Scoring, scan and commit: by the step's last head kernel for a single canvas (one launch
+    // fewer), by k_score_commit for several.
+    const ScoreParams sp = score_params(c, mask, B, N, tau, budget, out_commit, out_token, out_stats);
+    const bool fuse_score = B == 1;
 
-    // One projection pass: gather + RMSNorm prologue, head statistics, merge.  Rows, layers
-    // and positions of the pass come from the device-side meta words.
+    // One projection pass: the head kernel (gather + RMSNorm prologue, head statistics, merge).
     const MergeArgs mg{c->partials, c->max_splits, c->row_arg, c->row_pmax, c->row_H};
     auto pass = [&](const int32_t *sel_list, bool last) -> cudaError_t {
-        cudaError_t err;
-        {
-            KernelTimer t(c, 0);
-            NormParams np{static_cast<const __nv_bfloat16 *>(hidden),
-                          static_cast<const __nv_bfloat16 *>(c->g), c->pos_of_q, sel_list, c->meta,
-                          c->u, c->inv_rms, bn, c->d, c->eps};
-            // one warp per row: no more CTAs than the largest possible row count needs
-            const long long max_rows = static_cast<long long>(c->K) * bn;
-            const int grid = static_cast<int>(std::min<long long>(c->num_sms * 8, (max_rows + 7) / 8));
-            err = launch_gather_norm(np, grid, c->stream);
-        }
-        if (err != cudaSuccess) return err;
-        {
-            KernelTimer t(c, 1);
-            HeadParams hp{c->inv_rms, c->partials, c->meta, c->V, c->d, c->max_splits,
-                          c->wait_limit_ns, c->stall_next ? 1 : 0, c->W_tiled != nullptr ? 1 : 0};
-            // One launch: the kernel reads the tiling chosen on the device for this pass.
-            err = launch_head(c->maps, hp, c->head_grid, c->stream);
-        }
-        if (err != cudaSuccess) return err;
-        KernelTimer t(c, 2);
-        if (last && fuse_score)
-            return launch_merge_score(mg, c->meta, sel_list, c->num_sms * 4, sp, c->stream);
-        return launch_merge(mg, c->meta, sel_list, c->num_sms * 4, c->stream);
+        KernelTimer t(c, 1);
+        // The kernel reads the tiling chosen on the device for this pass.
+        HeadParams hp = head_params(c, cp, hidden, sel_list, from_mask && !sel_list, last, mg);
+        hp.score = sp;
+        hp.score_canvas = last && fuse_score ? 1 : 0;
+        return launch_head(c->maps, hp, c->head_grid, c->stream);
     };
     e = pass(nullptr, !lazy);
     if (e == cudaSuccess && lazy) {
@@ -457,7 +474,7 @@ int run_step(rpd_ctx *c, const void *hidden, uint8_t *mask, int B, int N, const 
             bp.N = N;
             bp.K = c->K;
             bp.theta_c = c->rule.theta_c;
-            bp.plan_in = plan_in;
+            bp.plan_in = cp.plan_in;
             bp.plan = c->plan;
             bp.plan_rows = c->plan_rows;
             for (int b = 0; b < B; ++b) bp.tau[b] = tau[b];
@@ -467,12 +484,10 @@ int run_step(rpd_ctx *c, const void *hidden, uint8_t *mask, int B, int N, const 
     }
     c->stall_next = false;
     if (e != cudaSuccess) return cuda_fail(e, "projection launch");
-    // The step's last merge also scores the canvas when there is a single canvas of at most
-    // kFuseScoreMaxN positions (one launch fewer); otherwise score/commit is its own launch.
     if (fuse_score) return RPD_OK;
     {
         KernelTimer t(c, 3);
-        e = launch_score_commit(sp, c->stream);
+        e = launch_score_commit(batch_score_params(sp, tau, budget), c->stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "score/commit launch");
     return RPD_OK;
@@ -936,29 +951,12 @@ int rpd_step_shard_partials(rpd_ctx *c, const void *hidden, const uint8_t *mask,
         return fail(RPD_ERR_INVALID_ARGUMENT, "out_partials must be 16-byte aligned device memory");
     rc = ensure_scratch(c, 1, N);
     if (rc) return rc;
-    const HeadPlanInputs plan_in = plan_inputs(c);
-    CompactParams cp{mask, c->q_of_pos, c->pos_of_q, c->canvas_off, c->meta, 1, N, c->K,
-                     plan_in, c->plan, c->plan_rows, c->rule.block, 0};
-    cudaError_t e = launch_compact(cp, c->stream);
-    if (e == cudaSuccess) {
-        NormParams np{static_cast<const __nv_bfloat16 *>(hidden),
-                      static_cast<const __nv_bfloat16 *>(c->g), c->pos_of_q, nullptr, c->meta,
-                      c->u, c->inv_rms, N, c->d, c->eps};
-        const long long max_rows = static_cast<long long>(c->K) * N;
-        e = launch_gather_norm(np, static_cast<int>(std::min<long long>(c->num_sms * 8, (max_rows + 7) / 8)),
-                               c->stream);
-    }
-    if (e == cudaSuccess) {
-        HeadParams hp{c->inv_rms, c->partials, c->meta, c->V, c->d, c->max_splits, c->wait_limit_ns,
-                      c->stall_next ? 1 : 0, c->W_tiled != nullptr ? 1 : 0};
-        e = launch_head(c->maps, hp, c->head_grid, c->stream);
-        c->stall_next = false;
-    }
-    if (e == cudaSuccess) {
-        MergeArgs mg{c->partials, c->max_splits, c->row_arg, c->row_pmax, c->row_H,
-                     reinterpret_cast<float4 *>(out_partials), c->pos_of_q, N, c->v_offset};
-        e = launch_merge(mg, c->meta, nullptr, c->num_sms * 4, c->stream);
-    }
+    const CompactParams cp = compact_params(c, mask, 1, N, 0);
+    const MergeArgs mg{c->partials, c->max_splits, c->row_arg, c->row_pmax, c->row_H,
+                       reinterpret_cast<float4 *>(out_partials), N, c->v_offset};
+    const HeadParams hp = head_params(c, cp, hidden, nullptr, true, true, mg);  // N <= kFusedMaxPositions
+    const cudaError_t e = launch_head(c->maps, hp, c->head_grid, c->stream);
+    c->stall_next = false;
     if (e != cudaSuccess) return cuda_fail(e, "sharded projection launch");
     return RPD_OK;
 }
@@ -980,20 +978,16 @@ int rpd_step_shard_finish(rpd_ctx *c, const float *gathered, int P, uint8_t *mas
     if (!aligned16(gathered)) return fail(RPD_ERR_INVALID_ARGUMENT, "gathered must be 16-byte aligned");
     rc = ensure_scratch(c, 1, N);
     if (rc) return rc;
-    const HeadPlanInputs plan_in = plan_inputs(c);
-    CompactParams cp{mask, c->q_of_pos, c->pos_of_q, c->canvas_off, c->meta, 1, N, c->K,
-                     plan_in, c->plan, c->plan_rows, c->rule.block, 0,
-                     1 /* keep the partials call's status (a timed-out wait) */};
-    cudaError_t e = launch_compact(cp, c->stream);
+    // the status that the partials call published stays (a timed-out wait)
+    cudaError_t e = launch_compact(compact_params(c, mask, 1, N, 0), c->stream);
     if (e == cudaSuccess) {
         ShardMergeParams mp{reinterpret_cast<const float4 *>(gathered), P, c->K, N, c->pos_of_q,
                             c->meta, c->row_arg, c->row_pmax, c->row_H};
         e = launch_merge_shards(mp, c->num_sms * 2, c->stream);
     }
     if (e == cudaSuccess) {
-        const ScoreParams sp = score_params(c, mask, 1, N, &tau, &budget, out_commit, out_token,
-                                            out_stats, false);
-        e = launch_score_commit(sp, c->stream);
+        const ScoreParams sp = score_params(c, mask, 1, N, &tau, &budget, out_commit, out_token, out_stats);
+        e = launch_score_commit(batch_score_params(sp, &tau, &budget), c->stream);
     }
     if (e != cudaSuccess) return cuda_fail(e, "shard merge / score launch");
     return RPD_OK;

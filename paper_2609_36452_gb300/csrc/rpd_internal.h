@@ -40,30 +40,35 @@ constexpr int kSwapStageBytesA = kPairHalfRows * kTileK * 2;
 constexpr int kSwapEpiWarps = 8;   // two per TMEM sub-partition, alternating its chunks
 constexpr int kSwapXposeStride = 33;                             // floats per padded row
 constexpr int kSwapXposeBytes = kSwapEpiWarps * 32 * kSwapXposeStride * 4;  // 32 x 32 fp32 per warp
-// rows on N: running statistics [sub-partition][row of the group], 4 * ng float4
+// rows on N, per row of the group: running statistics of the four sub-partitions, RMS factor
+constexpr int kSwapRowBytes = 4 * 16 + 4;
 constexpr int kUBoxRows = 16;  // granularity of a half group's rows (the TMA box heights)
 // Roles: warp 0 TMA, warp 1 MMA + TMEM owner, warps 2-9 epilogue (pair tiles use warps 2-5).
-// At 128 registers a thread the CTA holds 40 K of an SM's 64 K registers, which leaves room for
-// a CTA of the next kernel in the stream (launched early, waiting on this grid).
 constexpr int kHeadKernelThreads = 64 + 32 * kSwapEpiWarps;
-constexpr int kHeadBarrierBytes = 512;
+constexpr int kHeadBarrierBytes = 448;
+// Canvas positions (B * N) whose masks the head kernel compacts itself, as a bitmap in its shared
+// memory: any single canvas, and batches of up to this many positions together.
+constexpr int kFusedMaxPositions = 8192;
+constexpr int kMaskWords = kFusedMaxPositions / 32;
+constexpr int kHeadMaskBytes = kMaskWords * 4 + (kMaskWords + 8) * 2 + 32;  // bitmap, prefixes, plan
 // The pair tiles' operand ring, or the rows-on-N ring, transpose blocks and statistics (the
 // ring takes what the other two leave): the 7-stage pair ring, 224 KB.
 constexpr int kHeadRegionBytes = 224 * 1024;
 static_assert(kPairStages <= kSwapMaxStages, "the stage barriers are shared by both tilings");
 static_assert(kPairStages * (kPairStageBytesA + kPairStageBytesB) <= kHeadRegionBytes,
               "the pair tiles' operand ring fits the region");
-static_assert(kHeadRegionBytes - kSwapXposeBytes - 4 * kSwapMaxRows * 16 >=
+static_assert(kHeadRegionBytes - kSwapXposeBytes - kSwapMaxRows * kSwapRowBytes >=
                   3 * (kSwapStageBytesA + (kSwapMaxRows / 2) * kTileK * 2),
               "a 512-row group still gets three stages");
-// 1024-byte alignment slack + that region + barriers
-constexpr int kHeadKernelSmemBytes = 1024 + kHeadRegionBytes + kHeadBarrierBytes;
+// 1024-byte alignment slack + that region + barriers + the compaction's bitmap
+constexpr int kHeadKernelSmemBytes = 1024 + kHeadRegionBytes + kHeadBarrierBytes + kHeadMaskBytes;
 static_assert(kHeadKernelSmemBytes <= 232448, "dynamic shared memory per CTA");
 // Values of meta[kMetaHeadMode].
 constexpr int kHeadModePair = 2;
 constexpr int kHeadModeRowsN = 3;
 constexpr int kMaxBatch = 128;
 constexpr int kMaxCanvas = 8192;
+static_assert(kMaxCanvas <= kFusedMaxPositions, "a single canvas never needs k_compact");
 constexpr int kScoreThreads = 1024;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 constexpr long long kBandBytes = 32ll << 20;       // u tiles a band of head work units re-reads
@@ -79,10 +84,24 @@ enum MetaIndex : int {
     kMetaLayer0 = 6,   // first window layer of the current pass (rows are layer-major)
     kMetaRowsTotal = 7,// rows projected by all passes of this step
     kMetaLazy = 8,     // 1 when this step projects lazily (two passes)
-    kMetaUnitNext = 9, // next head work unit to claim (zeroed before each projection pass)
-    kMetaMergeDone = 10, // CTAs that finished the fused merge-and-score (zeroed per step)
+    kMetaUnitNext = 9, // next head work unit to claim
+    kMetaMergeDone = 10, // merged blocks of rows
     kMetaSwapRows = 11,  // rows per row group of the "rows on N" tiling (mode 3)
-    kMetaWords = 16
+    kMetaRowNext = 12,   // next rows of the pass to gather (claimed by the head kernel's warps)
+    kMetaMergeNext = 13, // next block of rows to merge (claimed by the head kernel's CTAs)
+    kMetaExit = 14,      // CTAs of the head kernel that are done; the last one zeroes the counters
+    kMetaStepStatus = 15,// the step's status, published when its last head kernel ends
+    kMetaClosed = 16,    // the canvas is being scored: the mask no longer describes the pass
+    // counts that the head kernel's CTAs wait for, on a line of their own
+    kMetaRowsDone = 32,  // gathered rows of the pass
+    kMetaUnitsDone = 33, // head work units whose partials are written, counted by both CTAs of a pair
+    kMetaWords = 64
+};
+
+// A projection pass as the head kernel sees it (from its own compaction, or from the meta words).
+struct PassInfo {
+    int rows, sel, layer0, masked, lazy;
+    int mode, splits, swap_rows;
 };
 
 // Tiling plan of a projection pass (head_plan.h): which tiling the head kernel runs, with how
@@ -115,7 +134,6 @@ struct CompactParams {
     int plan_rows;
     int block;            // 0: every masked position; > 0: only each canvas's active block
     int lazy;             // 0: all window layers; 1: lazy; 2: lazy when it is estimated cheaper
-    int keep_status;      // 1: leave the status word as the previous call of the step left it
 };
 
 // Band fraction assumed when the device weighs lazy against full projection before the
@@ -137,7 +155,6 @@ struct MergeArgs {
     // (max, sum, tsum, argmax + v_offset) go to shard_out[layer * shard_stride + position]
     // instead of the derived outputs above.
     float4 *shard_out;
-    const int32_t *pos_of_q;
     int shard_stride;
     int v_offset;
 };
@@ -205,16 +222,6 @@ struct NormParams {
     float eps;
 };
 
-struct HeadParams {
-    const float *inv_rms;  // [rows]
-    float4 *partials;      // [rows][max_splits]: (max, sum, tsum, argmax bits), log2 units
-    int32_t *meta;
-    int V, d, max_splits;
-    uint64_t wait_limit_ns;  // bound on every mbarrier wait
-    int stall;               // diagnostics: issue no loads (the waits run out)
-    int w_tiled;             // W is the context's tiled copy (rpd_set_head_layout), else row-major
-};
-
 // Time to stream the head once, in units of one 128 x 256 tile's MMA time on one SM.
 inline float head_stream_in_tiles(int V, int d, int num_sms) {
     (void)num_sms;
@@ -226,7 +233,6 @@ inline float head_stream_in_tiles(int V, int d, int num_sms) {
 struct ScoreParams {
     uint8_t *mask;              // [B][N] in/out
     const int32_t *q_of_pos;    // [B*N]
-    const int32_t *canvas_off;  // [B+1]
     const int32_t *meta;
     const int32_t *row_arg;
     const float *row_pmax;
@@ -239,9 +245,31 @@ struct ScoreParams {
     float theta_c, theta_s, w;
     int k_max, window;
     int block;                  // 0: full RPD; > 0: RPD-block (no budget, in-block fallback)
-    int lazy;                   // 1: earlier window layers exist only for band positions
+    float tau, budget;          // of a single canvas
+};
+
+// Several canvases, each with thresholds of its own.
+struct BatchScoreParams {
+    ScoreParams canvas;
     float tau[kMaxBatch];
     float budget[kMaxBatch];
+};
+
+struct HeadParams {
+    CompactParams compact; // the mask and what its compaction writes
+    NormParams norm;       // the rows gathered before the contraction
+    float4 *partials;      // [rows][max_splits]: (max, sum, tsum, argmax bits), log2 units
+    int32_t *meta;
+    int from_mask;         // the kernel compacts the mask itself (B * N <= kFusedMaxPositions);
+                           // otherwise the pass is described by the meta words
+    int last_pass;         // the step's last projection pass: publish its status
+    int score_canvas;      // score the (single) canvas after the merge
+    MergeArgs merge;
+    ScoreParams score;
+    int V, d, max_splits;
+    uint64_t wait_limit_ns;  // bound on every mbarrier wait
+    int stall;               // diagnostics: issue no loads (the waits run out)
+    int w_tiled;             // W is the context's tiled copy (rpd_set_head_layout), else row-major
 };
 
 // Launch with programmatic stream serialisation, so that the kernel's prologue overlaps the
@@ -324,7 +352,6 @@ inline bool pointer_usable(const void *p, int device, bool host_mapped_ok) {
 }
 
 cudaError_t launch_compact(const CompactParams &p, cudaStream_t s);
-cudaError_t launch_gather_norm(const NormParams &p, int grid, cudaStream_t s);
 // Tensor maps of the head kernel's operands (128-byte swizzling, K boxes of 64): u in boxes of
 // 128 rows (pair tiles) and, for the rows-on-N tiles, in boxes of 16, 32, ..., 128 rows (one
 // per half-group height, so that a stage copies each MMA's share of u with one instruction:
@@ -344,18 +371,10 @@ cudaError_t launch_head(const HeadMaps &maps, const HeadParams &p, int grid, cud
 cudaError_t launch_tile_head(const void *W, void *Wt, int V, int d, cudaStream_t s);
 // Largest number of clusters of the head kernel that can be resident at once.
 int head_max_clusters();
-cudaError_t launch_merge(const MergeArgs &mg, const int32_t *meta, const int32_t *sel_list,
-                         int grid, cudaStream_t s);
 cudaError_t launch_band(const BandParams &p, cudaStream_t s);
-cudaError_t launch_score_commit(const ScoreParams &p, cudaStream_t s);
+cudaError_t launch_score_commit(const BatchScoreParams &p, cudaStream_t s);
 // Stop test of the decoding loop: counts the step and sets the loop's condition (one thread).
 cudaError_t launch_loop_test(cudaGraphConditionalHandle handle, const rpd_stats *stats, int B, int N,
                              float stop_frac, int max_steps, int32_t *steps, cudaStream_t s);
 cudaError_t launch_merge_shards(const ShardMergeParams &p, int grid, cudaStream_t s);
-// The step's last merge fused with the scoring of its canvas (one canvas of at most
-// kFuseScoreMaxN positions); the separate score launch is then skipped.
-constexpr int kFuseScoreMaxN = 2048;
-cudaError_t launch_merge_score(const MergeArgs &mg, int32_t *meta, const int32_t *sel_list,
-                               int grid, const ScoreParams &p, cudaStream_t s);
-
 }  // namespace rpd

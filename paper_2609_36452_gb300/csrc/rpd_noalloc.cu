@@ -46,7 +46,7 @@ constexpr int kNaMaxRows = 1024;
 constexpr int kNaMaxD = 4096;
 constexpr int kNaMaxN = 1024;
 constexpr int kNaMaxSplits = 320;
-static_assert(kNaMaxN <= kFuseScoreMaxN, "the canvas is scored by the merge's last CTA");
+static_assert(kNaMaxN <= kFusedMaxPositions, "the head kernel compacts the mask");
 constexpr int kNaMaxDevices = 64;
 
 // Arena layout (byte offsets, each 256-byte aligned).
@@ -215,30 +215,29 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
     // The per-step count/status words must start from zero on every call.
     cudaError_t e = cudaMemsetAsync(meta, 0, kMetaWords * 4, stream);
     if (e == cudaSuccess) {
-        // no plan table (it would have to be allocated): the compaction kernel evaluates the
+        // no plan table (it would have to be allocated): the head kernel evaluates the
         // head-tiling plan itself
         const HeadPlanInputs plan_in{num_n, splits, pair_slots,
                                      head_stream_in_tiles(V, d, dev->num_sms), RPD_TILING_AUTO};
-        CompactParams cp{mask, q_of_pos, pos_of_q, canvas_off, meta, 1, N, K, plan_in, nullptr, 0,
-                         rule.block, 0};
-        e = launch_compact(cp, stream);
-    }
-    if (e == cudaSuccess) {
-        NormParams np{static_cast<const __nv_bfloat16 *>(hidden),
-                      static_cast<const __nv_bfloat16 *>(g_norm), pos_of_q, nullptr, meta, u,
-                      inv_rms, N, d, eps};
-        e = launch_gather_norm(np, std::min(dev->num_sms * 8, (K * N + 7) / 8), stream);
-    }
-    if (e == cudaSuccess) {
-        HeadParams hp{inv_rms, partials, meta, V, d, splits, kWaitLimitNs, 0};
-        e = launch_head(maps, hp, dev->head_grid, stream);
-    }
-    if (e == cudaSuccess) {
-        // the merge's last CTA scores the canvas (N <= kNaMaxN <= kFuseScoreMaxN), as rpd_step does
-        ScoreParams sp{};
+        HeadParams hp{};
+        hp.compact = CompactParams{mask, q_of_pos, pos_of_q, canvas_off, meta, 1, N, K, plan_in,
+                                   nullptr, 0, rule.block, 0};
+        hp.norm = NormParams{static_cast<const __nv_bfloat16 *>(hidden),
+                             static_cast<const __nv_bfloat16 *>(g_norm), pos_of_q, nullptr, meta, u,
+                             inv_rms, N, d, eps};
+        hp.partials = partials;
+        hp.meta = meta;
+        hp.from_mask = 1;
+        hp.last_pass = 1;
+        hp.V = V;
+        hp.d = d;
+        hp.max_splits = splits;
+        hp.wait_limit_ns = kWaitLimitNs;
+        hp.merge = MergeArgs{partials, splits, row_arg, row_pmax, row_H};
+        hp.score_canvas = 1;
+        ScoreParams &sp = hp.score;
         sp.mask = mask;
         sp.q_of_pos = q_of_pos;
-        sp.canvas_off = canvas_off;
         sp.meta = meta;
         sp.row_arg = row_arg;
         sp.row_pmax = row_pmax;
@@ -255,10 +254,9 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
         sp.k_max = rule.k_max;
         sp.window = rule.window;
         sp.block = rule.block;
-        sp.tau[0] = tau;
-        sp.budget[0] = budget;
-        e = launch_merge_score(MergeArgs{partials, splits, row_arg, row_pmax, row_H}, meta, nullptr,
-                               dev->num_sms * 4, sp, stream);
+        sp.tau = tau;
+        sp.budget = budget;
+        e = launch_head(maps, hp, dev->head_grid, stream);
     }
     if (e != cudaSuccess) {
         set_last_error((std::string("rpd_step_noalloc launch failed: ") + cudaGetErrorString(e)).c_str());

@@ -1,0 +1,81 @@
+"""The step as one kernel: sizes at the edges of the in-kernel compaction (words of the bitmap,
+the largest number of positions it takes, masks at any address), of the claimed rows and of the
+merge, against the oracle."""
+import pytest
+import torch
+
+import workloads as WL
+from oracle import rpd_oracle as O
+
+pytestmark = pytest.mark.gpu
+
+if not torch.cuda.is_available():  # collected on CPU machines, never run there
+    pytest.skip("needs a CUDA GPU", allow_module_level=True)
+
+from gpu_util import DeviceRunner, bits  # noqa: E402
+from parity import compare_block_step, compare_step  # noqa: E402
+
+
+def make(seed, K, N, d, V):
+    W, g = WL.make_head(V, d, seed, w_std=0.08)
+    cv = WL.make_hidden(W, K, N, seed + 1000, WL.u_profile(N, 0.5, 3.0),
+                        WL.calibrated_sigma(V, d, 0.08, 3.0), flip_frac=0.1)
+    return W, g, cv.hidden
+
+
+@pytest.mark.parametrize("N,count", [(1, 1), (15, 7), (16, 16), (31, 2), (33, 33), (64, 1), (320, 200),
+                                     (321, 9)])
+@pytest.mark.parametrize("offset", [0, 1, 8])
+def test_compaction_at_word_edges_and_any_mask_address(N, count, offset):
+    K, d, V = 2, 128, 1024
+    W, g, hidden = make(700 + N, K, N, d, V)
+    mask = WL.uniform_fraction_mask(N, count / N, N)
+    ref = O.rpd_step(bits(hidden), mask.numpy(), bits(g), bits(W), 1e-6, 0.9, 1.0, "llada")
+    runner = DeviceRunner(W, g, K)
+    try:
+        room = torch.zeros(N + 32, dtype=torch.uint8, device="cuda")
+        m = room[offset:offset + N]
+        m.copy_(mask)
+        h = hidden.cuda()
+        out = runner._alloc(1, N)
+        runner.ctx.step(h, m, 0.9, 1.0, out["commit"][0], out["token"][0], out["stats"][0])
+        got = runner._fetch(out, m.reshape(1, N), 1)[0]
+        assert int(room.sum()) == int(m.sum())  # nothing beside the mask was written
+    finally:
+        runner.close()
+    compare_step(ref, got)
+
+
+@pytest.mark.parametrize("B,N", [(8, 1024), (9, 911), (3, 2731)])  # 8192, 8199 and 8193 positions
+@pytest.mark.parametrize("block", [0, 32])
+def test_batches_around_the_compaction_limit(B, N, block):
+    K, d, V = 1, 64, 512
+    W, g = WL.make_head(V, d, 41, w_std=0.08)
+    gen = torch.Generator().manual_seed(B)
+    hidden = torch.randn(K, B, N, d, generator=gen).to(torch.bfloat16) * 2
+    masks = torch.stack([WL.uniform_fraction_mask(N, 0.02 + 0.9 * b / B, 50 + b) for b in range(B)])
+    masks[1] = 0
+    runner = DeviceRunner(W, g, K, rule="llada_block" if block else "llada")
+    try:
+        got = runner.step_batched(hidden, masks, [0.9] * B, [1.5] * B)
+    finally:
+        runner.close()
+    for b in (0, 1, 2, B - 1):
+        args = (bits(hidden[:, b].contiguous()), masks[b].numpy(), bits(g), bits(W), 1e-6, 0.9)
+        ref = O.rpd_block_step(*args, "llada", block) if block else O.rpd_step(*args, 1.5, "llada")
+        (compare_block_step if block else compare_step)(ref, got[b])
+        assert got[b]["stats"]["n_rows"] == got[0]["stats"]["n_rows"]
+
+
+def test_more_rows_than_the_grid_has_warps_and_splits_of_every_width():
+    """Rows that warps claim several at a time (over 2432), and merges of 1 to 32 lanes per row."""
+    for V, N in [(300, 640), (2048, 650), (20000, 5)]:
+        K, d = 4, 64
+        W, g, hidden = make(90 + N, K, N, d, V)
+        mask = torch.ones(N, dtype=torch.uint8)
+        ref = O.rpd_step(bits(hidden), mask.numpy(), bits(g), bits(W), 1e-6, 0.9, 1.0, "llada")
+        runner = DeviceRunner(W, g, K)
+        try:
+            compare_step(ref, runner.step(hidden, mask, 0.9, 1.0))
+        finally:
+            runner.close()

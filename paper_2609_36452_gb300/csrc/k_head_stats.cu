@@ -85,40 +85,65 @@ struct UnitCursor {
     }
 };
 
-// Fold one 32-entry chunk of logits, column col0 + i in v[i], into the running statistics
-// (v is scaled to log2 units in place).
+// Fold one 32-entry chunk of a row's logits, column col0 + i in v[i], into the row's running
+// statistics: top = the largest logit so far (unscaled), and in log2 units, x = logit * scale,
+// s = sum 2^(x - x_top), t = sum 2^(x - x_top) (x - x_top), a = its lowest index.
+//
+// Bound by instruction issue (two warps per scheduler, beside the MMA issuer): the maximum is
+// taken of the unscaled logits, three at a time, its index is looked for only in a chunk that
+// raises it, and the rest runs on pairs.  5 instructions per logit where scaling, comparing and
+// exponentiating one logit at a time took 11.  (v - top) * scale is also closer to x - x_top than
+// the difference of two rounded products.
 template <bool kFull>
-__device__ __forceinline__ void fold_chunk(float (&x)[32], float scale, int col0, int V,
-                                           float &run_m, float &run_s, float &run_t,
-                                           int &run_a) {
-    float cmax = -INFINITY;
-    int carg = 0;
+__device__ __forceinline__ void fold_chunk(float (&v)[32], float scale, int col0, int V, float &top,
+                                           float &s, float &t, int &a) {
+    if (!kFull) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        x[i] *= scale;
-        if (!kFull && col0 + i >= V) x[i] = -INFINITY;
-        if (x[i] > cmax) {
-            cmax = x[i];
-            carg = i;
-        }
+        for (int i = 0; i < 32; ++i)
+            if (col0 + i >= V) v[i] = -INFINITY;
     }
-    if (cmax > run_m) {
-        if (run_s > 0.f) {
-            const float dm = run_m - cmax;
-            const float alpha = exp2f(dm);
-            run_t = alpha * fmaf(dm, run_s, run_t);
-            run_s = alpha * run_s;
-        }
-        run_m = cmax;
-        run_a = col0 + carg;
-    }
+    float c = v[0];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-        if (kFull || col0 + i < V) {
-            const float dl = x[i] - run_m;
-            const float e = exp2f(dl);
-            run_s += e;
-            run_t = fmaf(e, dl, run_t);
+    for (int i = 1; i < 32; ++i) c = fmaxf(c, v[i]);
+    if (c > top) {
+        if (s > 0.f) {
+            const float d = (top - c) * scale;
+            const float alpha = ex2(d);
+            t = alpha * fmaf(d, s, t);
+            s = alpha * s;
+        }
+        top = c;
+        int first = 31;
+#pragma unroll
+        for (int i = 30; i >= 0; --i) first = v[i] == c ? i : first;
+        a = col0 + first;
+    }
+    if (kFull) {
+        const f32x2 minus = pack2(-top, -top), scale2 = pack2(scale, scale);
+        f32x2 s2 = pack2(s, 0.f), t2 = pack2(t, 0.f);
+#pragma unroll
+        for (int i = 0; i < 32; i += 2) {
+            const f32x2 d = mul2(add2(pack2(v[i], v[i + 1]), minus), scale2);
+            float lo, hi;
+            unpack2(d, lo, hi);
+            const f32x2 e = pack2(ex2(lo), ex2(hi));
+            s2 = add2(s2, e);
+            t2 = fma2(e, d, t2);
+        }
+        float lo, hi;
+        unpack2(s2, lo, hi);
+        s = lo + hi;
+        unpack2(t2, lo, hi);
+        t = lo + hi;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 32; ++i) {
+            if (col0 + i < V) {
+                const float d = (v[i] - top) * scale;
+                const float e = ex2(d);
+                s += e;
+                t = fmaf(e, d, t);
+            }
         }
     }
 }
@@ -205,7 +230,7 @@ __device__ __forceinline__ void init_barriers(const HeadSmem &sm) {
         mbar_init(&sm.unit_full[i], 1);
         mbar_init(&sm.unit_empty[i], 2 + 2 * kSwapEpiWarps);
     }
-    // ring tiles: a chunk is read by one warp per TMEM sub-partition in each CTA
+    // a chunk is read by one warp per TMEM sub-partition in each CTA
     for (uint32_t i = 0; i < kTmemCols / 32; ++i) mbar_init(&sm.chunk_free[i], 8);
     mbar_init(sm.epi, 32 * kSwapEpiWarps);
     mbar_init(sm.drain, 1);
@@ -514,7 +539,7 @@ __device__ __forceinline__ int head_pair(const CUtensorMap *tmU, const CUtensorM
             if (!ok) break;
             if (valid && rpd_check(g < p.max_splits, p.meta + kMetaStatus)) {
                 p.partials[static_cast<size_t>(r) * p.max_splits + g] =
-                    make_float4(run_m, run_s, run_t, __int_as_float(run_a));
+                    make_float4(run_m * scale, run_s, run_t, __int_as_float(run_a));
             }
         }
     }
@@ -542,18 +567,14 @@ __device__ __forceinline__ bool epi_sync(uint64_t *bar, uint32_t &phase, volatil
 // stage, from the tensor map whose box has that height (16 to 256 rows; a stage with a second,
 // small copy measured far slower).
 //
-// TMEM: 16 chunks of 32 columns.  A tile of at most 256 columns alternates between the two
-// halves (double buffering); a tile of 288 or 320 columns follows its predecessor around the
-// ring of chunks, so that it waits only for the chunks it overwrites (with 288 columns, the
-// first two of its predecessor's nine) instead of for the whole epilogue of its predecessor;
-// larger tiles use columns [0, G) in turn.  A tile's columns are issued as one MMA per
-// contiguous segment of at most 256 columns per 16-wide K-step, and the MMA for columns
-// [c, c + N) of segment j takes the first N/2 of them from rows [o_j, o_j + N/2) of the even
-// CTA's half and the rest from the same rows of the odd CTA's half, o_j being half the columns
-// of the tile before segment j; the epilogue maps each column back to its row.
+// TMEM: 16 chunks of 32 columns, in which tiles alternate between two places (swap_place); the
+// MMAs of a tile wait for the chunks that it shares with its predecessor - two with 288 rows,
+// all of them with 512 -, which the epilogue reads and releases first.  A segment's MMA takes the
+// first half of its columns' rows from the even CTA's half of the group and the rest from the odd
+// CTA's; the epilogue maps each column back to its row.
 //
 // Epilogue: 8 warps, two per TMEM sub-partition, alternating its chunks.  A warp loads a
-// 32 x 32 block, releases the chunk (ring tiles), transposes the block through shared memory
+// 32 x 32 block, releases a shared chunk, transposes the block through shared memory
 // so that each thread holds one row's 32 vocabulary entries, and folds them into that row's
 // running statistics (per sub-partition, in shared memory).  At the end of a work unit the
 // four sub-partitions' statistics of each row are combined and each CTA writes one partial
@@ -564,10 +585,8 @@ __device__ __forceinline__ bool epi_sync(uint64_t *bar, uint32_t &phase, volatil
 template <int kSegs>
 __device__ __forceinline__ bool swap_tile_mmas(const HeadSmem &sm, int num_kb, int stages,
                                                int stage_bytes, int &stage, uint32_t &phase,
-                                               uint32_t d0, uint32_t d1, uint32_t d2, uint32_t id0,
-                                               uint32_t id1, uint32_t id2, uint32_t bo1,
-                                               uint32_t bo2, volatile int *abort_flag,
-                                               uint64_t limit) {
+                                               uint32_t d0, uint32_t d1, uint32_t id0, uint32_t id1,
+                                               uint32_t bo1, volatile int *abort_flag, uint64_t limit) {
     for (int kb = 0; kb < num_kb; ++kb) {
         if (!mbar_wait_bounded_warp(&sm.full[stage], phase, abort_flag, limit)) return false;
         tc_fence_after_sync();
@@ -580,9 +599,6 @@ __device__ __forceinline__ bool swap_tile_mmas(const HeadSmem &sm, int num_kb, i
             if (kSegs > 1)
                 umma_bf16_pair_warp(d1, smem_desc_sw128(a0 + kk * 32), smem_desc_sw128(b0 + bo1 + kk * 32),
                                     id1, accum);
-            if (kSegs > 2)
-                umma_bf16_pair_warp(d2, smem_desc_sw128(a0 + kk * 32), smem_desc_sw128(b0 + bo2 + kk * 32),
-                                    id2, accum);
         }
         umma_commit_pair_multicast_warp(&sm.empty[stage], 0x3);
         if (++stage == stages) {
@@ -593,21 +609,28 @@ __device__ __forceinline__ bool swap_tile_mmas(const HeadSmem &sm, int num_kb, i
     return true;
 }
 
-// Column segments of a rows-on-N tile placed at TMEM chunk c0: up to three contiguous column
-// ranges, each within [0, 512) and at most 256 wide (the MMA's N).
-struct SwapSegs {
-    int col0, col1, col2;  // first TMEM column of each
-    int n0, n1, n2;        // widths (0: unused)
+// Where a rows-on-N tile of ng columns lies in TMEM, and its column segments (the MMA's N is at
+// most 256).  Tiles alternate between two placements.  Up to 256 columns: the two halves, one
+// segment.  More: the two ends of TMEM, overlapping in the middle, and two segments as equal as
+// whole 32-column steps allow: an MMA of few columns costs nearly as much as one of 128 (the
+// head's half of the operands has to be read all the same; 44 cycles for 32 columns, 64 for 128),
+// so 288 columns take 144 cycles a step as 160 + 128 and 173 as 256 + 32.
+struct SwapPlace {
+    uint32_t chunk0;      // first TMEM chunk (of 32 columns)
+    uint32_t shared0, shared1;  // chunks that both placements use: [shared0, shared1)
+    int n0, n1;           // segment widths (n1 = 0: one segment)
 };
-__device__ __forceinline__ SwapSegs swap_segments(int c0, int ng) {
-    SwapSegs g;
-    g.col0 = c0 * 32;
-    g.n0 = min(min(ng, kTmemCols - g.col0), kPairTileM);
-    g.col1 = (g.col0 + g.n0) % kTmemCols;
-    g.n1 = min(min(ng - g.n0, kTmemCols - g.col1), kPairTileM);
-    g.col2 = (g.col1 + g.n1) % kTmemCols;
-    g.n2 = ng - g.n0 - g.n1;
-    return g;
+__device__ __forceinline__ SwapPlace swap_place(int ng, uint32_t odd_tile) {
+    constexpr uint32_t kChunks = kTmemCols / 32;
+    const uint32_t nch = static_cast<uint32_t>(ng) / 32;
+    SwapPlace s;
+    const uint32_t odd0 = nch > kChunks / 2 ? kChunks - nch : kChunks / 2;
+    s.chunk0 = odd_tile ? odd0 : 0u;
+    s.shared0 = odd0;
+    s.shared1 = nch > odd0 ? nch : odd0;
+    s.n0 = ng <= kPairTileM ? ng : static_cast<int>((nch + 1) / 2) * 32;
+    s.n1 = ng - s.n0;
+    return s;
 }
 
 __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] */,
@@ -622,15 +645,7 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
-    // TMEM placement: tiles of at most 256 columns alternate between the two halves; tiles of
-    // 288 to 320 columns follow one another around a ring of 16 chunks of 32 columns; larger
-    // tiles use all of TMEM in turn (with 11 or more chunks a tile would wait for nearly all of
-    // its predecessor's chunks anyway, and the ring's column splits measured slower there)
-    constexpr uint32_t kChunks = kTmemCols / 32;
-    constexpr uint32_t kRingMaxChunks = 10;
     const uint32_t nch = static_cast<uint32_t>(ng / 32);
-    const bool single = nch > kRingMaxChunks;
-    const bool ring = 2 * nch > kChunks && !single;
     const int stage_b = (ng / 2) * kTileK * 2;
     const int stage_bytes = kSwapStageBytesA + stage_b;
     // region: operand ring (as many stages as fit), transpose blocks, statistics [4][ng], RMS
@@ -679,46 +694,29 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
                 int m, g, v0, v1;
                 tw.unit(u, m, g, v0, v1);
                 for (int n = v0; ok && n < v1; ++n, ++tile_iter) {
-                    // tile t-2 read (its accumulator barrier is reused), or tile t-1 for tiles
-                    // that use all of TMEM ...
-                    const uint32_t acc = single ? 0u : (tile_iter & 1u);
-                    const uint32_t acc_phase = (single ? tile_iter : (tile_iter >> 1)) & 1u;
-                    if (!mbar_wait_bounded_warp(&acc_empty[acc], acc_phase ^ 1u, abort_flag,
+                    // tile t-2, which had the same place, has been read ...
+                    const uint32_t acc = tile_iter & 1u;
+                    if (!mbar_wait_bounded_warp(&acc_empty[acc], ((tile_iter >> 1) & 1u) ^ 1u, abort_flag,
                                                 p.wait_limit_ns)) {
                         ok = false;
                         break;
                     }
-                    // ... and, on the ring, the chunks of tile t-1 this tile overwrites
-                    const uint32_t a0 = tile_iter * nch;
-                    if (ring && tile_iter > 0) {
-                        for (uint32_t c = kChunks - nch; ok && c < nch; ++c) {
-                            const uint32_t a = a0 + c;  // previous use: a - 16, in tile t-1
-                            if (!mbar_wait_bounded_warp(&chunk_free[a % kChunks], ((a / kChunks) & 1u) ^ 1u,
-                                                        abort_flag, p.wait_limit_ns))
-                                ok = false;
-                        }
-                        if (!ok) break;
-                    }
+                    // ... and so have the chunks that this tile shares with tile t-1
+                    const SwapPlace place = swap_place(ng, acc);
+                    for (uint32_t c = place.shared0; ok && tile_iter > 0 && c < place.shared1; ++c)
+                        ok = mbar_wait_bounded_warp(&chunk_free[c], (tile_iter - 1) & 1u, abort_flag,
+                                                    p.wait_limit_ns);
+                    if (!ok) break;
                     tc_fence_after_sync();
-                    const SwapSegs sg = swap_segments(static_cast<int>(ring ? a0 % kChunks : acc * 8u), ng);
-                    // (single: acc = 0, the tile starts at column 0)
-                    const uint32_t d0 = tmem_base + sg.col0, d1 = tmem_base + sg.col1,
-                                   d2 = tmem_base + sg.col2;
-                    const uint32_t id0 = idesc_bf16_f32(kPairTileM, sg.n0);
-                    const uint32_t id1 = idesc_bf16_f32(kPairTileM, sg.n1 > 0 ? sg.n1 : 32);
-                    const uint32_t id2 = idesc_bf16_f32(kPairTileM, sg.n2 > 0 ? sg.n2 : 32);
-                    // segment j's rows of u start at row (columns before it) / 2 of each CTA's half
-                    const uint32_t bo1 = static_cast<uint32_t>((sg.n0 / 2) * kTileK * 2);
-                    const uint32_t bo2 = static_cast<uint32_t>(((sg.n0 + sg.n1) / 2) * kTileK * 2);
-                    ok = sg.n2 > 0 ? swap_tile_mmas<3>(sm, num_kb, stages, stage_bytes, stage, phase, d0, d1,
-                                                       d2, id0, id1, id2, bo1, bo2, abort_flag,
-                                                       p.wait_limit_ns)
-                       : sg.n1 > 0 ? swap_tile_mmas<2>(sm, num_kb, stages, stage_bytes, stage, phase, d0,
-                                                       d1, d2, id0, id1, id2, bo1, bo2, abort_flag,
-                                                       p.wait_limit_ns)
-                                   : swap_tile_mmas<1>(sm, num_kb, stages, stage_bytes, stage, phase, d0,
-                                                       d1, d2, id0, id1, id2, bo1, bo2, abort_flag,
-                                                       p.wait_limit_ns);
+                    const uint32_t d0 = tmem_base + place.chunk0 * 32, d1 = d0 + place.n0;
+                    const uint32_t id0 = idesc_bf16_f32(kPairTileM, place.n0);
+                    const uint32_t id1 = idesc_bf16_f32(kPairTileM, place.n1 > 0 ? place.n1 : 32);
+                    // the second segment's rows of u start at row n0 / 2 of each CTA's half
+                    const uint32_t bo1 = static_cast<uint32_t>((place.n0 / 2) * kTileK * 2);
+                    ok = place.n1 > 0 ? swap_tile_mmas<2>(sm, num_kb, stages, stage_bytes, stage, phase, d0,
+                                                          d1, id0, id1, bo1, abort_flag, p.wait_limit_ns)
+                                      : swap_tile_mmas<1>(sm, num_kb, stages, stage_bytes, stage, phase, d0,
+                                                          d1, id0, id1, bo1, abort_flag, p.wait_limit_ns);
                     if (!ok) break;
                     umma_commit_pair_multicast_warp(&acc_full[acc], 0x3);
                 }
@@ -733,6 +731,7 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
         const int etid = (warp - 2) * 32 + lane;  // 0 .. kEpiThreads-1
         const int chunk0 = (warp - 2) / 4;        // the two warps of a sub-partition alternate chunks
         constexpr int kChunkStep = kSwapEpiWarps / 4;
+        static_assert(kChunkStep == 2, "chunks are shared out by parity");
         const uint32_t lane_base = tmem_base + (static_cast<uint32_t>(sub * 32) << 16);
         const uint32_t acc_empty0 = mapa_shared(smem_u32(&acc_empty[0]), 0);
         const uint32_t chunk_free0 = mapa_shared(smem_u32(&chunk_free[0]), 0);
@@ -761,25 +760,31 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
                 scales[rl] = m * ng + rl < rows ? p.norm.inv_rms[m * ng + rl] * kLog2e : 0.f;
             if (!epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns)) break;
             for (int n = v0; n < v1; ++n, ++tile_iter) {
-                const uint32_t acc = single ? 0u : (tile_iter & 1u);
-                const uint32_t acc_phase = (single ? tile_iter : (tile_iter >> 1)) & 1u;
-                if (!mbar_wait_bounded(&acc_full[acc], acc_phase, abort_flag, p.wait_limit_ns)) {
+                const uint32_t acc = tile_iter & 1u;
+                if (!mbar_wait_bounded(&acc_full[acc], (tile_iter >> 1) & 1u, abort_flag, p.wait_limit_ns)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after_sync();
-                const uint32_t c0 = ring ? (tile_iter * nch) % kChunks : acc * 8u;
-                const SwapSegs sg = swap_segments(static_cast<int>(c0), ng);
-                const int x1 = sg.n0, x2 = sg.n0 + sg.n1;
+                const SwapPlace place = swap_place(ng, acc);
                 // the 32 vocabulary entries of this warp's sub-partition
                 const int vbase = n * kTileN + static_cast<int>(rank) * kPairHalfRows + sub * 32;
                 const bool full_tile = vbase + 32 <= p.V;
+                // This warp's chunks are always the same ones (their statistics are its own); the
+                // next tile waits for the shared chunks, so those come first.
+                const int chunks = (static_cast<int>(nch) - chunk0 + kChunkStep - 1) / kChunkStep;
+                int c = chunk0;
+                if (place.shared1 > place.shared0) {
+                    const int first = static_cast<int>(place.shared0 - place.chunk0);
+                    c = first + ((first ^ chunk0) & 1);
+                    if (c >= static_cast<int>(nch)) c = chunk0;
+                }
 #pragma unroll 1
-                for (int c = chunk0; c < static_cast<int>(nch); c += kChunkStep) {
+                for (int i = 0; i < chunks; ++i) {
                     float v[32];
-                    const uint32_t slot = (c0 + static_cast<uint32_t>(c)) % kChunks;
+                    const uint32_t slot = place.chunk0 + static_cast<uint32_t>(c);
                     tmem_ld_32x32b_x32(lane_base + slot * 32, v);
-                    if (ring) {  // the chunk's columns may be overwritten by the next tile now
+                    if (slot >= place.shared0 && slot < place.shared1) {  // the next tile may overwrite it
                         tc_fence_before_sync();
                         __syncwarp();
                         if (lane == 0) mbar_arrive_cluster(chunk_free0 + slot * static_cast<uint32_t>(sizeof(uint64_t)));
@@ -793,15 +798,15 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
 #pragma unroll
                     for (int i = 0; i < 32; ++i) v[i] = xp[i * kSwapXposeStride + lane];
                     __syncwarp();
-                    // now v[i] = logit of vocabulary entry vbase + i for TMEM column c*32 + lane,
-                    // i.e. for row rl of the group: MMA j takes its first N_j/2 columns from the
-                    // even CTA's rows [o_j, o_j + N_j/2) and the rest from the odd CTA's, and CTA r
-                    // holds the group's rows [r * ng/2, +ng/2) (o_0 = 0, o_1 = n0/2)
-                    const int col = c * 32 + lane;  // column of the tile
-                    const int xj = col < x1 ? 0 : (col < x2 ? x1 : x2);
-                    const int nj = col < x1 ? sg.n0 : (col < x2 ? sg.n1 : sg.n2);
-                    const int x = col - xj;
-                    const int rl = xj / 2 + (x < nj / 2 ? x : ng / 2 + (x - nj / 2));
+                    // now v[i] = logit of vocabulary entry vbase + i for column c*32 + lane, i.e. for
+                    // row rl of the group: a segment's MMA takes its first half of columns from the
+                    // even CTA's rows [o, o + n/2) and the rest from the odd CTA's, and CTA r holds
+                    // the group's rows [r * ng/2, +ng/2) (o = 0, then n0/2)
+                    const int col = c * 32 + lane;
+                    const int x0 = col < place.n0 ? 0 : place.n0;
+                    const int half_n = (col < place.n0 ? place.n0 : place.n1) / 2;
+                    const int x = col - x0;
+                    const int rl = x0 / 2 + (x < half_n ? x : ng / 2 + (x - half_n));
                     const float scale = scales[rl];
                     float4 st = stats[sub * ng + rl];
                     int a = __float_as_int(st.w);
@@ -811,6 +816,8 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
                         fold_chunk<false>(v, scale, vbase, p.V, st.x, st.y, st.z, a);
                     st.w = __int_as_float(a);
                     stats[sub * ng + rl] = st;
+                    c += kChunkStep;
+                    if (c >= static_cast<int>(nch)) c = chunk0;
                 }
                 tc_fence_before_sync();
                 __syncwarp();
@@ -824,12 +831,14 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
             if (!epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns)) break;
             for (int rl = etid; rl < ng; rl += kEpiThreads) {
                 const int r = m * ng + rl;
-                float4 acc4 = stats[rl];
-                stats[rl] = kEmpty;
-#pragma unroll
-                for (int s4 = 1; s4 < 4; ++s4) {
-                    acc4 = merge_stat(acc4, stats[s4 * ng + rl]);
+                const float scale = scales[rl];
+                float4 acc4 = kEmpty;
+#pragma unroll 1
+                for (int s4 = 0; s4 < 4; ++s4) {
+                    float4 st = stats[s4 * ng + rl];
                     stats[s4 * ng + rl] = kEmpty;
+                    st.x *= scale;  // log2 units
+                    acc4 = merge_stat(acc4, st);
                 }
                 if (r < rows && rpd_check(2 * g + static_cast<int>(rank) < p.max_splits, p.meta + kMetaStatus))
                     p.partials[static_cast<size_t>(r) * p.max_splits + 2 * g + static_cast<int>(rank)] = acc4;

@@ -180,6 +180,7 @@ struct HeadSmem {
     uint32_t *tmem_slot;
     volatile int *abort_flag;
     volatile int *unit_ring;  // [kUnitRing] claimed unit indices
+    volatile int *stale;      // the canvas was already being scored when the mask was read
     MaskMap map;              // the compaction (and the pass) of this CTA
 };
 
@@ -201,13 +202,14 @@ __device__ __forceinline__ HeadSmem carve_smem(uint8_t *raw) {
     s.tmem_slot = reinterpret_cast<uint32_t *>(s.chunk_free + kTmemCols / 32);
     s.abort_flag = reinterpret_cast<volatile int *>(s.tmem_slot + 1);
     s.unit_ring = s.abort_flag + 1;
+    s.stale = s.unit_ring + kUnitRing;
     s.map.words = reinterpret_cast<uint32_t *>(base + kHeadRegionBytes + kHeadBarrierBytes);
     s.map.before = reinterpret_cast<uint16_t *>(s.map.words + kMaskWords);
     s.map.pass = reinterpret_cast<PassInfo *>(s.map.before + kMaskWords + 8);
     return s;
 }
 
-static_assert((2 * kSwapMaxStages + 6 + 2 * kUnitRing + kTmemCols / 32) * 8 + 8 + 4 * kUnitRing <=
+static_assert((2 * kSwapMaxStages + 6 + 2 * kUnitRing + kTmemCols / 32) * 8 + 12 + 4 * kUnitRing <=
                   kHeadBarrierBytes,
               "barrier region");
 
@@ -235,12 +237,15 @@ __device__ __forceinline__ void init_barriers(const HeadSmem &sm) {
     mbar_init(sm.epi, 32 * kSwapEpiWarps);
     mbar_init(sm.drain, 1);
     *sm.abort_flag = 0;
+    *sm.stale = 0;
     fence_mbar_init();
 }
 
-// An epilogue warp's acquire of the other CTAs' inv_rms, long before its first tile is done.
-__device__ __forceinline__ bool wait_for_rows(const HeadParams &p, const HeadSmem &sm, int rows) {
-    return counter_wait(&p.meta[kMetaRowsDone], rows, sm.abort_flag, p.wait_limit_ns, 500);
+// Wait for every CTA's gathered rows (the bound grows with what the grid has to gather).
+__device__ __forceinline__ bool wait_for_rows(const HeadParams &p, const HeadSmem &sm, int rows,
+                                              unsigned sleep_ns) {
+    return counter_wait(&p.meta[kMetaRowsDone], rows, sm.abort_flag,
+                        p.wait_limit_ns * (1 + static_cast<unsigned>(rows) / 4096), sleep_ns);
 }
 
 // The TMA producer's claim of the next work unit (-1: none left): the even CTA takes it from the
@@ -331,7 +336,7 @@ __device__ __forceinline__ int copy_ahead(const HeadParams &p, const HeadSmem &s
         else
             tma_load_2d_pair(dst, c.w, bar, x, y);
     }
-    if (!counter_wait(&p.meta[kMetaRowsDone], rows, sm.abort_flag, p.wait_limit_ns)) return -1;
+    if (!wait_for_rows(p, sm, rows, 0)) return -1;
     proxy_fence();
     for (int s = 0; s < ahead; ++s)
         tma_load_2d_pair(sm.ring + s * c.stage_bytes + c.u_off, c.u,
@@ -339,19 +344,19 @@ __device__ __forceinline__ int copy_ahead(const HeadParams &p, const HeadSmem &s
     return ahead;
 }
 
-// The TMA producer of one CTA (one thread); returns the units it has taken.
+// The TMA producer of one CTA (one thread).
 //
 // With a single row tile every head tile is read once and is dropped from L2 first, which keeps
 // the hidden rows, the partials and the code of the step's other phases there from one step to
 // the next: 171.5 -> 166.4 us at 20 rows (LLaDA head), of which 3 us after the last tile.  Several
 // row tiles re-read a head tile at slightly different times: with that policy, and with an
 // explicit normal one instead of none, first-step and serving passes were 1.5 % slower.
-__device__ __forceinline__ int produce(const HeadParams &p, const HeadSmem &sm, const Copies &c,
-                                       uint32_t rank, const TileWalk &tw, int rows, int num_kb, int first) {
+__device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm, const Copies &c,
+                                        uint32_t rank, const TileWalk &tw, int rows, int num_kb, int first) {
     const uint32_t full0 = mapa_shared(smem_u32(&sm.full[0]), 0);
     const uint64_t evict_first = l2_evict_first();
     const bool once = tw.num_m == 1;
-    int taken = 0;
+    bool started = false;
     int stage = 0;
     uint32_t phase = 0;
     long long fills = 0;
@@ -365,7 +370,8 @@ __device__ __forceinline__ int produce(const HeadParams &p, const HeadSmem &sm, 
         tw.unit(u, m, g, n0, n1);
         const int u_row = m * c.u_rows + c.u_row0;
         int kb0 = 0;
-        if (taken++ == 0) {
+        if (!started) {
+            started = true;
             kb0 = copy_ahead(p, sm, c, rank, full0, once, evict_first, n0, u_row, rows, num_kb);
             fills = kb0 < 0 ? min(c.stages, num_kb) : kb0;
             if (kb0 < 0) break;
@@ -389,7 +395,6 @@ __device__ __forceinline__ int produce(const HeadParams &p, const HeadSmem &sm, 
         if (n_s > 0)
             mbar_wait_drain(&sm.empty[s], static_cast<uint32_t>((n_s - 1) & 1), p.wait_limit_ns / 8);
     }
-    return taken;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -404,7 +409,7 @@ __device__ __forceinline__ int produce(const HeadParams &p, const HeadSmem &sm, 
 // 64 KB per stage); empty[s], acc_full[a] and drain receive multicast commits from the MMA
 // thread in both CTAs; acc_empty[a] lives in the even CTA and counts the 4 epilogue warps
 // of both CTAs (8 arrivals).
-__device__ __forceinline__ int head_pair(const CUtensorMap *tmU, const CUtensorMap *tmW,
+__device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensorMap *tmW,
                                           const HeadParams &p, const HeadSmem &sm, int rows,
                                           int splits, int first_unit, uint32_t tmem_base) {
     constexpr int kStageBytes = kPairStageBytesA + kPairStageBytesB;
@@ -419,14 +424,13 @@ __device__ __forceinline__ int head_pair(const CUtensorMap *tmU, const CUtensorM
     TileWalk tw;
     tw.init(rows, kPairTileM, p.V, p.d, splits);
     const int num_kb = (p.d + kTileK - 1) / kTileK;
-    int taken = 0;
 
     if (warp == 0) {
         if (lane == 0 && !p.stall) {
             // ------------------------------------------------------- TMA producer (both CTAs)
             const Copies copies{tmW, tmU, kPairStages, kStageBytes, kPairStageBytesA, 0, kPairTileM,
                                 static_cast<int>(rank) * kPairHalfRows};
-            taken = produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
+            produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
         }
     } else if (warp == 1) {
         if (rank == 0) {
@@ -495,7 +499,8 @@ __device__ __forceinline__ int head_pair(const CUtensorMap *tmU, const CUtensorM
         const uint32_t acc_empty0 = mapa_shared(smem_u32(&acc_empty[0]), 0);
         const uint32_t unit_empty0 = mapa_shared(smem_u32(&unit_empty[0]), 0);
         uint32_t tile_iter = 0;
-        bool ok = wait_for_rows(p, sm, rows);
+        // the other CTAs' inv_rms, long before this warp's first tile is done
+        bool ok = wait_for_rows(p, sm, rows, 500);
         UnitCursor uc;
         while (ok) {
             if (!mbar_wait_bounded_cluster(&unit_full[uc.slot], uc.phase, abort_flag, p.wait_limit_ns))
@@ -541,9 +546,10 @@ __device__ __forceinline__ int head_pair(const CUtensorMap *tmU, const CUtensorM
                 p.partials[static_cast<size_t>(r) * p.max_splits + g] =
                     make_float4(run_m * scale, run_s, run_t, __int_as_float(run_a));
             }
+            __syncwarp();
+            if (lane == 0) counter_add_release(&p.meta[kMetaUnitsDone], 1);
         }
     }
-    return taken;
 }
 
 // Barrier of the rows-on-N epilogue's threads: every thread arrives (release) and waits
@@ -633,7 +639,7 @@ __device__ __forceinline__ SwapPlace swap_place(int ng, uint32_t odd_tile) {
     return s;
 }
 
-__device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] */,
+__device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps] */,
                                           const CUtensorMap *tmW,
                                           const HeadParams &p, const HeadSmem &sm, int rows,
                                           int splits, int ng, int first_unit, uint32_t tmem_base) {
@@ -660,7 +666,6 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
     TileWalk tw;
     tw.init(rows, ng, p.V, p.d, splits);
     const int num_kb = (p.d + kTileK - 1) / kTileK;
-    int taken = 0;
 
     if (warp == 0) {
         if (lane == 0 && !p.stall) {
@@ -672,7 +677,7 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
             tma_prefetch_desc(umap);
             const Copies copies{tmW, umap, stages, stage_bytes, 0, kSwapStageBytesA, ng,
                                 static_cast<int>(rank) * half};
-            taken = produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
+            produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
         }
     } else if (warp == 1) {
         if (rank == 0) {
@@ -741,7 +746,9 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
         for (int i = etid; i < 4 * ng; i += kEpiThreads) stats[i] = kEmpty;
         uint32_t epi_phase = 0;
         uint32_t tile_iter = 0;
-        bool ok = epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns) && wait_for_rows(p, sm, rows);
+        bool ok = epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns) &&
+                  // the other CTAs' inv_rms, long before this warp's first tile is done
+                  wait_for_rows(p, sm, rows, 500);
         UnitCursor uc;
         while (ok) {
             if (!mbar_wait_bounded_cluster(&unit_full[uc.slot], uc.phase, abort_flag, p.wait_limit_ns))
@@ -843,64 +850,83 @@ __device__ __forceinline__ int head_swap(const CUtensorMap *tmUrows /* [kUMaps] 
                 if (r < rows && rpd_check(2 * g + static_cast<int>(rank) < p.max_splits, p.meta + kMetaStatus))
                     p.partials[static_cast<size_t>(r) * p.max_splits + 2 * g + static_cast<int>(rank)] = acc4;
             }
+            __syncwarp();
+            if (lane == 0) counter_add_release(&p.meta[kMetaUnitsDone], 1);
             if (!epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns)) break;
         }
     }
-    return taken;
 }
 
-// After the contraction: this CTA's `taken` work units are counted, blocks of rows are claimed and
-// merged once every unit of the pass is, and the CTA that completes the merge scores the canvas.
-// Only running CTAs hold units, so the wait ends whatever part of the grid is resident.  It also
-// ends when another CTA has given up (the step's outputs are then meaningless) and, for a CTA
-// that came so late that the canvas was already being scored (`stale`), it is not begun.
+// After the contraction: CTAs claim blocks of rows and merge them once every work unit of the
+// pass is done, and the CTA that completes the merge scores the canvas.
+
+// A CTA's first claim of a block of rows and the wait for the units (the producer's thread, which
+// is done before the epilogue is); `blocks` if there is nothing to merge.  Only running CTAs hold
+// units, so the wait ends whatever part of the grid is resident.  It also ends when a CTA has
+// given up (the step's outputs are then meaningless), and after the time in which a unit's own
+// waits would have run out.  A CTA that came so late that the canvas was already being scored
+// claims nothing.
+__device__ __forceinline__ int claim_merge(const HeadParams &p, const HeadSmem &sm, const PassInfo &pass,
+                                           int blocks) {
+    int32_t *meta = p.meta;
+    if (blocks == 0 || *sm.stale) return blocks;
+    const int block = atomicAdd(&meta[kMetaMergeNext], 1);
+    if (block >= blocks) return blocks;
+    const bool pair = pass.mode == kHeadModePair;
+    const int splits = pair ? pass.splits : pass.splits / 2;
+    const int tile_rows = pair ? kPairTileM : pass.swap_rows;
+    const int units = (pass.rows + tile_rows - 1) / tile_rows * splits;
+    const int target = 2 * units * (pair ? kPairEpiWarps : kSwapEpiWarps);
+    const uint64_t limit = p.wait_limit_ns * (p.V / kTileN / splits + 2);
+    uint64_t t0 = globaltimer_ns();
+    int seen = 0;
+    while (true) {
+        const int done = ld_acquire(&meta[kMetaUnitsDone]);
+        if (done >= target || *sm.abort_flag || ld_acquire(&meta[kMetaStatus]) != RPD_OK) break;
+        const uint64_t now = globaltimer_ns();
+        if (done != seen) t0 = now;
+        seen = done;
+        if (now - t0 > limit) {
+            *sm.abort_flag = 1;
+            break;
+        }
+    }
+    return block;
+}
+
 __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem &sm,
-                                            const PassInfo &pass, int taken, bool stale) {
+                                            const PassInfo &pass) {
     int32_t *meta = p.meta;
     volatile int *share = reinterpret_cast<volatile int *>(sm.ring + kHeadRegionBytes - 16);
     const int gs = merge_lanes(pass.splits);
     const int per_block = kHeadKernelThreads / gs;
     const int blocks = (pass.rows + per_block - 1) / per_block;
+    const int first = threadIdx.x == 0 ? claim_merge(p, sm, pass, blocks) : 0;
+    __syncthreads();  // the ring is free: every role of this CTA is done
     if (threadIdx.x == 0) {
-        int block = blocks;
-        if (taken > 0) counter_add_release(&meta[kMetaUnitsDone], taken);
-        if (blocks > 0 && !stale) {
-            block = atomicAdd(&meta[kMetaMergeNext], 1);
-            const int units = pass.mode == kHeadModePair
-                                  ? (pass.rows + kPairTileM - 1) / kPairTileM * pass.splits
-                                  : (pass.rows + pass.swap_rows - 1) / pass.swap_rows * (pass.splits / 2);
-            const uint64_t t0 = globaltimer_ns();
-            while (block < blocks && ld_acquire(&meta[kMetaUnitsDone]) < 2 * units) {
-                if (ld_acquire(&meta[kMetaStatus]) != RPD_OK) break;
-                if (globaltimer_ns() - t0 > 2 * p.wait_limit_ns) {
-                    atomicExch(&meta[kMetaStatus], RPD_ERR_TIMEOUT);
-                    break;
-                }
-            }
-        }
-        share[0] = block;
+        if (*sm.abort_flag) atomicExch(&meta[kMetaStatus], RPD_ERR_TIMEOUT);
+        share[0] = first;
         // nothing to merge: the first CTA scores
-        share[1] = blocks == 0 && blockIdx.x == 0 && !stale;
+        share[1] = blocks == 0 && blockIdx.x == 0 && !*sm.stale;
     }
     __syncthreads();
     const int num_words = p.from_mask ? (p.compact.B * p.compact.N + 31) >> 5 : 0;
     for (int block = share[0]; block < blocks; block = share[0]) {
+        int next = 0;
+        if (threadIdx.x == 0) next = atomicAdd(&meta[kMetaMergeNext], 1);  // while this block is merged
         merge_block(p.merge, pass, p.norm.sel_list, block, gs, meta + kMetaStatus,
                     [&](int q) { return sm.map.position(q, num_words); });
-        __threadfence();  // this CTA's merged rows are visible before they are counted
         __syncthreads();
         if (threadIdx.x == 0) {
-            share[1] = atomicAdd(&meta[kMetaMergeDone], 1) == blocks - 1;
-            share[0] = atomicAdd(&meta[kMetaMergeNext], 1);
-            __threadfence();
+            share[1] = counter_add_acq_rel(&meta[kMetaMergeDone], 1) == blocks - 1;
+            share[0] = next;
         }
         __syncthreads();
     }
     if (!p.score_canvas || !share[1]) return;
     int status = RPD_OK, rows_total = pass.rows;
     if (threadIdx.x == 0) {
-        atomicExch(&meta[kMetaClosed], 1);
-        __threadfence();  // before any mask byte changes
+        *reinterpret_cast<volatile int32_t *>(&meta[kMetaClosed]) = 1;  // before any mask byte changes
         status = ld_acquire(&meta[kMetaStatus]);
         if (!p.from_mask) rows_total = meta[kMetaRowsTotal];
     }
@@ -938,20 +964,20 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     const uint32_t tmem_base = *sm.tmem_slot;
     pdl_wait();  // mask, hidden states and meta words come from preceding work of the stream
 
-    // The first claims need nothing of the pass, and return while it is worked out.
+    // The first claims need nothing of the pass, and return while it is worked out.  (Claiming and
+    // loading the mask before the set-up above is slower: its fences wait for both.)
     int first_unit = -1, first_row = 0;
     if (threadIdx.x == 0 && rank == 0) first_unit = atomicAdd(&p.meta[kMetaUnitNext], 1);
     if (warp >= 2 && lane == 0) first_row = atomicAdd(&p.meta[kMetaRowNext], 1);
 
     PassInfo pass;
     int num_words = 0;
-    bool stale = false;
     if (p.from_mask) {
         const int masked = compact_mask(p.compact, sm.map, reinterpret_cast<int *>(sm.ring));
         num_words = (p.compact.B * p.compact.N + 31) >> 5;
-        if (threadIdx.x == 0 && p.score_canvas) {  // read after the mask
+        if (threadIdx.x == 32 && p.score_canvas) {  // read after the mask
             __threadfence();
-            stale = ld_acquire(&p.meta[kMetaClosed]) != 0;
+            *sm.stale = ld_acquire(&p.meta[kMetaClosed]);
         }
         int lazy = 0;
         if (p.compact.lazy) {  // which rows there are may depend on the plan
@@ -1004,26 +1030,22 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         }
     }
 
-    int taken = 0;
     if (pass.rows > 0) {
         if (pass.mode == kHeadModePair)
-            taken = head_pair(&maps.u, &maps.w128, p, sm, pass.rows, pass.splits, first_unit, tmem_base);
+            head_pair(&maps.u, &maps.w128, p, sm, pass.rows, pass.splits, first_unit, tmem_base);
         else if (pass.mode == kHeadModeRowsN)
-            taken = head_swap(maps.u_rows, &maps.w128, p, sm, pass.rows, pass.splits / 2,
-                              pass.swap_rows, first_unit, tmem_base);
+            head_swap(maps.u_rows, &maps.w128, p, sm, pass.rows, pass.splits / 2, pass.swap_rows,
+                      first_unit, tmem_base);
     }
-
     __syncwarp();
     tc_fence_before_sync();
-    __syncthreads();
+    finish_pass(p, sm, pass);  // begins with a barrier of the CTA
     cluster_sync();  // no signal may still be in flight to a CTA that is about to exit
     tc_fence_after_sync();
-    if (*sm.abort_flag && threadIdx.x == 0) atomicExch(&p.meta[kMetaStatus], RPD_ERR_TIMEOUT);
     if (warp == 1) {
         __syncwarp();
         tmem_dealloc_pair(tmem_base, kTmemCols);
     }
-    finish_pass(p, sm, pass, taken, stale);
     // The last CTA of the grid leaves the counters at zero for the next pass.
     if (threadIdx.x == 0) {
         __threadfence();

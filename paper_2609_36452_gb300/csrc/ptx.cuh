@@ -184,6 +184,14 @@ __device__ __forceinline__ void counter_add_release(int *p, int n) {
     asm volatile("red.release.gpu.global.add.s32 [%0], %1;" ::"l"(p), "r"(n) : "memory");
 }
 
+// Adds n and returns the count before: the caller's stores (and those it has synchronised with) come
+// before it, what it reads afterwards comes after every earlier caller's.
+__device__ __forceinline__ int counter_add_acq_rel(int *p, int n) {
+    int old;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(n) : "memory");
+    return old;
+}
+
 __device__ __forceinline__ void proxy_fence() { asm volatile("fence.proxy.async;" ::: "memory"); }
 
 // Bounded and abort aware like the mbarrier waits; `sleep_ns` between polls.

@@ -45,6 +45,7 @@ constexpr int kSwapRowBytes = 4 * 16 + 4;
 constexpr int kUBoxRows = 16;  // granularity of a half group's rows (the TMA box heights)
 // Roles: warp 0 TMA, warp 1 MMA + TMEM owner, warps 2-9 epilogue (pair tiles use warps 2-5).
 constexpr int kHeadKernelThreads = 64 + 32 * kSwapEpiWarps;
+constexpr int kPairEpiWarps = 4;
 constexpr int kHeadBarrierBytes = 448;
 // Canvas positions (B * N) whose masks the head kernel compacts itself, as a bitmap in its shared
 // memory: any single canvas, and batches of up to this many positions together.
@@ -94,7 +95,7 @@ enum MetaIndex : int {
     kMetaClosed = 16,    // the canvas is being scored: the mask no longer describes the pass
     // counts that the head kernel's CTAs wait for, on a line of their own
     kMetaRowsDone = 32,  // gathered rows of the pass
-    kMetaUnitsDone = 33, // head work units whose partials are written, counted by both CTAs of a pair
+    kMetaUnitsDone = 33, // head work units whose partials are written, counted by each epilogue warp
     kMetaWords = 64
 };
 

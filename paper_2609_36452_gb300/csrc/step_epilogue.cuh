@@ -212,7 +212,6 @@ __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float 
         // Scored positions: every masked one, or (RPD-block) the active block's masked ones,
         // which are exactly those the compaction kept.
         const int q = compact_index(i, is_masked);
-        n_masked_all += is_masked;
         int y = -1, ki = 0;
         bool cand = false, high = false;
         float conf = 0.f, H = 0.f, r = 0.f, s = 0.f;
@@ -281,6 +280,7 @@ __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float 
                 if (p.dbg.layer_pmax) p.dbg.layer_pmax[o] = 0.f;
             }
         }
+        n_masked_all += is_masked;  // (after the loads that do not need it)
         sm.conf[i] = conf;
         sm.H[i] = H;
         sm.y[i] = y;
@@ -335,6 +335,7 @@ __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float 
         cnt.x += (f & kFlagCandidate) != 0;
         cnt.y += (f & (kFlagCandidate | kFlagHigh)) == (kFlagCandidate | kFlagHigh);
     }
+    if (threadIdx.x == 0) __threadfence();  // what the caller has stored comes before the commits
     const int4 tot = block_sum4(cnt, sm.sum);
     const int fallback_window = p.block > 0 ? p.block : p.window;
 

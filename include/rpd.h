@@ -330,7 +330,7 @@ int rpd_kernel_times(rpd_ctx *ctx, double *ms /*[RPD_NUM_KERNELS]*/,
  * Limits: K*N <= 1024, N <= 1024, d <= 4096 (plus rpd_create's shape rules); larger sizes
  * return RPD_ERR_UNSUPPORTED with a message naming the limit, before any work is enqueued.
  * All calls on a device share the one scratch array, which keeps the previous call's
- * contents (the step's count/status words are cleared at the start of every call): calls
+ * contents (the step's count/status words are zero again at the end of every call): calls
  * whose GPU work overlaps - concurrent host threads or different streams - race on it, so
  * order them on one stream.  The first call on each device finds the array's device address
  * (cudaGetSymbolAddress) and caches it; make that first call before any stream capture. */

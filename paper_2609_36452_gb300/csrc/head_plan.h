@@ -111,6 +111,17 @@ __host__ __device__ inline HeadPlan plan_head(long long rows, const HeadPlanInpu
     return plan_from_keys(in, key2, key3, ng);
 }
 
+// The kernel argument with the plans of every pass of up to kStepPlanRows rows; `plan(rows)`.
+template <typename Plan>
+inline void fill_step_plan(StepPlan &p, Plan plan) {
+    for (int i = 0; i < kStepPlanRows / 32; ++i) {
+        const HeadPlan hp = plan(32 * (i + 1));
+        p.splits[i] = hp.mode == kHeadModeRowsN ? -hp.splits : hp.splits;
+        p.swap_rows[i] = static_cast<uint16_t>(hp.swap_rows);
+        p.est[i] = hp.est;
+    }
+}
+
 #ifdef __CUDACC__
 // Device evaluation by one full warp (lanes share the split search); valid in every lane.
 __device__ inline HeadPlan plan_head_warp(long long rows, const HeadPlanInputs &in) {
@@ -134,6 +145,13 @@ __device__ inline HeadPlan plan_head_warp(long long rows, const HeadPlanInputs &
         key3 = b < key3 ? b : key3;
     }
     return plan_from_keys(in, key2, gmax3 > 0 ? key3 : ~0ull, ng);
+}
+
+// A pass's plan from a step's kernel argument (0 <= rows <= kStepPlanRows).
+__device__ inline HeadPlan step_plan(const StepPlan &p, long long rows) {
+    if (rows <= 0) return HeadPlan{kHeadModePair, 1, 0, 0.f};
+    const int i = static_cast<int>(rows - 1) / 32;
+    return HeadPlan{p.splits[i] < 0 ? kHeadModeRowsN : kHeadModePair, abs(p.splits[i]), p.swap_rows[i], p.est[i]};
 }
 
 // The plan of a pass: the context's table when it covers `rows`, else one warp evaluates it.

@@ -982,7 +982,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         int lazy = 0;
         if (p.compact.lazy) {  // which rows there are may depend on the plan
             if (warp == 0) {
-                lazy = choose_lazy(p.compact, masked);
+                lazy = choose_lazy(p.compact, p.plan, masked);
                 if (lane == 0) sm.map.pass->lazy = lazy;
             }
             __syncthreads();
@@ -994,7 +994,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         pass.layer0 = lazy ? p.compact.K - 1 : 0;
         pass.rows = lazy ? masked : p.compact.K * masked;
         if (warp == 0) {
-            const HeadPlan hp = lookup_plan(pass.rows, p.compact.plan, p.compact.plan_rows, p.compact.plan_in);
+            const HeadPlan hp = pass_plan(p.compact, p.plan, pass.rows);
             pass.mode = hp.mode;
             pass.splits = hp.splits;
             pass.swap_rows = hp.swap_rows;

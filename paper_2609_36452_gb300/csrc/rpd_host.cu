@@ -118,6 +118,7 @@ struct rpd_ctx {
     int32_t *q_of_pos = nullptr, *pos_of_q = nullptr, *canvas_off = nullptr, *meta = nullptr;
     HeadPlan *plan = nullptr;  // head-tiling plans by pass row count, rows 0..plan_rows
     int plan_rows = 0;
+    StepPlan step_plan{};      // the same for few rows, passed to the head kernel
     int32_t *sel_q = nullptr;  // lazy projection: compact indices of the band positions
     int32_t *band_off = nullptr;  // lazy projection: [B+1] each canvas's first band entry
     int v_offset = 0, V_total = 0;  // vocabulary shard: rows of the head are entries
@@ -186,10 +187,11 @@ int build_plan(rpd_ctx *c) {
     const HeadPlanInputs in = plan_inputs(c);
     const int gmax2 = std::min(in.num_n, in.max_splits);
     const int gmax3 = std::min(in.num_n, in.max_splits / 2);
-    std::vector<HeadPlan> table(static_cast<size_t>(n) + 1);
-    std::vector<unsigned long long> key2((n + kPairTileM - 1) / kPairTileM + 1, 0ull);
+    const int m = std::max(n, kStepPlanRows);
+    std::vector<HeadPlan> table(static_cast<size_t>(m) + 1);
+    std::vector<unsigned long long> key2((m + kPairTileM - 1) / kPairTileM + 1, 0ull);
     std::vector<std::vector<unsigned long long>> key3;  // [groups][ng / step]
-    for (int r = 0; r <= n; ++r) {
+    for (int r = 0; r <= m; ++r) {
         if (r == 0 || in.pair_slots <= 0) {
             table[r] = plan_head(r, in);
             continue;
@@ -209,7 +211,9 @@ int build_plan(rpd_ctx *c) {
         }
         table[r] = plan_from_keys(in, key2[tiles2], k3, ng);
     }
-    cudaError_t e = cudaMemcpy(c->plan, table.data(), table.size() * sizeof(HeadPlan), cudaMemcpyHostToDevice);
+    fill_step_plan(c->step_plan, [&](int r) { return table[r]; });
+    cudaError_t e = cudaMemcpy(c->plan, table.data(), (static_cast<size_t>(n) + 1) * sizeof(HeadPlan),
+                               cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(plan table)");
     c->plan_rows = n;
     return RPD_OK;
@@ -372,6 +376,7 @@ HeadParams head_params(const rpd_ctx *c, const CompactParams &cp, const void *hi
                        const int32_t *sel_list, bool from_mask, bool last_pass, const MergeArgs &mg) {
     HeadParams hp{};
     hp.compact = cp;
+    hp.plan = c->step_plan;
     hp.norm = NormParams{static_cast<const __nv_bfloat16 *>(hidden),
                          static_cast<const __nv_bfloat16 *>(c->g), c->pos_of_q, sel_list, c->meta,
                          c->u, c->inv_rms, cp.B * cp.N, c->d, c->eps};

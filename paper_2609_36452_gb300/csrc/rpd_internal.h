@@ -123,6 +123,17 @@ struct HeadPlanInputs {
 // Rows up to which a context tabulates the plan (larger passes evaluate it on the device).
 constexpr int kPlanRows = 16384;
 
+// The plans of passes of up to kStepPlanRows rows as a kernel argument: a plan depends on the row
+// count only through its multiple of 32 (groups are padded to 32 rows, pair tiles to 256).  Reading
+// a table in global memory, or evaluating the plan on the device (9 us), lay between a step's
+// compaction and its first copies.
+constexpr int kStepPlanRows = 1024;
+struct StepPlan {
+    int32_t splits[kStepPlanRows / 32];  // negative: rows on N
+    uint16_t swap_rows[kStepPlanRows / 32];
+    float est[kStepPlanRows / 32];
+};
+
 struct CompactParams {
     const uint8_t *mask;  // [B*N]
     int32_t *q_of_pos;    // [B*N] compact index or -1
@@ -258,6 +269,7 @@ struct BatchScoreParams {
 
 struct HeadParams {
     CompactParams compact; // the mask and what its compaction writes
+    StepPlan plan;         // of the passes that the kernel compacts itself
     NormParams norm;       // the rows gathered before the contraction
     float4 *partials;      // [rows][max_splits]: (max, sum, tsum, argmax bits), log2 units
     int32_t *meta;

@@ -16,7 +16,7 @@
 //   every GPU that loads this library until the process exits.
 //
 // Sharing: every call on a device uses the same arena and leaves its contents behind.
-// The step's status/count words are cleared at the start of each call, and every array the
+// The step's status/count words are zero again at the end of each call, and every array the
 // step reads is rewritten by the same call before it is read, with one exception: the last
 // head tile also reads the rows of the compact head operand past the call's live row count
 // (left over from an earlier call, or zero), and its epilogue discards what those rows
@@ -36,6 +36,7 @@
 #include <mutex>
 #include <string>
 
+#include "head_plan.h"
 #include "rpd_internal.h"
 
 using namespace rpd;
@@ -46,6 +47,7 @@ constexpr int kNaMaxRows = 1024;
 constexpr int kNaMaxD = 4096;
 constexpr int kNaMaxN = 1024;
 constexpr int kNaMaxSplits = 320;
+static_assert(kNaMaxRows <= kStepPlanRows, "every plan fits the kernel argument");
 static_assert(kNaMaxN <= kFusedMaxPositions, "the head kernel compacts the mask");
 constexpr int kNaMaxDevices = 64;
 
@@ -66,12 +68,21 @@ constexpr size_t kArenaBytes = kOffMeta + 256;
 
 static __device__ __align__(256) uint8_t g_noalloc_arena[kArenaBytes];
 
+// A head shape's plans: a few hundred thousand operations to make, so the last few are kept.
+struct ShapePlan {
+    int V = 0, d = 0;
+    StepPlan plan{};
+};
+constexpr int kShapePlans = 4;
+
 struct DeviceSetup {
     bool ready = false;
     int device = 0;
     uint8_t *arena = nullptr;  // device address of g_noalloc_arena on this device
     int num_sms = 0;
     int head_grid = 0;         // CTAs of the head kernel (same choice as rpd_step)
+    ShapePlan plans[kShapePlans];
+    int next_plan = 0;
 };
 
 std::mutex g_setup_mutex;
@@ -139,6 +150,19 @@ int setup_device(DeviceSetup **out) {
     }
     *out = &s;
     return RPD_OK;
+}
+
+// The plans of a head shape (any host thread).
+StepPlan step_plan_for(DeviceSetup &dev, const HeadPlanInputs &in, int V, int d) {
+    std::lock_guard<std::mutex> lock(g_setup_mutex);
+    for (const ShapePlan &s : dev.plans)
+        if (s.V == V && s.d == d) return s.plan;
+    ShapePlan &s = dev.plans[dev.next_plan];
+    dev.next_plan = (dev.next_plan + 1) % kShapePlans;
+    fill_step_plan(s.plan, [&](int rows) { return plan_head(rows, in); });
+    s.V = V;
+    s.d = d;
+    return s.plan;
 }
 
 }  // namespace
@@ -212,16 +236,16 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
     int splits = 2 * num_n < 2 * dev->num_sms ? 2 * num_n : 2 * dev->num_sms;
     if (splits > kNaMaxSplits) splits = kNaMaxSplits;
 
-    // The per-step count/status words must start from zero on every call.
-    cudaError_t e = cudaMemsetAsync(meta, 0, kMetaWords * 4, stream);
-    if (e == cudaSuccess) {
-        // no plan table (it would have to be allocated): the head kernel evaluates the
-        // head-tiling plan itself
+    // (the count and status words are zero: every call leaves them so)
+    cudaError_t e;
+    {
+        // the plans of all row counts fit the kernel argument: no table (it would have to be allocated)
         const HeadPlanInputs plan_in{num_n, splits, pair_slots,
                                      head_stream_in_tiles(V, d, dev->num_sms), RPD_TILING_AUTO};
         HeadParams hp{};
         hp.compact = CompactParams{mask, q_of_pos, pos_of_q, canvas_off, meta, 1, N, K, plan_in,
                                    nullptr, 0, rule.block, 0};
+        hp.plan = step_plan_for(*dev, plan_in, V, d);
         hp.norm = NormParams{static_cast<const __nv_bfloat16 *>(hidden),
                              static_cast<const __nv_bfloat16 *>(g_norm), pos_of_q, nullptr, meta, u,
                              inv_rms, N, d, eps};

@@ -1,0 +1,61 @@
+"""The plans that a step passes to the head kernel (StepPlan, one entry per 32 rows) are those of
+every row count up to its limit, at the two models' heads, small and ragged ones (no GPU)."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2609_36452_gb300", "csrc")
+
+DRIVER = r"""
+#include "head_plan.h"
+#include <cstdio>
+#include <cstdlib>
+int main(int argc, char **argv) {
+    const int V = atoi(argv[1]), d = atoi(argv[2]), sms = atoi(argv[3]), force = atoi(argv[4]);
+    rpd::HeadPlanInputs in{};
+    in.num_n = (V + 255) / 256;
+    in.max_splits = 2 * in.num_n < 2 * sms ? 2 * in.num_n : 2 * sms;
+    in.pair_slots = sms / 2;
+    in.hbm_tiles = rpd::head_stream_in_tiles(V, d, sms);
+    in.force = force;
+    rpd::StepPlan sp;
+    rpd::fill_step_plan(sp, [&](int r) { return rpd::plan_head(r, in); });
+    int bad = 0;
+    for (int r = 1; r <= rpd::kStepPlanRows; ++r) {
+        const rpd::HeadPlan a = rpd::plan_head(r, in);
+        const int i = (r - 1) / 32;
+        const int splits = sp.splits[i] < 0 ? -sp.splits[i] : sp.splits[i];
+        const int mode = sp.splits[i] < 0 ? rpd::kHeadModeRowsN : rpd::kHeadModePair;
+        bad += a.mode != mode || a.splits != splits || a.swap_rows != sp.swap_rows[i] || a.est != sp.est[i];
+    }
+    std::printf("%d\n", bad);
+    return 0;
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def driver(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    inc = "/usr/local/cuda/include"
+    if not cxx or not os.path.exists(os.path.join(inc, "cuda_runtime.h")):
+        pytest.skip("needs a host C++ compiler and the CUDA headers")
+    d = tmp_path_factory.mktemp("step_plan")
+    src, exe = d / "plan.cpp", d / "plan"
+    src.write_text(DRIVER)
+    r = subprocess.run([cxx, "-std=c++17", "-O1", "-I", inc, "-I", CSRC, "-I",
+                        os.path.join(ROOT, "include"), str(src), "-o", str(exe)],
+                       capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr
+    return str(exe)
+
+
+@pytest.mark.parametrize("force", [0, 1, 2])
+@pytest.mark.parametrize("V,d,sms", [(126464, 4096, 152), (152064, 3584, 152), (256, 64, 152),
+                                     (4100, 256, 152), (15872, 4096, 148), (50257, 768, 2)])
+def test_one_entry_per_32_rows_is_exact(driver, V, d, sms, force):
+    out = subprocess.run([driver, str(V), str(d), str(sms), str(force)], capture_output=True, text=True, check=True)
+    assert int(out.stdout) == 0

@@ -130,8 +130,8 @@ struct rpd_ctx {
     HeadMaps maps{};     // u (scratch) and W tensor maps of the head kernel
     int head_grid = 0;   // CTAs of the head kernel: 2 x resident clusters of two, <= SMs
 
-    // host-buffer entry point staging: device buffer, and a pinned host copy of its small
-    // part (mask, commit, tokens, stats) so that those move in one copy each way
+    // host-buffer entry point staging: a device copy of hidden states that are not page-locked,
+    // and a pinned buffer for mask, commits, tokens and statistics
     size_t stage_bytes = 0;
     uint8_t *stage = nullptr;
     size_t stage_host_bytes = 0;
@@ -879,23 +879,24 @@ int rpd_step_host(rpd_ctx *c, const void *hidden, uint8_t *mask, int N, float ta
             in_place = a.devicePointer;
         cudaGetLastError();  // clear the (non-sticky) error the query may have recorded
     }
+    // Mask, commits, tokens and statistics stay in a pinned buffer that the kernels read and write
+    // in place across the host link: a few hundred bytes, for which a copy each way cost 9 us of
+    // copy engine and hand-over between engines.
     const size_t hid = in_place ? 0 : static_cast<size_t>(c->K) * N * c->d * 2;
-    const size_t off_mask = (hid + 255) & ~size_t(255);
-    const size_t off_commit = off_mask + ((N + 255) & ~255);
-    const size_t off_token = off_commit + ((N + 255) & ~255);
+    const size_t off_commit = (static_cast<size_t>(N) + 255) & ~size_t(255);
+    const size_t off_token = 2 * off_commit;
     const size_t off_stats = off_token + ((static_cast<size_t>(N) * 4 + 255) & ~size_t(255));
-    const size_t need = off_stats + 256;
-    if (need > c->stage_bytes) {
+    const size_t small = off_stats + 256;
+    if (hid > c->stage_bytes) {
         cudaError_t e = cudaStreamSynchronize(c->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
         if (c->stage) cudaFree(c->stage);
         c->stage = nullptr;
         c->stage_bytes = 0;
-        e = cudaMalloc(&c->stage, need);
+        e = cudaMalloc(&c->stage, hid);
         if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(staging)");
-        c->stage_bytes = need;
+        c->stage_bytes = hid;
     }
-    const size_t small = need - off_mask;  // mask, commit, tokens, stats (with padding)
     if (small > c->stage_host_bytes) {
         if (c->stage_host) cudaFreeHost(c->stage_host);
         c->stage_host = nullptr;
@@ -904,29 +905,23 @@ int rpd_step_host(rpd_ctx *c, const void *hidden, uint8_t *mask, int N, float ta
         if (e != cudaSuccess) return cuda_fail(e, "cudaMallocHost(staging)");
         c->stage_host_bytes = small;
     }
-    const void *d_hidden = in_place ? in_place : c->stage;
-    uint8_t *d_mask = c->stage + off_mask;
-    uint8_t *d_commit = c->stage + off_commit;
-    int32_t *d_token = reinterpret_cast<int32_t *>(c->stage + off_token);
-    rpd_stats *d_stats = reinterpret_cast<rpd_stats *>(c->stage + off_stats);
-    uint8_t *h = c->stage_host;  // same layout as the device region from off_mask on
+    uint8_t *h = c->stage_host;
+    int32_t *token = reinterpret_cast<int32_t *>(h + off_token);
+    rpd_stats *stats = reinterpret_cast<rpd_stats *>(h + off_stats);
     // tokens are written only where committed: the step starts from the caller's canvas
     std::memcpy(h, mask, static_cast<size_t>(N));
-    std::memcpy(h + (off_token - off_mask), out_token, static_cast<size_t>(N) * 4);
+    std::memcpy(token, out_token, static_cast<size_t>(N) * 4);
     cudaError_t e = cudaSuccess;
     if (!in_place) e = cudaMemcpyAsync(c->stage, hidden, hid, cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(d_mask, h, off_stats - off_mask, cudaMemcpyHostToDevice, c->stream);
     if (e != cudaSuccess) return cuda_fail(e, "host->device copy");
-    int rc = run_step(c, d_hidden, d_mask, 1, N, &tau, &budget, d_commit, d_token, d_stats);
+    int rc = run_step(c, in_place ? in_place : c->stage, h, 1, N, &tau, &budget, h + off_commit, token, stats);
     if (rc) return rc;
-    e = cudaMemcpyAsync(h, d_mask, small, cudaMemcpyDeviceToHost, c->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "device->host copy");
+    e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
     std::memcpy(mask, h, static_cast<size_t>(N));
-    std::memcpy(out_commit, h + (off_commit - off_mask), static_cast<size_t>(N));
-    std::memcpy(out_token, h + (off_token - off_mask), static_cast<size_t>(N) * 4);
-    std::memcpy(out_stats, h + (off_stats - off_mask), sizeof(rpd_stats));
+    std::memcpy(out_commit, h + off_commit, static_cast<size_t>(N));
+    std::memcpy(out_token, token, static_cast<size_t>(N) * 4);
+    std::memcpy(out_stats, stats, sizeof(rpd_stats));
     return RPD_OK;
 }
 

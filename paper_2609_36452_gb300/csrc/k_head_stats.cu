@@ -858,7 +858,13 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
 }
 
 // After the contraction: CTAs claim blocks of rows and merge them once every work unit of the
-// pass is done, and the CTA that completes the merge scores the canvas.
+// pass is done, and the CTA that completes the merge scores the canvas, or selects what the second
+// of two passes projects.
+
+// Whether kernels after this one read of its compaction.
+__device__ __forceinline__ bool publishes(const HeadParams &p) {
+    return p.from_mask && (!p.score_canvas || p.select_band);
+}
 
 // A CTA's first claim of a block of rows and the wait for the units (the producer's thread, which
 // is done before the epilogue is); `blocks` if there is nothing to merge.  Only running CTAs hold
@@ -876,7 +882,8 @@ __device__ __forceinline__ int claim_merge(const HeadParams &p, const HeadSmem &
     const int splits = pair ? pass.splits : pass.splits / 2;
     const int tile_rows = pair ? kPairTileM : pass.swap_rows;
     const int units = (pass.rows + tile_rows - 1) / tile_rows * splits;
-    const int target = 2 * units * (pair ? kPairEpiWarps : kSwapEpiWarps);
+    // and the warp that publishes the pass
+    const int target = 2 * units * (pair ? kPairEpiWarps : kSwapEpiWarps) + (publishes(p) ? 1 : 0);
     const uint64_t limit = p.wait_limit_ns * (p.V / kTileN / splits + 2);
     uint64_t t0 = globaltimer_ns();
     int seen = 0;
@@ -906,8 +913,8 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
     if (threadIdx.x == 0) {
         if (*sm.abort_flag) atomicExch(&meta[kMetaStatus], RPD_ERR_TIMEOUT);
         share[0] = first;
-        // nothing to merge: the first CTA scores
-        share[1] = blocks == 0 && blockIdx.x == 0 && !*sm.stale;
+        // nothing to merge: the first CTA goes on
+        share[1] = blocks == 0 && blockIdx.x == 0 && !*sm.stale && !meta[kMetaScored];
     }
     __syncthreads();
     const int num_words = p.from_mask ? (p.compact.B * p.compact.N + 31) >> 5 : 0;
@@ -923,7 +930,35 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
         }
         __syncthreads();
     }
-    if (!p.score_canvas || !share[1]) return;
+    if (!share[1]) return;
+    if (p.select_band) {
+        // The positions whose earlier window layers a second pass projects (none if this one had
+        // every layer); without any the canvas can be scored now.
+        const int per_canvas = p.compact.N;
+        const int band = pass.lazy
+                             ? select_band(p.merge.row_pmax + static_cast<size_t>(p.compact.K - 1) * pass.masked,
+                                           pass.masked, p.score.theta_c, p.tau, p.sel_q,
+                                           reinterpret_cast<int *>(sm.ring), [&](int q) {
+                                               return p.compact.B == 1 ? 0 : sm.map.position(q, num_words) / per_canvas;
+                                           })
+                             : 0;
+        const int rows = (p.compact.K - 1) * band;
+        if (threadIdx.x < 32) {
+            const HeadPlan hp = pass_plan(p.compact, p.plan, rows);
+            if (threadIdx.x == 0) {
+                meta[kMetaRows] = rows;
+                meta[kMetaRowsTotal] = pass.rows + rows;
+                meta[kMetaSel] = band;
+                meta[kMetaLayer0] = 0;
+                meta[kMetaSwapRows] = hp.swap_rows;
+                meta[kMetaSplits] = hp.splits;
+                meta[kMetaHeadMode] = hp.mode;
+                meta[kMetaScored] = band == 0 && p.score_canvas;
+            }
+        }
+        if (band > 0) return;
+    }
+    if (!p.score_canvas) return;
     int status = RPD_OK, rows_total = pass.rows;
     if (threadIdx.x == 0) {
         *reinterpret_cast<volatile int32_t *>(&meta[kMetaClosed]) = 1;  // before any mask byte changes
@@ -975,7 +1010,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     if (p.from_mask) {
         const int masked = compact_mask(p.compact, sm.map, reinterpret_cast<int *>(sm.ring));
         num_words = (p.compact.B * p.compact.N + 31) >> 5;
-        if (threadIdx.x == 32 && p.score_canvas) {  // read after the mask
+        if (threadIdx.x == 32) {  // read after the mask
             __threadfence();
             *sm.stale = ld_acquire(&p.meta[kMetaClosed]);
         }
@@ -1025,8 +1060,12 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
             pass = *sm.map.pass;
             // for the kernels after this one, by the warp that gathered row 0 (or, without rows,
             // one of the first CTA)
-            if (!p.score_canvas && warp >= 2 && (pass.rows > 0 ? first_row == 0 : blockIdx.x == 0 && warp == 2))
+            if (publishes(p) && warp >= 2 &&
+                (pass.rows > 0 ? first_row == 0 : blockIdx.x == 0 && warp == 2)) {
                 publish_pass(p.compact, sm.map, lane);
+                __syncwarp();
+                if (lane == 0) counter_add_release(&p.meta[kMetaUnitsDone], 1);
+            }
         }
     }
 
@@ -1059,6 +1098,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
             p.meta[kMetaUnitsDone] = 0;
             p.meta[kMetaClosed] = 0;
             p.meta[kMetaExit] = 0;
+            if (p.last_pass) p.meta[kMetaScored] = 0;
             if (p.last_pass) p.meta[kMetaStepStatus] = atomicExch(&p.meta[kMetaStatus], RPD_OK);
         }
     }

@@ -1,9 +1,9 @@
 // k_merge_commit.cu - the step's small kernels: the lazy projection's band selection, the scoring
 // of several canvases, the merge of vocabulary shards and the decoding loop's stop test.
 //
-// k_band (one CTA; lazy projection only): selects the positions whose final confidence lies
-//   in their canvas's stability band theta_c <= c < tau (Eq. 5 reads S_i only there) and sets
-//   up the second pass over their earlier window layers.
+// k_band (one CTA; lazy projection of batches that the head kernel does not compact itself): selects
+//   the positions whose final confidence lies in their canvas's stability band theta_c <= c < tau
+//   (Eq. 5 reads S_i only there) and sets up the second pass over their earlier window layers.
 //
 // k_score_commit (one CTA per canvas): scores and commits several canvases (score_canvas in
 //   step_epilogue.cuh; a single canvas is scored by the head kernel itself).
@@ -40,7 +40,6 @@ __global__ void __launch_bounds__(kMergeThreads) k_merge_shards(ShardMergeParams
 }
 
 constexpr int kBandThreads = 1024;
-constexpr int kBandItems = 4;
 
 __global__ void __launch_bounds__(kBandThreads, 1) k_band(BandParams p) {
     __shared__ int warp_sum[32];
@@ -51,54 +50,10 @@ __global__ void __launch_bounds__(kBandThreads, 1) k_band(BandParams p) {
     const bool lazy_on = p.meta[kMetaLazy] != 0;  // else the first pass covered every layer
     // 1. band positions, in compact order (the first pass is merged)
     const float *final_p = p.mg.row_pmax + static_cast<size_t>(p.K - 1) * nmt;
-    int carry = 0;
-    for (int base = 0; lazy_on && base < nmt; base += kBandThreads * kBandItems) {
-        const int q0 = base + tid * kBandItems;
-        int f[kBandItems];
-        int cnt = 0;
-#pragma unroll
-        for (int j = 0; j < kBandItems; ++j) {
-            const int q = q0 + j;
-            f[j] = 0;
-            if (q < nmt && p.K > 1) {
-                const float c = final_p[q];
-                const int b = p.pos_of_q[q] / p.N;
-                f[j] = (c >= p.theta_c && c < p.tau[b]) ? 1 : 0;
-            }
-            cnt += f[j];
-        }
-        const int incl = warp_inclusive_scan(cnt, lane);
-        if (lane == 31) warp_sum[warp] = incl;
-        __syncthreads();
-        if (warp == 0) {
-            const int v = warp_sum[lane];
-            const int vi = warp_inclusive_scan(v, lane);
-            warp_sum[lane] = vi - v;
-        }
-        __syncthreads();
-        int excl = carry + warp_sum[warp] + incl - cnt;
-#pragma unroll
-        for (int j = 0; j < kBandItems; ++j) {
-            if (f[j]) p.sel_q[excl] = q0 + j;
-            excl += f[j];
-        }
-        __syncthreads();
-        if (tid == kBandThreads - 1) warp_sum[0] = excl;
-        __syncthreads();
-        carry = warp_sum[0];
-        __syncthreads();
-    }
-    // 2. each canvas's range in the band list (the list is sorted, canvases are contiguous)
-    for (int b = tid; b <= p.B; b += kBandThreads) {
-        const int key = p.canvas_off[b];
-        int lo = 0, hi = carry;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (p.sel_q[mid] < key) lo = mid + 1; else hi = mid;
-        }
-        p.band_off[b] = lo;
-    }
-    // 3. the second pass: the K-1 earlier window layers of the band positions
+    const int carry = lazy_on ? select_band(final_p, nmt, p.theta_c, p.tau, p.sel_q, warp_sum,
+                                            [&](int q) { return p.pos_of_q[q] / p.N; })
+                              : 0;
+    // 2. the second pass: the K-1 earlier window layers of the band positions
     const long long rows = static_cast<long long>(p.K - 1) * carry;
     if (warp == 0) {
         const HeadPlan hp = lookup_plan(rows, p.plan, p.plan_rows, p.plan_in);

@@ -4,7 +4,8 @@
 // Step = k_head (compaction, gather, contraction, merge and, for a single canvas, score and
 // commit), sized from device-resident counts (nothing is read back mid-step).  Several canvases
 // are scored by k_score_commit; batches of more than kFusedMaxPositions positions are compacted
-// by k_compact first; lazy projection runs k_band and a second k_head.  Scratch is owned by the context and sized for the largest B*N seen.
+// by k_compact first.  Lazy projection runs a second k_head, over positions that the first one
+// selects (k_band after k_compact).  Scratch is owned by the context and sized for the largest B*N seen.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -120,7 +121,6 @@ struct rpd_ctx {
     int plan_rows = 0;
     StepPlan step_plan{};      // the same for few rows, passed to the head kernel
     int32_t *sel_q = nullptr;  // lazy projection: compact indices of the band positions
-    int32_t *band_off = nullptr;  // lazy projection: [B+1] each canvas's first band entry
     int v_offset = 0, V_total = 0;  // vocabulary shard: rows of the head are entries
                                     // [v_offset, v_offset + V) of a V_total vocabulary
     int projection = RPD_PROJECT_ALL;
@@ -151,7 +151,7 @@ struct rpd_ctx {
 
     void free_scratch() {
         void *ptrs[] = {u, inv_rms, partials, row_arg, row_pmax, row_H, q_of_pos, pos_of_q,
-                        canvas_off, meta, sel_q, band_off, plan};
+                        canvas_off, meta, sel_q, plan};
         for (void *p : ptrs)
             if (p) cudaFree(p);
         u = nullptr;
@@ -159,7 +159,7 @@ struct rpd_ctx {
         partials = nullptr;
         row_arg = nullptr;
         row_pmax = row_H = nullptr;
-        q_of_pos = pos_of_q = canvas_off = meta = sel_q = band_off = nullptr;
+        q_of_pos = pos_of_q = canvas_off = meta = sel_q = nullptr;
         plan = nullptr;
         cap_bn = cap_b = cap_rows = plan_rows = 0;
     }
@@ -249,7 +249,6 @@ int ensure_scratch(rpd_ctx *c, int B, int N) {
         {reinterpret_cast<void **>(&c->pos_of_q), static_cast<size_t>(new_bn) * 4},
         {reinterpret_cast<void **>(&c->sel_q), static_cast<size_t>(new_bn) * 4},
         {reinterpret_cast<void **>(&c->canvas_off), static_cast<size_t>(new_b + 1) * 4},
-        {reinterpret_cast<void **>(&c->band_off), static_cast<size_t>(new_b + 1) * 4},
         {reinterpret_cast<void **>(&c->meta), kMetaWords * 4},
         {reinterpret_cast<void **>(&c->plan),
          (static_cast<size_t>(std::min<long long>(rows, kPlanRows)) + 1) * sizeof(HeadPlan)},
@@ -461,20 +460,21 @@ int run_step(rpd_ctx *c, const void *hidden, uint8_t *mask, int B, int N, const 
         // The kernel reads the tiling chosen on the device for this pass.
         HeadParams hp = head_params(c, cp, hidden, sel_list, from_mask && !sel_list, last, mg);
         hp.score = sp;
-        hp.score_canvas = last && fuse_score ? 1 : 0;
+        hp.score_canvas = fuse_score && (last || from_mask) ? 1 : 0;
+        hp.select_band = !last && from_mask ? 1 : 0;
+        hp.sel_q = c->sel_q;
+        if (hp.select_band) std::copy(tau, tau + B, hp.tau);
         return launch_head(c->maps, hp, c->head_grid, c->stream);
     };
     e = pass(nullptr, !lazy);
     if (e == cudaSuccess && lazy) {
-        {
+        if (!from_mask) {
             KernelTimer t(c, 2);
             BandParams bp{};
             bp.meta = c->meta;
             bp.mg = mg;
             bp.pos_of_q = c->pos_of_q;
-            bp.canvas_off = c->canvas_off;
             bp.sel_q = c->sel_q;
-            bp.band_off = c->band_off;
             bp.B = B;
             bp.N = N;
             bp.K = c->K;

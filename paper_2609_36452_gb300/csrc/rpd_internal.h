@@ -93,6 +93,7 @@ enum MetaIndex : int {
     kMetaExit = 14,      // CTAs of the head kernel that are done; the last one zeroes the counters
     kMetaStepStatus = 15,// the step's status, published when its last head kernel ends
     kMetaClosed = 16,    // the canvas is being scored: the mask no longer describes the pass
+    kMetaScored = 17,    // the first of two passes scored the canvas: nothing is left for the second
     // counts that the head kernel's CTAs wait for, on a line of their own
     kMetaRowsDone = 32,  // gathered rows of the pass
     kMetaUnitsDone = 33, // head work units whose partials are written, counted by each epilogue warp
@@ -188,9 +189,7 @@ struct BandParams {
     int32_t *meta;
     MergeArgs mg;              // merged first-pass statistics (final-layer confidences)
     const int32_t *pos_of_q;   // [NMT] flat position b*N+i of compact index q
-    const int32_t *canvas_off; // [B+1] first compact index of each canvas
     int32_t *sel_q;            // out: compact indices of the band positions
-    int32_t *band_off;         // out: [B+1] first band entry of each canvas
     int B, N, K;
     float theta_c;
     HeadPlanInputs plan_in;
@@ -276,7 +275,10 @@ struct HeadParams {
     int from_mask;         // the kernel compacts the mask itself (B * N <= kFusedMaxPositions);
                            // otherwise the pass is described by the meta words
     int last_pass;         // the step's last projection pass: publish its status
-    int score_canvas;      // score the (single) canvas after the merge
+    int score_canvas;      // score the (single) canvas once nothing is left to project
+    int select_band;       // the first of two passes: select the second's positions after the merge
+    int32_t *sel_q;        // out: their compact indices
+    float tau[kMaxBatch];  // upper end of each canvas's band (the lower one is score.theta_c)
     MergeArgs merge;
     ScoreParams score;
     int V, d, max_splits;

@@ -82,6 +82,42 @@ __device__ __forceinline__ void merge_block(const MergeArgs &mg, const PassInfo 
     }
 }
 
+// ------------------------------------------------------------------------------ band
+
+// Lazy projection, after the final layer's pass: the compact indices of the positions whose
+// confidence lies in their canvas's stability band theta_c <= c < tau (Eq. 5 reads S_i only
+// there), in order; the whole CTA.  `final_p`: the final layer's probabilities by compact index;
+// `canvas(q)`: the canvas of compact index q; `warp_sum`: 32 ints of shared memory.  Returns how
+// many there are.
+template <typename Canvas>
+__device__ __forceinline__ int select_band(const float *final_p, int masked, float theta_c,
+                                           const float *tau, int32_t *sel_q, int *warp_sum, Canvas canvas) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nwarps = blockDim.x >> 5;
+    int carry = 0;
+#pragma unroll 1
+    for (int base = 0; base < masked; base += blockDim.x) {
+        const int q = base + threadIdx.x;
+        bool in = false;
+        if (q < masked) {
+            const float c = __ldcg(final_p + q);
+            in = c >= theta_c && c < tau[canvas(q)];
+        }
+        const unsigned ballot = __ballot_sync(0xffffffffu, in);
+        if (lane == 0) warp_sum[warp] = __popc(ballot);
+        __syncthreads();
+        int at = carry;
+#pragma unroll 1
+        for (int w = 0; w < nwarps; ++w) {
+            if (w < warp) at += warp_sum[w];
+            carry += warp_sum[w];
+        }
+        if (in) sel_q[at + __popc(ballot & ((1u << lane) - 1u))] = q;
+        __syncthreads();
+    }
+    return carry;
+}
+
 // ------------------------------------------------------------------------------ score
 
 struct ScanPair {

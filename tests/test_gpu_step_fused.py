@@ -79,3 +79,26 @@ def test_more_rows_than_the_grid_has_warps_and_splits_of_every_width():
             compare_step(ref, runner.step(hidden, mask, 0.9, 1.0))
         finally:
             runner.close()
+
+
+@pytest.mark.parametrize("tau,prefix", [(0.9, 0), (0.62, 0), (0.9, 96)])  # a band, a thin one, nothing masked
+@pytest.mark.parametrize("projection", ["lazy", "auto"])
+@pytest.mark.parametrize("N", [96, 700])
+def test_two_pass_steps_one_after_another(N, projection, tau, prefix):
+    """The first pass selects the second's positions, or scores the canvas itself when there are
+    none; the steps that follow on the same context find its counters as they should be."""
+    K, d, V = 6, 128, 2048
+    W, g, hidden = make(60 + N, K, N, d, V)
+    mask = torch.ones(N, dtype=torch.uint8)
+    if prefix:
+        mask[:] = 0
+    runner = DeviceRunner(W, g, K)
+    try:
+        for mode in (projection, "all", projection):
+            runner.ctx.set_projection(mode)
+            got = runner.step(hidden, mask, tau, 1.0)
+            ref = O.rpd_step(bits(hidden), mask.numpy(), bits(g), bits(W), 1e-6, tau, 1.0, "llada")
+            lazy = got["stats"]["n_rows"] < K * int(mask.sum())
+            compare_step(ref, got, lazy=lazy)
+    finally:
+        runner.close()

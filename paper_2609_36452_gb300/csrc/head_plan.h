@@ -2,11 +2,10 @@
 // projection pass of `rows` rows (host and device).  It changes no computed quantity, only
 // how the contraction is laid out on the GPU.
 //
-// A context evaluates it on the host for every row count up to kPlanRows when it sizes its
-// scratch and keeps the results in a device table, so that the step's compaction kernel - on
-// the critical path of every step - only looks its row count up.  Passes with more rows (and
-// the allocation-free entry point, which keeps no table) evaluate it on the device with one
-// warp.
+// It is evaluated on the host: for passes of up to kStepPlanRows rows into an argument of the head
+// kernel, for larger ones into a context's device table (every row count up to kPlanRows, then
+// every 256th).  On the device a search over the split counts cost 4 to 9 us of every step's
+// critical path.
 #pragma once
 
 #include <cstring>
@@ -95,7 +94,7 @@ __host__ __device__ inline HeadPlan plan_from_keys(const HeadPlanInputs &in, uns
     return rows_n ? HeadPlan{kHeadModeRowsN, 2 * g3, ng3, e3} : pair;
 }
 
-// Host evaluation (and the device's, in one thread).
+// The plan of a pass of `rows` rows.
 __host__ __device__ inline HeadPlan plan_head(long long rows, const HeadPlanInputs &in) {
     if (rows <= 0 || in.pair_slots <= 0) return HeadPlan{kHeadModePair, 1, 0, 0.f};
     const int tiles2 = static_cast<int>((rows + kPairTileM - 1) / kPairTileM);
@@ -123,30 +122,6 @@ inline void fill_step_plan(StepPlan &p, Plan plan) {
 }
 
 #ifdef __CUDACC__
-// Device evaluation by one full warp (lanes share the split search); valid in every lane.
-__device__ inline HeadPlan plan_head_warp(long long rows, const HeadPlanInputs &in) {
-    if (rows <= 0 || in.pair_slots <= 0) return HeadPlan{kHeadModePair, 1, 0, 0.f};
-    const int lane = threadIdx.x & 31;
-    const int tiles2 = static_cast<int>((rows + kPairTileM - 1) / kPairTileM);
-    const int gmax2 = in.num_n < in.max_splits ? in.num_n : in.max_splits;
-    unsigned long long key2 =
-        best_split_key(kPairTileCost, tiles2, in.pair_slots, in.num_n, gmax2, lane + 1, 32);
-    const int gmax3 = in.num_n < in.max_splits / 2 ? in.num_n : in.max_splits / 2;
-    const int groups = swap_groups(rows);
-    const int ng = swap_group_rows(rows, groups);
-    unsigned long long key3 =
-        gmax3 > 0 ? best_split_key(swap_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax3, lane + 1, 32)
-                  : ~0ull;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long a = __shfl_xor_sync(0xffffffffu, key2, o);
-        const unsigned long long b = __shfl_xor_sync(0xffffffffu, key3, o);
-        key2 = a < key2 ? a : key2;
-        key3 = b < key3 ? b : key3;
-    }
-    return plan_from_keys(in, key2, gmax3 > 0 ? key3 : ~0ull, ng);
-}
-
 // A pass's plan from a step's kernel argument (0 <= rows <= kStepPlanRows).
 __device__ inline HeadPlan step_plan(const StepPlan &p, long long rows) {
     if (rows <= 0) return HeadPlan{kHeadModePair, 1, 0, 0.f};
@@ -154,12 +129,13 @@ __device__ inline HeadPlan step_plan(const StepPlan &p, long long rows) {
     return HeadPlan{p.splits[i] < 0 ? kHeadModeRowsN : kHeadModePair, abs(p.splits[i]), p.swap_rows[i], p.est[i]};
 }
 
-// The plan of a pass: the context's table when it covers `rows`, else one warp evaluates it.
-// Called by the first warp of the CTA.
-__device__ inline HeadPlan lookup_plan(long long rows, const HeadPlan *table, int table_rows,
-                                       const HeadPlanInputs &in) {
-    if (table && rows <= table_rows) return table[rows];
-    return plan_head_warp(rows, in);
+// A pass's plan from a context's tables: one entry per row count up to table_rows, then one per
+// 256 rows (the plan of the most rows with that many pair tiles, its groups fitted to the rows).
+__device__ inline HeadPlan table_plan(long long rows, const HeadPlan *table, int table_rows) {
+    if (rows <= table_rows) return table[rows];
+    HeadPlan hp = table[table_rows + (rows + kPairTileM - 1) / kPairTileM - table_rows / kPairTileM];
+    if (hp.mode == kHeadModeRowsN) hp.swap_rows = swap_group_rows(rows, swap_groups(rows));
+    return hp;
 }
 #endif
 

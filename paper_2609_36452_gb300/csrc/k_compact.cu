@@ -91,13 +91,12 @@ __global__ void __maxnreg__(48) k_compact(CompactParams p) {
         int lz = (p.lazy == 1 && p.K > 1) ? 1 : 0;
         if (p.lazy == 2 && p.K > 1) {
             const long long guess = static_cast<long long>(kLazyBandGuess * (p.K - 1) * carry);
-            const float e_all = lookup_plan(all_rows, p.plan, p.plan_rows, p.plan_in).est;
-            const float e_fin = lookup_plan(carry, p.plan, p.plan_rows, p.plan_in).est;
-            const float e_band = lookup_plan(guess, p.plan, p.plan_rows, p.plan_in).est;
+            const float e_all = table_plan(all_rows, p.plan, p.plan_rows).est;
+            const float e_fin = table_plan(carry, p.plan, p.plan_rows).est;
+            const float e_band = table_plan(guess, p.plan, p.plan_rows).est;
             lz = (e_fin + e_band < e_all) ? 1 : 0;
         }
-        const HeadPlan hp = lookup_plan(lz ? static_cast<long long>(carry) : all_rows, p.plan,
-                                        p.plan_rows, p.plan_in);
+        const HeadPlan hp = table_plan(lz ? static_cast<long long>(carry) : all_rows, p.plan, p.plan_rows);
         if (lane == 0) {
             lazy_on = lz;
             plan = hp;

@@ -148,21 +148,6 @@ __device__ __forceinline__ void fold_chunk(float (&v)[32], float scale, int col0
     }
 }
 
-// Combine two partial statistics (same rule as the merge kernel's): m = max, alpha =
-// 2^(m_j - m), s = sum alpha s_j, t = sum alpha (t_j + (m_j - m) s_j), argmax the lowest index
-// attaining m.
-__device__ __forceinline__ float4 merge_stat(float4 x, float4 y) {
-    if (y.y <= 0.f) return x;
-    if (x.y <= 0.f) return y;
-    const float m = fmaxf(x.x, y.x);
-    const float dx = x.x - m, dy = y.x - m;
-    const float ax = exp2f(dx), ay = exp2f(dy);
-    const int a = (x.x > y.x) ? __float_as_int(x.w)
-                : (y.x > x.x) ? __float_as_int(y.w) : min(__float_as_int(x.w), __float_as_int(y.w));
-    return make_float4(m, ax * x.y + ay * y.y, ax * fmaf(dx, x.y, x.z) + ay * fmaf(dy, y.y, y.z),
-                       __int_as_float(a));
-}
-
 // Shared memory of the head kernel: the operand ring (and for rows on N the transpose blocks
 // and running statistics), then the barriers.
 struct HeadSmem {
@@ -275,6 +260,13 @@ __device__ __forceinline__ bool claim_unit(const HeadParams &p, const HeadSmem &
     }
     uc.advance();
     return true;
+}
+
+// Rows on N: a stage of 128 head rows and half a group's rows, and how many there are in the region
+// beside the transpose blocks and the rows' statistics and RMS factors.
+__device__ __forceinline__ int swap_stage_bytes(int ng) { return kSwapStageBytesA + (ng / 2) * kTileK * 2; }
+__device__ __forceinline__ int swap_stages(int ng) {
+    return min((kHeadRegionBytes - kSwapXposeBytes - ng * kSwapRowBytes) / swap_stage_bytes(ng), kSwapMaxStages);
 }
 
 // What one CTA's TMA producer copies: per stage 128 head rows x 64 columns (w_off bytes into the
@@ -409,9 +401,8 @@ __device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm,
 // 64 KB per stage); empty[s], acc_full[a] and drain receive multicast commits from the MMA
 // thread in both CTAs; acc_empty[a] lives in the even CTA and counts the 4 epilogue warps
 // of both CTAs (8 arrivals).
-__device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensorMap *tmW,
-                                          const HeadParams &p, const HeadSmem &sm, int rows,
-                                          int splits, int first_unit, uint32_t tmem_base) {
+__device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &sm, const TileWalk &tw,
+                                          int rows, int splits, int num_kb, uint32_t tmem_base) {
     constexpr int kStageBytes = kPairStageBytesA + kPairStageBytesB;
     uint64_t *full = sm.full, *empty = sm.empty, *acc_full = sm.acc_full,
              *acc_empty = sm.acc_empty, *unit_full = sm.unit_full, *unit_empty = sm.unit_empty;
@@ -421,18 +412,7 @@ __device__ __forceinline__ void head_pair(const CUtensorMap *tmU, const CUtensor
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();  // 0 = even CTA (issues the MMAs), 1 = odd
 
-    TileWalk tw;
-    tw.init(rows, kPairTileM, p.V, p.d, splits);
-    const int num_kb = (p.d + kTileK - 1) / kTileK;
-
-    if (warp == 0) {
-        if (lane == 0 && !p.stall) {
-            // ------------------------------------------------------- TMA producer (both CTAs)
-            const Copies copies{tmW, tmU, kPairStages, kStageBytes, kPairStageBytesA, 0, kPairTileM,
-                                static_cast<int>(rank) * kPairHalfRows};
-            produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
-        }
-    } else if (warp == 1) {
+    if (warp == 1) {
         if (rank == 0) {
             // -------------------------------------------- MMA issuer (even CTA only): the whole
             // warp runs the loop, one elected lane issues (every branch below is warp-uniform)
@@ -639,12 +619,9 @@ __device__ __forceinline__ SwapPlace swap_place(int ng, uint32_t odd_tile) {
     return s;
 }
 
-__device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps] */,
-                                          const CUtensorMap *tmW,
-                                          const HeadParams &p, const HeadSmem &sm, int rows,
-                                          int splits, int ng, int first_unit, uint32_t tmem_base) {
-    uint64_t *full = sm.full, *empty = sm.empty, *acc_full = sm.acc_full,
-             *acc_empty = sm.acc_empty, *unit_full = sm.unit_full, *unit_empty = sm.unit_empty,
+__device__ __forceinline__ void head_swap(const HeadParams &p, const HeadSmem &sm, const TileWalk &tw,
+                                          int rows, int splits, int num_kb, int ng, uint32_t tmem_base) {
+    uint64_t *acc_full = sm.acc_full, *acc_empty = sm.acc_empty, *unit_full = sm.unit_full, *unit_empty = sm.unit_empty,
              *chunk_free = sm.chunk_free;
     volatile int *abort_flag = sm.abort_flag;
     volatile int *unit_ring = sm.unit_ring;
@@ -652,34 +629,14 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
     const uint32_t nch = static_cast<uint32_t>(ng / 32);
-    const int stage_b = (ng / 2) * kTileK * 2;
-    const int stage_bytes = kSwapStageBytesA + stage_b;
-    // region: operand ring (as many stages as fit), transpose blocks, statistics [4][ng], RMS
-    // factors [ng]
-    int stages = (kHeadRegionBytes - kSwapXposeBytes - ng * kSwapRowBytes) / stage_bytes;
-    stages = stages < kSwapMaxStages ? stages : kSwapMaxStages;
+    const int stage_bytes = swap_stage_bytes(ng);
+    const int stages = swap_stages(ng);
     float *xpose = reinterpret_cast<float *>(sm.ring + stages * stage_bytes);
     float4 *stats = reinterpret_cast<float4 *>(sm.ring + stages * stage_bytes + kSwapXposeBytes);
     float *scales = reinterpret_cast<float *>(stats + 4 * ng);
     constexpr int kEpiThreads = 32 * kSwapEpiWarps;
 
-    TileWalk tw;
-    tw.init(rows, ng, p.V, p.d, splits);
-    const int num_kb = (p.d + kTileK - 1) / kTileK;
-
-    if (warp == 0) {
-        if (lane == 0 && !p.stall) {
-            // ------------------------------------------------------- TMA producer (both CTAs)
-            // this CTA's half of the group's rows, one copy: the map whose box is that many rows
-            // high (rows [rank * half, +half) of the group; see the epilogue's row order)
-            const int half = ng / 2;
-            const CUtensorMap *umap = &tmUrows[half / kUBoxRows - 1];
-            tma_prefetch_desc(umap);
-            const Copies copies{tmW, umap, stages, stage_bytes, 0, kSwapStageBytesA, ng,
-                                static_cast<int>(rank) * half};
-            produce(p, sm, copies, rank, tw, rows, num_kb, first_unit);
-        }
-    } else if (warp == 1) {
+    if (warp == 1) {
         if (rank == 0) {
             // -------------------------------------------- MMA issuer (even CTA only): the whole
             // warp runs the loop, one elected lane issues (every branch below is warp-uniform)
@@ -839,16 +796,16 @@ __device__ __forceinline__ void head_swap(const CUtensorMap *tmUrows /* [kUMaps]
             for (int rl = etid; rl < ng; rl += kEpiThreads) {
                 const int r = m * ng + rl;
                 const float scale = scales[rl];
-                float4 acc4 = kEmpty;
+                Stat all{-INFINITY, 0.f, 0.f, 0};
 #pragma unroll 1
                 for (int s4 = 0; s4 < 4; ++s4) {
-                    float4 st = stats[s4 * ng + rl];
+                    const float4 st = stats[s4 * ng + rl];
                     stats[s4 * ng + rl] = kEmpty;
-                    st.x *= scale;  // log2 units
-                    acc4 = merge_stat(acc4, st);
+                    all = merge2(all, Stat{st.x * scale /* log2 units */, st.y, st.z, __float_as_int(st.w)});
                 }
                 if (r < rows && rpd_check(2 * g + static_cast<int>(rank) < p.max_splits, p.meta + kMetaStatus))
-                    p.partials[static_cast<size_t>(r) * p.max_splits + 2 * g + static_cast<int>(rank)] = acc4;
+                    p.partials[static_cast<size_t>(r) * p.max_splits + 2 * g + static_cast<int>(rank)] =
+                        make_float4(all.m, all.s, all.t, __int_as_float(all.a));
             }
             __syncwarp();
             if (lane == 0) counter_add_release(&p.meta[kMetaUnitsDone], 1);
@@ -1070,11 +1027,32 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     }
 
     if (pass.rows > 0) {
-        if (pass.mode == kHeadModePair)
-            head_pair(&maps.u, &maps.w128, p, sm, pass.rows, pass.splits, first_unit, tmem_base);
-        else if (pass.mode == kHeadModeRowsN)
-            head_swap(maps.u_rows, &maps.w128, p, sm, pass.rows, pass.splits / 2, pass.swap_rows,
-                      first_unit, tmem_base);
+        const bool pair = pass.mode == kHeadModePair;
+        const int ng = pair ? kPairTileM : pass.swap_rows;
+        const int splits = pair ? pass.splits : pass.splits / 2;
+        const int num_kb = (p.d + kTileK - 1) / kTileK;
+        TileWalk tw;
+        tw.init(pass.rows, ng, p.V, p.d, splits);
+        if (warp == 0) {
+            if (lane == 0 && !p.stall) {
+                // this CTA's half of the tile's rows, one copy (rows on N: the map whose box is half
+                // a group high)
+                const int half = ng / 2;
+                const CUtensorMap *u = pair ? &maps.u : &maps.u_rows[half / kUBoxRows - 1];
+                if (!pair) tma_prefetch_desc(u);
+                const Copies copies{&maps.w128, u,
+                                    pair ? kPairStages : swap_stages(ng),
+                                    pair ? kPairStageBytesA + kPairStageBytesB : swap_stage_bytes(ng),
+                                    pair ? kPairStageBytesA : 0,
+                                    pair ? 0 : kSwapStageBytesA,
+                                    ng, static_cast<int>(rank) * half};
+                produce(p, sm, copies, rank, tw, pass.rows, num_kb, first_unit);
+            }
+        } else if (pair) {
+            head_pair(p, sm, tw, pass.rows, splits, num_kb, tmem_base);
+        } else {
+            head_swap(p, sm, tw, pass.rows, splits, num_kb, ng, tmem_base);
+        }
     }
     __syncwarp();
     tc_fence_before_sync();

@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(kBandThreads, 1) k_band(BandParams p) {
     // 2. the second pass: the K-1 earlier window layers of the band positions
     const long long rows = static_cast<long long>(p.K - 1) * carry;
     if (warp == 0) {
-        const HeadPlan hp = lookup_plan(rows, p.plan, p.plan_rows, p.plan_in);
+        const HeadPlan hp = table_plan(rows, p.plan, p.plan_rows);
         if (lane == 0) {
             p.meta[kMetaSwapRows] = hp.swap_rows;
             p.meta[kMetaSplits] = hp.splits;

@@ -177,23 +177,28 @@ HeadPlanInputs plan_inputs(const rpd_ctx *c) {
     return in;
 }
 
-// The head-tiling plan of every pass row count up to min(scratch rows, kPlanRows), evaluated
-// here (memoised by the quantities the plan depends on: the pair tile count, and the rows-on-N
-// group count and size) and uploaded to the device table the step's kernels look up.  The
-// stream must be idle (no step may be reading the table).
+// The head-tiling plans: of every pass row count up to kPlanRows and of every 256th row count up
+// to the scratch's rows (memoised by the quantities a plan depends on: the pair tile count, and the
+// rows-on-N group count and size), uploaded to the device table the step's kernels look up, and
+// those of small passes for the head kernel's argument.  The stream must be idle (no step may be
+// reading the table).
+int plan_entries(int cap_rows) {  // of the device table (cap_rows: a multiple of kPairTileM)
+    return std::min(cap_rows, kPlanRows) + 1 + std::max(0, cap_rows - kPlanRows) / kPairTileM;
+}
+
 int build_plan(rpd_ctx *c) {
-    const int n = std::min(c->cap_rows, kPlanRows);
-    if (!c->plan || n < 0) return RPD_OK;
+    if (!c->plan) return RPD_OK;
     const HeadPlanInputs in = plan_inputs(c);
     const int gmax2 = std::min(in.num_n, in.max_splits);
     const int gmax3 = std::min(in.num_n, in.max_splits / 2);
-    const int m = std::max(n, kStepPlanRows);
-    std::vector<HeadPlan> table(static_cast<size_t>(m) + 1);
-    std::vector<unsigned long long> key2((m + kPairTileM - 1) / kPairTileM + 1, 0ull);
+    const int entries = plan_entries(c->cap_rows);
+    std::vector<HeadPlan> table(static_cast<size_t>(std::max(entries, kStepPlanRows + 1)));
+    std::vector<unsigned long long> key2(std::max(c->cap_rows, kStepPlanRows) / kPairTileM + 1, 0ull);
     std::vector<std::vector<unsigned long long>> key3;  // [groups][ng / step]
-    for (int r = 0; r <= m; ++r) {
+    for (int i = 0; i < static_cast<int>(table.size()); ++i) {
+        const int r = i <= kPlanRows ? i : kPlanRows + (i - kPlanRows) * kPairTileM;
         if (r == 0 || in.pair_slots <= 0) {
-            table[r] = plan_head(r, in);
+            table[i] = plan_head(r, in);
             continue;
         }
         const int tiles2 = (r + kPairTileM - 1) / kPairTileM;
@@ -209,13 +214,13 @@ int build_plan(rpd_ctx *c) {
             if (!row[slot]) row[slot] = best_split_key(swap_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax3, 1, 1);
             k3 = row[slot];
         }
-        table[r] = plan_from_keys(in, key2[tiles2], k3, ng);
+        table[i] = plan_from_keys(in, key2[tiles2], k3, ng);
     }
     fill_step_plan(c->step_plan, [&](int r) { return table[r]; });
-    cudaError_t e = cudaMemcpy(c->plan, table.data(), (static_cast<size_t>(n) + 1) * sizeof(HeadPlan),
+    cudaError_t e = cudaMemcpy(c->plan, table.data(), static_cast<size_t>(entries) * sizeof(HeadPlan),
                                cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(plan table)");
-    c->plan_rows = n;
+    c->plan_rows = std::min(c->cap_rows, kPlanRows);
     return RPD_OK;
 }
 
@@ -251,7 +256,7 @@ int ensure_scratch(rpd_ctx *c, int B, int N) {
         {reinterpret_cast<void **>(&c->canvas_off), static_cast<size_t>(new_b + 1) * 4},
         {reinterpret_cast<void **>(&c->meta), kMetaWords * 4},
         {reinterpret_cast<void **>(&c->plan),
-         (static_cast<size_t>(std::min<long long>(rows, kPlanRows)) + 1) * sizeof(HeadPlan)},
+         static_cast<size_t>(plan_entries(static_cast<int>(rows))) * sizeof(HeadPlan)},
     };
     for (auto &a : allocs) {
         e = cudaMalloc(a.p, a.bytes);
@@ -366,7 +371,7 @@ BatchScoreParams batch_score_params(const ScoreParams &sp, const float *tau, con
 // The compaction of a step's mask; `lazy` as in CompactParams.
 CompactParams compact_params(const rpd_ctx *c, const uint8_t *mask, int B, int N, int lazy) {
     return CompactParams{mask, c->q_of_pos, c->pos_of_q, c->canvas_off, c->meta, B, N, c->K,
-                         plan_inputs(c), c->plan, c->plan_rows, c->rule.block, lazy};
+                         c->plan, c->plan_rows, c->rule.block, lazy};
 }
 
 // One launch of the head kernel: the pass over the mask's positions (from_mask) or over those the
@@ -479,7 +484,6 @@ int run_step(rpd_ctx *c, const void *hidden, uint8_t *mask, int B, int N, const 
             bp.N = N;
             bp.K = c->K;
             bp.theta_c = c->rule.theta_c;
-            bp.plan_in = cp.plan_in;
             bp.plan = c->plan;
             bp.plan_rows = c->plan_rows;
             for (int b = 0; b < B; ++b) bp.tau[b] = tau[b];

@@ -121,7 +121,7 @@ struct HeadPlanInputs {
     float hbm_tiles;  // time to stream the head once, in tile units
     int force;        // RPD_TILING_*
 };
-// Rows up to which a context tabulates the plan (larger passes evaluate it on the device).
+// Rows up to which a context tabulates the plan row by row (a multiple of kPairTileM).
 constexpr int kPlanRows = 16384;
 
 // The plans of passes of up to kStepPlanRows rows as a kernel argument: a plan depends on the row
@@ -142,8 +142,7 @@ struct CompactParams {
     int32_t *canvas_off;  // [B+1]
     int32_t *meta;        // [kMetaWords]
     int B, N, K;
-    HeadPlanInputs plan_in;
-    const HeadPlan *plan; // [plan_rows + 1] plans by row count, or null
+    const HeadPlan *plan; // the context's tables (table_plan)
     int plan_rows;
     int block;            // 0: every masked position; > 0: only each canvas's active block
     int lazy;             // 0: all window layers; 1: lazy; 2: lazy when it is estimated cheaper
@@ -192,7 +191,6 @@ struct BandParams {
     int32_t *sel_q;            // out: compact indices of the band positions
     int B, N, K;
     float theta_c;
-    HeadPlanInputs plan_in;
     const HeadPlan *plan;
     int plan_rows;
     float tau[kMaxBatch];

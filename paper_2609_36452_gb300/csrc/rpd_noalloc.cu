@@ -243,7 +243,7 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
         const HeadPlanInputs plan_in{num_n, splits, pair_slots,
                                      head_stream_in_tiles(V, d, dev->num_sms), RPD_TILING_AUTO};
         HeadParams hp{};
-        hp.compact = CompactParams{mask, q_of_pos, pos_of_q, canvas_off, meta, 1, N, K, plan_in,
+        hp.compact = CompactParams{mask, q_of_pos, pos_of_q, canvas_off, meta, 1, N, K,
                                    nullptr, 0, rule.block, 0};
         hp.plan = step_plan_for(*dev, plan_in, V, d);
         hp.norm = NormParams{static_cast<const __nv_bfloat16 *>(hidden),

@@ -3,6 +3,7 @@
 #pragma once
 
 #include "head_plan.h"
+#include "ptx.cuh"
 #include "rpd_internal.h"
 
 namespace rpd {
@@ -32,7 +33,7 @@ __device__ __forceinline__ Stat merge2(const Stat &x, const Stat &y) {
     Stat r;
     r.m = fmaxf(x.m, y.m);
     const float dx = x.m - r.m, dy = y.m - r.m;
-    const float ax = exp2f(dx), ay = exp2f(dy);
+    const float ax = ex2(dx), ay = ex2(dy);
     r.s = ax * x.s + ay * y.s;
     r.t = ax * fmaf(dx, x.s, x.t) + ay * fmaf(dy, y.s, y.t);
     r.a = (x.m > y.m) ? x.a : (y.m > x.m) ? y.a : min(x.a, y.a);

@@ -138,7 +138,7 @@ __device__ __forceinline__ int compact_mask(const CompactParams &p, const MaskMa
 
 // The plan of a pass that the kernel compacts itself; one warp.
 __device__ __forceinline__ HeadPlan pass_plan(const CompactParams &p, const StepPlan &plan, long long rows) {
-    return rows <= kStepPlanRows ? step_plan(plan, rows) : lookup_plan(rows, p.plan, p.plan_rows, p.plan_in);
+    return rows <= kStepPlanRows ? step_plan(plan, rows) : table_plan(rows, p.plan, p.plan_rows);
 }
 
 // Which window layers the step's first pass projects; one warp.  Automatic choice: lazy when its
@@ -146,11 +146,9 @@ __device__ __forceinline__ HeadPlan pass_plan(const CompactParams &p, const Step
 // fraction) are estimated cheaper than one pass over all layers.
 __device__ __forceinline__ bool choose_lazy(const CompactParams &p, const StepPlan &plan, int masked) {
     if (p.lazy != 2 || p.K <= 1) return p.lazy == 1 && p.K > 1;
-    const long long all_rows = static_cast<long long>(p.K) * masked;
-    const long long guess = static_cast<long long>(kLazyBandGuess * (p.K - 1) * masked);
-    const float e_all = pass_plan(p, plan, all_rows).est;
+    const float e_all = pass_plan(p, plan, static_cast<long long>(p.K) * masked).est;
     const float e_fin = pass_plan(p, plan, masked).est;
-    const float e_band = pass_plan(p, plan, guess).est;
+    const float e_band = pass_plan(p, plan, static_cast<long long>(kLazyBandGuess * (p.K - 1) * masked)).est;
     return e_fin + e_band < e_all;
 }
 

@@ -110,6 +110,41 @@ __host__ __device__ inline HeadPlan plan_head(long long rows, const HeadPlanInpu
     return plan_from_keys(in, key2, key3, ng);
 }
 
+// Row groups of a pass of more than one group, with their sizes weighed against pair tiles once
+// more: plan_head has as few groups as possible, but smaller ones may fit the rows better (1068
+// rows: five groups of 224 leave 52 rows of padding, five pair tiles 212).  Time per tile in pair
+// tiles' time, at groups that share the head's tiles through L2 (measured with 2 to 6 groups of
+// 96 to 512 rows at the LLaDA head, d = 4096; in the power-limited steady state, where the clock
+// follows the work, the differences are larger: 1068 rows 732 us with pair tiles, 704 with groups of 224).
+__host__ __device__ inline float group_tile_cost(int ng) {
+    // groups of 32, 64, ..., 512 rows
+    constexpr float kCost[kSwapMaxRows / kSwapRowStep] = {0.70f, 0.70f, 0.72f, 0.74f, 0.79f, 0.85f,
+                                                          0.94f, 1.05f, 1.22f, 1.41f, 1.57f, 1.68f,
+                                                          1.95f, 2.05f, 2.16f, 2.30f};
+    return kCost[ng / kSwapRowStep - 1];
+}
+constexpr int kRegroupMaxGroups = 8;
+
+inline HeadPlan regroup_plan(const HeadPlan &plan, long long rows, const HeadPlanInputs &in) {
+    const int gmax = (in.num_n < in.max_splits / 2 ? in.num_n : in.max_splits / 2);
+    if (!in.regroup || in.force != RPD_TILING_AUTO || rows <= kSwapMaxRows || in.pair_slots <= 0 || gmax <= 0 ||
+        rows > static_cast<long long>(kRegroupMaxGroups) * kPairTileM)
+        return plan;
+    const int tiles2 = static_cast<int>((rows + kPairTileM - 1) / kPairTileM);
+    unsigned long long best = best_split_key(1.f, tiles2, in.pair_slots, in.num_n,
+                                             in.num_n < in.max_splits ? in.num_n : in.max_splits, 1, 1);
+    HeadPlan chosen{kHeadModePair, static_cast<int>(best & 0xFFFFFull), 0, plan.est};
+    for (int groups = swap_groups(rows); groups <= kRegroupMaxGroups; ++groups) {
+        const int ng = swap_group_rows(rows, groups);
+        const unsigned long long key =
+            best_split_key(group_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax, 1, 1);
+        if (key >> 20 >= best >> 20) continue;
+        best = key;
+        chosen = HeadPlan{kHeadModeRowsN, 2 * static_cast<int>(key & 0xFFFFFull), ng, plan.est};
+    }
+    return chosen;
+}
+
 // The kernel argument with the plans of every pass of up to kStepPlanRows rows; `plan(rows)`.
 template <typename Plan>
 inline void fill_step_plan(StepPlan &p, Plan plan) {

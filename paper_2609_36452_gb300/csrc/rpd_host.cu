@@ -174,6 +174,7 @@ HeadPlanInputs plan_inputs(const rpd_ctx *c) {
     in.pair_slots = c->head_grid / 2;
     in.hbm_tiles = head_stream_in_tiles(c->V, c->d, c->num_sms);
     in.force = c->tiling;
+    in.regroup = 1;
     return in;
 }
 
@@ -195,6 +196,7 @@ int build_plan(rpd_ctx *c) {
     std::vector<HeadPlan> table(static_cast<size_t>(std::max(entries, kStepPlanRows + 1)));
     std::vector<unsigned long long> key2(std::max(c->cap_rows, kStepPlanRows) / kPairTileM + 1, 0ull);
     std::vector<std::vector<unsigned long long>> key3;  // [groups][ng / step]
+    HeadPlan regrouped{};
     for (int i = 0; i < static_cast<int>(table.size()); ++i) {
         const int r = i <= kPlanRows ? i : kPlanRows + (i - kPlanRows) * kPairTileM;
         if (r == 0 || in.pair_slots <= 0) {
@@ -215,6 +217,10 @@ int build_plan(rpd_ctx *c) {
             k3 = row[slot];
         }
         table[i] = plan_from_keys(in, key2[tiles2], k3, ng);
+        if (r <= kRegroupMaxGroups * kPairTileM) {  // a function of the multiple of 32 rows
+            if (r % kSwapRowStep == 1) regrouped = regroup_plan(table[i], r, in);
+            table[i] = regrouped;
+        }
     }
     fill_step_plan(c->step_plan, [&](int r) { return table[r]; });
     cudaError_t e = cudaMemcpy(c->plan, table.data(), static_cast<size_t>(entries) * sizeof(HeadPlan),

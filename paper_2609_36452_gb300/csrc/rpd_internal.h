@@ -120,6 +120,7 @@ struct HeadPlanInputs {
     int pair_slots;   // CTA pairs of the head kernel
     float hbm_tiles;  // time to stream the head once, in tile units
     int force;        // RPD_TILING_*
+    int regroup;      // also weigh more, smaller row groups (regroup_plan)
 };
 // Rows up to which a context tabulates the plan row by row (a multiple of kPairTileM).
 constexpr int kPlanRows = 16384;

@@ -21,11 +21,22 @@ int main(int argc, char **argv) {
     in.pair_slots = sms / 2;
     in.hbm_tiles = rpd::head_stream_in_tiles(V, d, sms);
     in.force = force;
+    in.regroup = 1;
+    auto plan = [&](int r) { return rpd::regroup_plan(rpd::plan_head(r, in), r, in); };
     rpd::StepPlan sp;
-    rpd::fill_step_plan(sp, [&](int r) { return rpd::plan_head(r, in); });
+    rpd::fill_step_plan(sp, plan);
     int bad = 0;
+    for (int r = 1; r <= 4096; ++r) {  // regrouping keeps the plan's rules at every row count
+        const rpd::HeadPlan a = plan(r);
+        const bool rows_n = a.mode == rpd::kHeadModeRowsN;
+        const int splits = rows_n ? a.splits / 2 : a.splits;
+        bad += splits < 1 || splits > in.num_n || a.splits > in.max_splits || a.est != rpd::plan_head(r, in).est;
+        bad += rows_n && (a.swap_rows % 32 || a.swap_rows < 32 || a.swap_rows > 512);
+        bad += force == RPD_TILING_PAIR && rows_n;
+        bad += force == RPD_TILING_ROWS_N && !rows_n && in.max_splits >= 2;
+    }
     for (int r = 1; r <= rpd::kStepPlanRows; ++r) {
-        const rpd::HeadPlan a = rpd::plan_head(r, in);
+        const rpd::HeadPlan a = plan(r);
         const int i = (r - 1) / 32;
         const int splits = sp.splits[i] < 0 ? -sp.splits[i] : sp.splits[i];
         const int mode = sp.splits[i] < 0 ? rpd::kHeadModeRowsN : rpd::kHeadModePair;

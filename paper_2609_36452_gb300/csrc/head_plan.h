@@ -145,6 +145,30 @@ inline HeadPlan regroup_plan(const HeadPlan &plan, long long rows, const HeadPla
     return chosen;
 }
 
+// Pair tiles in whole waves over the CTA pairs and a rest of at most half a wave: the rest runs as
+// half tiles (128 vocabulary entries), two to a tile, in about half a wave.  Each row then has two
+// partials per vocabulary tile, which the scratch must hold.  One of eight slices of the LLaDA
+// head, 748 rows: 186 tiles on 76 pairs took three waves.
+struct TailSplit {
+    int whole, units;  // tiles in whole waves; work units in all
+};
+__host__ __device__ inline TailSplit tail_split(int tiles, int pairs) {
+    const int rest = tiles % pairs;
+    return TailSplit{tiles - rest, tiles + rest};
+}
+constexpr int kTailMaxWaves = 8;  // with more, the rest is no longer worth the partials
+
+inline HeadPlan split_tail(const HeadPlan &plan, long long rows, const HeadPlanInputs &in) {
+    if (!in.regroup || in.force != RPD_TILING_AUTO || plan.mode != kHeadModePair || in.pair_slots <= 0 ||
+        rows <= 0 || 2 * in.num_n > in.max_splits)
+        return plan;
+    const long long tiles = (rows + kPairTileM - 1) / kPairTileM * in.num_n;
+    const int rest = static_cast<int>(tiles % in.pair_slots);
+    if (tiles > static_cast<long long>(kTailMaxWaves) * in.pair_slots || rest == 0 || 2 * rest > in.pair_slots)
+        return plan;
+    return HeadPlan{kHeadModePair, 2 * in.num_n, kSplitTail, plan.est};
+}
+
 // The kernel argument with the plans of every pass of up to kStepPlanRows rows; `plan(rows)`.
 template <typename Plan>
 inline void fill_step_plan(StepPlan &p, Plan plan) {

@@ -43,17 +43,28 @@ constexpr float kLog2e = 1.4426950408889634f;
 // The units running at the same time therefore share W tiles (each streamed from HBM once
 // per band) and re-read at most `band` u tiles (kept in L2 while the band runs).  With few
 // row tiles there is a single band and the order is plain (m fastest).
+// With a split tail every unit is one tile, and those after the last whole wave are half tiles.
 struct TileWalk {
     int num_m, num_n, splits, units, band;
-    __device__ __forceinline__ void init(int rows, int tile_rows, int V, int d, int g) {
+    int whole;  // units before the half tiles
+    __device__ __forceinline__ void init(int rows, int tile_rows, int V, int d, int g, bool tail) {
         num_m = (rows + tile_rows - 1) / tile_rows;
         num_n = (V + kTileN - 1) / kTileN;
-        splits = g;
+        splits = tail ? num_n : g;
         units = num_m * splits;
+        whole = units;
+        if (tail) {
+            const TailSplit t = tail_split(units, gridDim.x / 2);
+            whole = t.whole;
+            units = t.units;
+        }
         band = static_cast<int>(kBandBytes / 2) / tile_rows / d;
         band = max(1, min(num_m, band));
     }
-    __device__ __forceinline__ void unit(int u, int &m, int &g, int &n0, int &n1) const {
+    // A unit's vocabulary range is given in half tiles [v0, v1); an odd one is a half tile.
+    __device__ __forceinline__ void unit(int u, int &m, int &g, int &v0, int &v1) const {
+        const int half = u - whole;  // of tile whole + half / 2
+        if (half >= 0) u = whole + (half >> 1);
         const int per_band = band * splits;
         const int b = u / per_band;
         const int r = u - b * per_band;
@@ -62,8 +73,12 @@ struct TileWalk {
         m = m0 + r % in_band;
         g = r / in_band;
         // at most a few hundred splits of at most 2^23 tiles: the products fit 32 bits
-        n0 = static_cast<int>(static_cast<unsigned>(g) * num_n / splits);
-        n1 = static_cast<int>(static_cast<unsigned>(g + 1) * num_n / splits);
+        v0 = 2 * static_cast<int>(static_cast<unsigned>(g) * num_n / splits);
+        v1 = 2 * static_cast<int>(static_cast<unsigned>(g + 1) * num_n / splits);
+        if (half >= 0) {
+            v0 += half & 1;
+            v1 = v0 + 1;
+        }
     }
 };
 
@@ -272,9 +287,21 @@ __device__ __forceinline__ int swap_stages(int ng) {
 // What one CTA's TMA producer copies: per stage 128 head rows x 64 columns (w_off bytes into the
 // stage) and this CTA's rows of u x 64 columns (u_off), u_rows * m + u_row0 on for row tile m.
 struct Copies {
-    const CUtensorMap *w, *u;
+    const CUtensorMap *w, *w_half, *u;
     int stages, stage_bytes, w_off, u_off, u_rows, u_row0;
 };
+
+// Bytes of a stage that the pair expects: a half tile brings 64 head rows to each CTA, not 128.
+__device__ __forceinline__ uint32_t stage_bytes(const Copies &c, bool half) {
+    return 2u * (c.stage_bytes - (half ? 64 * kTileK * 2 : 0));
+}
+
+// First row of the head that this CTA copies for the tile at half tile v, in rows of W (of the tiled
+// copy: block (v + rank, kb = 0), 128 contiguous rows of 64 columns).
+__device__ __forceinline__ int head_row(const HeadParams &p, int v, bool half, uint32_t rank, int num_kb) {
+    const int block = half ? v : v + static_cast<int>(rank);
+    return (p.w_tiled ? block * num_kb : block) * kPairHalfRows + (half ? static_cast<int>(rank) * 64 : 0);
+}
 
 // One tile's K-steps kb0 .. num_kb - 1; returns how many were issued (fewer if a wait gave up).
 // The loop is kept as tight as it gets: the same copies issued
@@ -282,25 +309,25 @@ struct Copies {
 // mid-decode passes 1.5 to 3 % slower.  kOnce: drop the head tile from L2 first (see produce).
 template <bool kOnce>
 __device__ __forceinline__ int copy_tile(const HeadParams &p, const HeadSmem &sm, const Copies &c,
-                                          uint32_t rank, uint32_t full0, uint64_t evict_first, int n,
-                                          int u_row, int kb0, int num_kb, int &stage, uint32_t &phase) {
-    // block (2n + rank, kb) of the tiled copy (128 contiguous rows of 64), or the same rows and
-    // columns of W in place
-    const int block = 2 * n + static_cast<int>(rank);
+                                          uint32_t rank, uint32_t full0, uint64_t evict_first, int v,
+                                          bool half, int u_row, int kb0, int num_kb, int &stage,
+                                          uint32_t &phase) {
     const int dx = p.w_tiled ? 0 : kTileK, dy = p.w_tiled ? kPairHalfRows : 0;
     int x = kb0 * dx;
-    int y = (p.w_tiled ? block * num_kb + kb0 : block) * kPairHalfRows;
+    int y = head_row(p, v, half, rank, num_kb) + kb0 * dy;
+    const CUtensorMap *w = half ? c.w_half : c.w;
+    const uint32_t bytes = stage_bytes(c, half);
     int kb = kb0;
     for (; kb < num_kb; ++kb, x += dx, y += dy) {
         if (!mbar_wait_bounded(&sm.empty[stage], phase ^ 1u, sm.abort_flag, p.wait_limit_ns)) break;
-        if (rank == 0) mbar_arrive_expect_tx(&sm.full[stage], 2 * c.stage_bytes);
+        if (rank == 0) mbar_arrive_expect_tx(&sm.full[stage], bytes);
         const uint32_t bar = full0 + static_cast<uint32_t>(stage * sizeof(uint64_t));
         uint8_t *st = sm.ring + stage * c.stage_bytes;
         tma_load_2d_pair(st + c.u_off, c.u, bar, kb * kTileK, u_row);
         if (kOnce)
-            tma_load_2d_pair_hint(st + c.w_off, c.w, bar, x, y, evict_first);
+            tma_load_2d_pair_hint(st + c.w_off, w, bar, x, y, evict_first);
         else
-            tma_load_2d_pair(st + c.w_off, c.w, bar, x, y);
+            tma_load_2d_pair(st + c.w_off, w, bar, x, y);
         if (++stage == c.stages) {
             stage = 0;
             phase ^= 1u;
@@ -314,19 +341,20 @@ __device__ __forceinline__ int copy_tile(const HeadParams &p, const HeadSmem &sm
 // K-steps issued, or -1 if the wait gave up.
 __device__ __forceinline__ int copy_ahead(const HeadParams &p, const HeadSmem &sm, const Copies &c,
                                           uint32_t rank, uint32_t full0, bool once, uint64_t evict_first,
-                                          int n, int u_row, int rows, int num_kb) {
+                                          int v, bool half, int u_row, int rows, int num_kb) {
     const int ahead = min(c.stages, num_kb);
-    const int block = 2 * n + static_cast<int>(rank);
+    const int y0 = head_row(p, v, half, rank, num_kb);
+    const CUtensorMap *w = half ? c.w_half : c.w;
     for (int s = 0; s < ahead; ++s) {
-        if (rank == 0) mbar_arrive_expect_tx(&sm.full[s], 2 * c.stage_bytes);
+        if (rank == 0) mbar_arrive_expect_tx(&sm.full[s], stage_bytes(c, half));
         const uint32_t bar = full0 + static_cast<uint32_t>(s * sizeof(uint64_t));
         uint8_t *dst = sm.ring + s * c.stage_bytes + c.w_off;
         const int x = p.w_tiled ? 0 : s * kTileK;
-        const int y = (p.w_tiled ? block * num_kb + s : block) * kPairHalfRows;
+        const int y = y0 + (p.w_tiled ? s * kPairHalfRows : 0);
         if (once)
-            tma_load_2d_pair_hint(dst, c.w, bar, x, y, evict_first);
+            tma_load_2d_pair_hint(dst, w, bar, x, y, evict_first);
         else
-            tma_load_2d_pair(dst, c.w, bar, x, y);
+            tma_load_2d_pair(dst, w, bar, x, y);
     }
     if (!wait_for_rows(p, sm, rows, 0)) return -1;
     proxy_fence();
@@ -358,13 +386,13 @@ __device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm,
     while (ok) {
         int u;
         if (!claim_unit(p, sm, rank, tw.units, uc, first, u) || u < 0) break;
-        int m, g, n0, n1;
-        tw.unit(u, m, g, n0, n1);
+        int m, g, v0, v1;
+        tw.unit(u, m, g, v0, v1);
         const int u_row = m * c.u_rows + c.u_row0;
         int kb0 = 0;
         if (!started) {
             started = true;
-            kb0 = copy_ahead(p, sm, c, rank, full0, once, evict_first, n0, u_row, rows, num_kb);
+            kb0 = copy_ahead(p, sm, c, rank, full0, once, evict_first, v0, v0 + 1 == v1, u_row, rows, num_kb);
             fills = kb0 < 0 ? min(c.stages, num_kb) : kb0;
             if (kb0 < 0) break;
             if (kb0 == c.stages)
@@ -372,10 +400,11 @@ __device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm,
             else
                 stage = kb0;
         }
-        for (int n = n0; ok && n < n1; ++n, kb0 = 0) {
+        for (int v = v0; ok && v < v1; v += 2, kb0 = 0) {
+            const bool half = v + 1 == v1;
             const int issued =
-                once ? copy_tile<true>(p, sm, c, rank, full0, evict_first, n, u_row, kb0, num_kb, stage, phase)
-                     : copy_tile<false>(p, sm, c, rank, full0, evict_first, n, u_row, kb0, num_kb, stage, phase);
+                once ? copy_tile<true>(p, sm, c, rank, full0, evict_first, v, half, u_row, kb0, num_kb, stage, phase)
+                     : copy_tile<false>(p, sm, c, rank, full0, evict_first, v, half, u_row, kb0, num_kb, stage, phase);
             fills += issued;
             ok = issued == num_kb - kb0;
         }
@@ -402,7 +431,7 @@ __device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm,
 // thread in both CTAs; acc_empty[a] lives in the even CTA and counts the 4 epilogue warps
 // of both CTAs (8 arrivals).
 __device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &sm, const TileWalk &tw,
-                                          int rows, int splits, int num_kb, uint32_t tmem_base) {
+                                          int rows, int splits, bool tail, int num_kb, uint32_t tmem_base) {
     constexpr int kStageBytes = kPairStageBytesA + kPairStageBytesB;
     uint64_t *full = sm.full, *empty = sm.empty, *acc_full = sm.acc_full,
              *acc_empty = sm.acc_empty, *unit_full = sm.unit_full, *unit_empty = sm.unit_empty;
@@ -416,7 +445,6 @@ __device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &s
         if (rank == 0) {
             // -------------------------------------------- MMA issuer (even CTA only): the whole
             // warp runs the loop, one elected lane issues (every branch below is warp-uniform)
-            constexpr uint32_t idesc = idesc_bf16_f32(kPairTileM, kTileN);
             int stage = 0;
             uint32_t phase = 0;
             uint32_t tile_iter = 0;
@@ -430,9 +458,10 @@ __device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &s
                 if (lane == 0) mbar_arrive(&unit_empty[uc.slot]);
                 uc.advance();
                 if (u < 0) break;
-                int m, g, n0, n1;
-                tw.unit(u, m, g, n0, n1);
-                for (int n = n0; ok && n < n1; ++n, ++tile_iter) {
+                int m, g, v0, v1;
+                tw.unit(u, m, g, v0, v1);
+                const uint32_t idesc = idesc_bf16_f32(kPairTileM, v0 + 1 == v1 ? kTileN / 2 : kTileN);
+                for (int v = v0; ok && v < v1; v += 2, ++tile_iter) {
                     const uint32_t acc = tile_iter & 1u;
                     const uint32_t acc_phase = (tile_iter >> 1) & 1u;
                     if (!mbar_wait_bounded_warp(&acc_empty[acc], acc_phase ^ 1u, abort_flag,
@@ -491,14 +520,15 @@ __device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &s
                 mbar_arrive_cluster(unit_empty0 + static_cast<uint32_t>(uc.slot * sizeof(uint64_t)));
             uc.advance();
             if (u < 0) break;
-            int m, g, n0, n1;
-            tw.unit(u, m, g, n0, n1);
+            int m, g, v0, v1;
+            tw.unit(u, m, g, v0, v1);
+            const int chunks = (v0 + 1 == v1 ? kTileN / 2 : kTileN) / 32;
             const int r = m * kPairTileM + row_in_tile;
             const bool valid = r < rows;
             const float scale = valid ? p.norm.inv_rms[r] * kLog2e : 0.f;
             float run_m = -INFINITY, run_s = 0.f, run_t = 0.f;
             int run_a = 0;
-            for (int n = n0; n < n1; ++n, ++tile_iter) {
+            for (int tile = v0; tile < v1; tile += 2, ++tile_iter) {
                 const uint32_t acc = tile_iter & 1u;
                 const uint32_t acc_phase = (tile_iter >> 1) & 1u;
                 if (!mbar_wait_bounded(&acc_full[acc], acc_phase, abort_flag, p.wait_limit_ns)) {
@@ -506,10 +536,10 @@ __device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &s
                     break;
                 }
                 tc_fence_after_sync();
-                const int col_base = n * kTileN;
-                const bool full_tile = col_base + kTileN <= p.V;
+                const int col_base = tile * (kTileN / 2);
+                const bool full_tile = col_base + chunks * 32 <= p.V;
 #pragma unroll 1
-                for (int c = 0; c < kTileN / 32; ++c) {
+                for (int c = 0; c < chunks; ++c) {
                     float v[32];
                     tmem_ld_32x32b_x32(lane_base + acc * kTileN + c * 32, v);
                     if (full_tile)
@@ -522,9 +552,12 @@ __device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &s
                 if (lane < 2) mbar_arrive_cluster(acc_empty0 + acc * static_cast<uint32_t>(sizeof(uint64_t)));
             }
             if (!ok) break;
-            if (valid && rpd_check(g < p.max_splits, p.meta + kMetaStatus)) {
-                p.partials[static_cast<size_t>(r) * p.max_splits + g] =
-                    make_float4(run_m * scale, run_s, run_t, __int_as_float(run_a));
+            // with a split tail a row has a partial per half tile: a whole tile's second one is empty
+            const int slot = tail ? v0 : g;
+            if (valid && rpd_check(slot + (tail && v0 + 1 < v1) < p.max_splits, p.meta + kMetaStatus)) {
+                float4 *part = p.partials + static_cast<size_t>(r) * p.max_splits + slot;
+                part[0] = make_float4(run_m * scale, run_s, run_t, __int_as_float(run_a));
+                if (tail && v0 + 1 < v1) part[1] = make_float4(-INFINITY, 0.f, 0.f, __int_as_float(0));
             }
             __syncwarp();
             if (lane == 0) counter_add_release(&p.meta[kMetaUnitsDone], 1);
@@ -655,7 +688,7 @@ __device__ __forceinline__ void head_swap(const HeadParams &p, const HeadSmem &s
                 if (u < 0) break;
                 int m, g, v0, v1;
                 tw.unit(u, m, g, v0, v1);
-                for (int n = v0; ok && n < v1; ++n, ++tile_iter) {
+                for (int v = v0; ok && v < v1; v += 2, ++tile_iter) {
                     // tile t-2, which had the same place, has been read ...
                     const uint32_t acc = tile_iter & 1u;
                     if (!mbar_wait_bounded_warp(&acc_empty[acc], ((tile_iter >> 1) & 1u) ^ 1u, abort_flag,
@@ -723,7 +756,7 @@ __device__ __forceinline__ void head_swap(const HeadParams &p, const HeadSmem &s
             for (int rl = etid; rl < ng; rl += kEpiThreads)
                 scales[rl] = m * ng + rl < rows ? p.norm.inv_rms[m * ng + rl] * kLog2e : 0.f;
             if (!epi_sync(sm.epi, epi_phase, abort_flag, p.wait_limit_ns)) break;
-            for (int n = v0; n < v1; ++n, ++tile_iter) {
+            for (int tile = v0; tile < v1; tile += 2, ++tile_iter) {
                 const uint32_t acc = tile_iter & 1u;
                 if (!mbar_wait_bounded(&acc_full[acc], (tile_iter >> 1) & 1u, abort_flag, p.wait_limit_ns)) {
                     ok = false;
@@ -732,7 +765,7 @@ __device__ __forceinline__ void head_swap(const HeadParams &p, const HeadSmem &s
                 tc_fence_after_sync();
                 const SwapPlace place = swap_place(ng, acc);
                 // the 32 vocabulary entries of this warp's sub-partition
-                const int vbase = n * kTileN + static_cast<int>(rank) * kPairHalfRows + sub * 32;
+                const int vbase = tile * (kTileN / 2) + static_cast<int>(rank) * kPairHalfRows + sub * 32;
                 const bool full_tile = vbase + 32 <= p.V;
                 // This warp's chunks are always the same ones (their statistics are its own); the
                 // next tile waits for the shared chunks, so those come first.
@@ -838,7 +871,9 @@ __device__ __forceinline__ int claim_merge(const HeadParams &p, const HeadSmem &
     const bool pair = pass.mode == kHeadModePair;
     const int splits = pair ? pass.splits : pass.splits / 2;
     const int tile_rows = pair ? kPairTileM : pass.swap_rows;
-    const int units = (pass.rows + tile_rows - 1) / tile_rows * splits;
+    int units = (pass.rows + tile_rows - 1) / tile_rows * splits;
+    if (pair && pass.swap_rows == kSplitTail)
+        units = tail_split((pass.rows + tile_rows - 1) / tile_rows * (splits / 2), gridDim.x / 2).units;
     // and the warp that publishes the pass
     const int target = 2 * units * (pair ? kPairEpiWarps : kSwapEpiWarps) + (publishes(p) ? 1 : 0);
     const uint64_t limit = p.wait_limit_ns * (p.V / kTileN / splits + 2);
@@ -1032,7 +1067,8 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         const int splits = pair ? pass.splits : pass.splits / 2;
         const int num_kb = (p.d + kTileK - 1) / kTileK;
         TileWalk tw;
-        tw.init(pass.rows, ng, p.V, p.d, splits);
+        const bool tail = pair && pass.swap_rows == kSplitTail;
+        tw.init(pass.rows, ng, p.V, p.d, splits, tail);
         if (warp == 0) {
             if (lane == 0 && !p.stall) {
                 // this CTA's half of the tile's rows, one copy (rows on N: the map whose box is half
@@ -1040,7 +1076,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
                 const int half = ng / 2;
                 const CUtensorMap *u = pair ? &maps.u : &maps.u_rows[half / kUBoxRows - 1];
                 if (!pair) tma_prefetch_desc(u);
-                const Copies copies{&maps.w128, u,
+                const Copies copies{&maps.w128, &maps.w64, u,
                                     pair ? kPairStages : swap_stages(ng),
                                     pair ? kPairStageBytesA + kPairStageBytesB : swap_stage_bytes(ng),
                                     pair ? kPairStageBytesA : 0,
@@ -1049,7 +1085,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
                 produce(p, sm, copies, rank, tw, pass.rows, num_kb, first_unit);
             }
         } else if (pair) {
-            head_pair(p, sm, tw, pass.rows, splits, num_kb, tmem_base);
+            head_pair(p, sm, tw, pass.rows, splits, tail, num_kb, tmem_base);
         } else {
             head_swap(p, sm, tw, pass.rows, splits, num_kb, ng, tmem_base);
         }

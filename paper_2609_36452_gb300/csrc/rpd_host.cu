@@ -218,7 +218,7 @@ int build_plan(rpd_ctx *c) {
         }
         table[i] = plan_from_keys(in, key2[tiles2], k3, ng);
         if (r <= kRegroupMaxGroups * kPairTileM) {  // a function of the multiple of 32 rows
-            if (r % kSwapRowStep == 1) regrouped = regroup_plan(table[i], r, in);
+            if (r % kSwapRowStep == 1) regrouped = split_tail(regroup_plan(table[i], r, in), r, in);
             table[i] = regrouped;
         }
     }
@@ -584,7 +584,7 @@ int rpd_set_head(rpd_ctx *c, const void *W_head, const void *g_norm) {
     c->W_tiled = nullptr;
     c->W = nullptr;
     ++c->buffers_gen;
-    CUtensorMap m2;
+    CUtensorMap m2, m2_half;
     int rc;
     if (c->head_layout == RPD_HEAD_TILED && c->d % 64 == 0) {
         // rows as 2-D tensor map rows of 64 columns: block (t, k) is map rows
@@ -600,6 +600,7 @@ int rpd_set_head(rpd_ctx *c, const void *W_head, const void *g_norm) {
             return cuda_fail(e, "tiled copy of the head");
         }
         rc = encode_bf16_2d(&m2, wt, vpad * static_cast<uint64_t>(c->d) / 64, 64, kPairHalfRows);
+        if (!rc) rc = encode_bf16_2d(&m2_half, wt, vpad * static_cast<uint64_t>(c->d) / 64, 64, kPairHalfRows / 2);
         if (rc) {
             cudaFree(wt);
             return rc;
@@ -607,9 +608,11 @@ int rpd_set_head(rpd_ctx *c, const void *W_head, const void *g_norm) {
         c->W_tiled = wt;
     } else {
         rc = encode_bf16_2d(&m2, W_head, static_cast<uint64_t>(c->V), c->d, kPairHalfRows);
+        if (!rc) rc = encode_bf16_2d(&m2_half, W_head, static_cast<uint64_t>(c->V), c->d, kPairHalfRows / 2);
         if (rc) return rc;
     }
     c->maps.w128 = m2;
+    c->maps.w64 = m2_half;
     ++c->buffers_gen;
     c->W = W_head;
     c->g = g_norm;

@@ -111,7 +111,7 @@ struct PassInfo {
 struct HeadPlan {
     int mode;       // kHeadModePair or kHeadModeRowsN
     int splits;     // partials per row the merge reads (vocabulary splits; twice that for rows on N)
-    int swap_rows;  // rows per group of the rows-on-N tiling (0 for pair tiles)
+    int swap_rows;  // rows per group of the rows-on-N tiling; pair tiles: 0, or kSplitTail
     float est;      // estimated time, in 128 x 256-tile units
 };
 struct HeadPlanInputs {
@@ -122,6 +122,8 @@ struct HeadPlanInputs {
     int force;        // RPD_TILING_*
     int regroup;      // also weigh more, smaller row groups (regroup_plan)
 };
+// Pair tiles whose last, partly filled wave is issued as half tiles (split_tail).
+constexpr int kSplitTail = 1;
 // Rows up to which a context tabulates the plan row by row (a multiple of kPairTileM).
 constexpr int kPlanRows = 16384;
 
@@ -374,7 +376,7 @@ cudaError_t launch_compact(const CompactParams &p, cudaStream_t s);
 constexpr int kUMaps = (kSwapMaxRows / 2) / kUBoxRows;  // box heights kUBoxRows * (1 .. kUMaps)
 struct HeadMaps {
     CUtensorMap u;                // box 64 x 128 rows
-    CUtensorMap w128;             // box 64 x 128 rows of W
+    CUtensorMap w128, w64;        // boxes 64 x 128 and 64 x 64 rows of W
     CUtensorMap u_rows[kUMaps];   // u_rows[j]: box 64 x kUBoxRows*(j+1) rows
 };
 // The head kernel (every tiling; the pass's choice is read from the meta words), launched as

@@ -159,7 +159,7 @@ StepPlan step_plan_for(DeviceSetup &dev, const HeadPlanInputs &in, int V, int d)
         if (s.V == V && s.d == d) return s.plan;
     ShapePlan &s = dev.plans[dev.next_plan];
     dev.next_plan = (dev.next_plan + 1) % kShapePlans;
-    fill_step_plan(s.plan, [&](int rows) { return regroup_plan(plan_head(rows, in), rows, in); });
+    fill_step_plan(s.plan, [&](int rows) { return split_tail(regroup_plan(plan_head(rows, in), rows, in), rows, in); });
     s.V = V;
     s.d = d;
     return s.plan;
@@ -226,7 +226,9 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
     HeadMaps maps;
     bool maps_ok = encode_tile_map(&maps.u, u, kNaMaxRows, static_cast<uint64_t>(d), kTileM) &&
                    encode_tile_map(&maps.w128, W_head, static_cast<uint64_t>(V),
-                                   static_cast<uint64_t>(d), kPairHalfRows);
+                                   static_cast<uint64_t>(d), kPairHalfRows) &&
+                   encode_tile_map(&maps.w64, W_head, static_cast<uint64_t>(V),
+                                   static_cast<uint64_t>(d), kPairHalfRows / 2);
     for (int j = 0; maps_ok && j < kUMaps; ++j)
         maps_ok = encode_tile_map(&maps.u_rows[j], u, kNaMaxRows, static_cast<uint64_t>(d),
                                   static_cast<uint32_t>(kUBoxRows * (j + 1)));

@@ -102,3 +102,24 @@ def test_two_pass_steps_one_after_another(N, projection, tau, prefix):
             compare_step(ref, got, lazy=lazy)
     finally:
         runner.close()
+
+
+@pytest.mark.parametrize("V,N", [(4100, 200),    # under half a wave: only half tiles, the last one empty
+                                 (20480, 200),   # one wave and four tiles
+                                 (19713, 300),   # two row tiles, a last half tile of one entry
+                                 (9728, 600)])   # three row tiles of 38: one wave and a half exactly
+def test_pair_tiles_with_a_split_tail(V, N):
+    """Whole waves of pair tiles and a rest of half tiles, whose rows have two partials per tile."""
+    K, d = 1, 128
+    W, g, hidden = make(800 + N, K, N, d, V)
+    mask = torch.ones(N, dtype=torch.uint8)
+    ref = O.rpd_step(bits(hidden), mask.numpy(), bits(g), bits(W), 1e-6, 0.9, 1.0, "llada")
+    runner = DeviceRunner(W, g, K)
+    try:
+        got = runner.step(hidden, mask, 0.9, 1.0)
+        runner.ctx.set_head_tiling("pair")  # without the split
+        whole = runner.step(hidden, mask, 0.9, 1.0)
+    finally:
+        runner.close()
+    compare_step(ref, got)
+    compare_step(ref, whole)

@@ -851,10 +851,19 @@ __device__ __forceinline__ void head_swap(const HeadParams &p, const HeadSmem &s
 // pass is done, and the CTA that completes the merge scores the canvas, or selects what the second
 // of two passes projects.
 
-// Whether kernels after this one read of its compaction.
-__device__ __forceinline__ bool publishes(const HeadParams &p) {
-    return p.from_mask && (!p.score_canvas || p.select_band);
-}
+// The kernel is compiled twice: for the plain step - one canvas, one pass over every window layer,
+// scored in the kernel (kPlain) - and for everything else.  What the plain step does not run is
+// not in its code, which it has to fetch anew in every step.
+template <bool kPlain>
+struct StepKind {
+    const HeadParams &p;
+    __device__ __forceinline__ bool from_mask() const { return kPlain || p.from_mask; }
+    __device__ __forceinline__ bool scores() const { return kPlain || p.score_canvas; }
+    __device__ __forceinline__ bool selects() const { return !kPlain && p.select_band; }
+    __device__ __forceinline__ bool lazy() const { return !kPlain && p.compact.lazy; }
+    // whether kernels after this one read of its compaction
+    __device__ __forceinline__ bool publishes() const { return !kPlain && p.from_mask && (!p.score_canvas || p.select_band); }
+};
 
 // A CTA's first claim of a block of rows and the wait for the units (the producer's thread, which
 // is done before the epilogue is); `blocks` if there is nothing to merge.  Only running CTAs hold
@@ -862,6 +871,7 @@ __device__ __forceinline__ bool publishes(const HeadParams &p) {
 // given up (the step's outputs are then meaningless), and after the time in which a unit's own
 // waits would have run out.  A CTA that came so late that the canvas was already being scored
 // claims nothing.
+template <bool kPlain>
 __device__ __forceinline__ int claim_merge(const HeadParams &p, const HeadSmem &sm, const PassInfo &pass,
                                            int blocks) {
     int32_t *meta = p.meta;
@@ -875,7 +885,7 @@ __device__ __forceinline__ int claim_merge(const HeadParams &p, const HeadSmem &
     if (pair && pass.swap_rows == kSplitTail)
         units = tail_split((pass.rows + tile_rows - 1) / tile_rows * (splits / 2), gridDim.x / 2).units;
     // and the warp that publishes the pass
-    const int target = 2 * units * (pair ? kPairEpiWarps : kSwapEpiWarps) + (publishes(p) ? 1 : 0);
+    const int target = 2 * units * (pair ? kPairEpiWarps : kSwapEpiWarps) + (StepKind<kPlain>{p}.publishes() ? 1 : 0);
     const uint64_t limit = p.wait_limit_ns * (p.V / kTileN / splits + 2);
     uint64_t t0 = globaltimer_ns();
     int seen = 0;
@@ -893,27 +903,29 @@ __device__ __forceinline__ int claim_merge(const HeadParams &p, const HeadSmem &
     return block;
 }
 
+template <bool kPlain>
 __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem &sm,
                                             const PassInfo &pass) {
+    const StepKind<kPlain> kind{p};
     int32_t *meta = p.meta;
     volatile int *share = reinterpret_cast<volatile int *>(sm.ring + kHeadRegionBytes - 16);
     const int gs = merge_lanes(pass.splits);
     const int per_block = kHeadKernelThreads / gs;
     const int blocks = (pass.rows + per_block - 1) / per_block;
-    const int first = threadIdx.x == 0 ? claim_merge(p, sm, pass, blocks) : 0;
+    const int first = threadIdx.x == 0 ? claim_merge<kPlain>(p, sm, pass, blocks) : 0;
     __syncthreads();  // the ring is free: every role of this CTA is done
     if (threadIdx.x == 0) {
         if (*sm.abort_flag) atomicExch(&meta[kMetaStatus], RPD_ERR_TIMEOUT);
         share[0] = first;
         // nothing to merge: the first CTA goes on
-        share[1] = blocks == 0 && blockIdx.x == 0 && !*sm.stale && !meta[kMetaScored];
+        share[1] = blocks == 0 && blockIdx.x == 0 && !*sm.stale && (kPlain || !meta[kMetaScored]);
     }
     __syncthreads();
-    const int num_words = p.from_mask ? (p.compact.B * p.compact.N + 31) >> 5 : 0;
+    const int num_words = kind.from_mask() ? (p.compact.B * p.compact.N + 31) >> 5 : 0;
     for (int block = share[0]; block < blocks; block = share[0]) {
         int next = 0;
         if (threadIdx.x == 0) next = atomicAdd(&meta[kMetaMergeNext], 1);  // while this block is merged
-        merge_block(p.merge, pass, p.norm.sel_list, block, gs, meta + kMetaStatus,
+        merge_block<kPlain>(p.merge, pass, p.norm.sel_list, block, gs, meta + kMetaStatus,
                     [&](int q) { return sm.map.position(q, num_words); });
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -923,7 +935,7 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
         __syncthreads();
     }
     if (!share[1]) return;
-    if (p.select_band) {
+    if (kind.selects()) {
         // The positions whose earlier window layers a second pass projects (none if this one had
         // every layer); without any the canvas can be scored now.
         const int per_canvas = p.compact.N;
@@ -950,16 +962,16 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
         }
         if (band > 0) return;
     }
-    if (!p.score_canvas) return;
+    if (!kind.scores()) return;
     int status = RPD_OK, rows_total = pass.rows;
     if (threadIdx.x == 0) {
         *reinterpret_cast<volatile int32_t *>(&meta[kMetaClosed]) = 1;  // before any mask byte changes
         status = ld_acquire(&meta[kMetaStatus]);
-        if (!p.from_mask) rows_total = meta[kMetaRowsTotal];
+        if (!kind.from_mask()) rows_total = meta[kMetaRowsTotal];
     }
     score_canvas(p.score, 0, p.score.tau, p.score.budget, pass, status, rows_total,
                  carve_score(sm.ring, p.score.N), [&](int i, bool masked) {
-                     if (p.from_mask) return sm.map.scored(i) ? sm.map.rank(i) : -1;
+                     if (kind.from_mask()) return sm.map.scored(i) ? sm.map.rank(i) : -1;
                      const int q = p.score.q_of_pos[i];
                      return masked ? q : -1;
                  });
@@ -968,10 +980,12 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
 // The head kernel: one launch per projection pass, clusters of two CTAs, one CTA per SM.  It
 // compacts the mask (or reads the pass from the meta words), gathers and normalises the pass's
 // rows, contracts them with the head, merges the splits' statistics and scores a single canvas.
+template <bool kPlain>
 __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     k_head(const __grid_constant__ HeadMaps maps, const __grid_constant__ HeadParams p) {
     extern __shared__ uint8_t smem_raw[];
     const HeadSmem sm = carve_smem(smem_raw);
+    const StepKind<kPlain> kind{p};
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();
@@ -999,7 +1013,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
 
     PassInfo pass;
     int num_words = 0;
-    if (p.from_mask) {
+    if (kind.from_mask()) {
         const int masked = compact_mask(p.compact, sm.map, reinterpret_cast<int *>(sm.ring));
         num_words = (p.compact.B * p.compact.N + 31) >> 5;
         if (threadIdx.x == 32) {  // read after the mask
@@ -1007,7 +1021,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
             *sm.stale = ld_acquire(&p.meta[kMetaClosed]);
         }
         int lazy = 0;
-        if (p.compact.lazy) {  // which rows there are may depend on the plan
+        if (kind.lazy()) {  // which rows there are may depend on the plan
             if (warp == 0) {
                 lazy = choose_lazy(p.compact, p.plan, masked);
                 if (lane == 0) sm.map.pass->lazy = lazy;
@@ -1040,10 +1054,10 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
 
     if (warp >= 2) {
         first_row = __shfl_sync(0xffffffffu, first_row, 0);
-        gather_rows(p.norm, sm.map, num_words, pass.rows, pass.sel, pass.layer0, first_row,
+        gather_rows<kPlain>(p.norm, sm.map, num_words, pass.rows, pass.sel, pass.layer0, first_row,
                     rows_per_claim(pass.rows, gridDim.x * kSwapEpiWarps), p.meta, lane);
     }
-    if (p.from_mask) {  // the plan, from warp 0, which does not wait for the others
+    if (kind.from_mask()) {  // the plan, from warp 0, which does not wait for the others
         if (warp == 0) {
             __syncwarp();
             asm volatile("bar.arrive 1, %0;" ::"n"(kHeadKernelThreads) : "memory");
@@ -1052,7 +1066,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
             pass = *sm.map.pass;
             // for the kernels after this one, by the warp that gathered row 0 (or, without rows,
             // one of the first CTA)
-            if (publishes(p) && warp >= 2 &&
+            if (kind.publishes() && warp >= 2 &&
                 (pass.rows > 0 ? first_row == 0 : blockIdx.x == 0 && warp == 2)) {
                 publish_pass(p.compact, sm.map, lane);
                 __syncwarp();
@@ -1092,7 +1106,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     }
     __syncwarp();
     tc_fence_before_sync();
-    finish_pass(p, sm, pass);  // begins with a barrier of the CTA
+    finish_pass<kPlain>(p, sm, pass);  // begins with a barrier of the CTA
     cluster_sync();  // no signal may still be in flight to a CTA that is about to exit
     tc_fence_after_sync();
     if (warp == 1) {
@@ -1112,8 +1126,8 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
             p.meta[kMetaUnitsDone] = 0;
             p.meta[kMetaClosed] = 0;
             p.meta[kMetaExit] = 0;
-            if (p.last_pass) p.meta[kMetaScored] = 0;
-            if (p.last_pass) p.meta[kMetaStepStatus] = atomicExch(&p.meta[kMetaStatus], RPD_OK);
+            if (!kPlain && p.last_pass) p.meta[kMetaScored] = 0;
+            if (kPlain || p.last_pass) p.meta[kMetaStepStatus] = atomicExch(&p.meta[kMetaStatus], RPD_OK);
         }
     }
 }
@@ -1153,8 +1167,11 @@ cudaError_t opt_in_smem() {
     const int dev = current_device();
     if (dev < 0) return cudaErrorInvalidDevice;
     if (g_head_ready[dev].load(std::memory_order_acquire)) return cudaSuccess;
-    cudaError_t e = cudaFuncSetAttribute(k_head, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_head<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          kHeadKernelSmemBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_head<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kHeadKernelSmemBytes);
     if (e == cudaSuccess) g_head_ready[dev].store(1, std::memory_order_release);
     return e;
 }
@@ -1179,7 +1196,7 @@ int head_max_clusters() {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, k_head, &cfg) != cudaSuccess) n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, k_head<false>, &cfg) != cudaSuccess) n = 0;
     g_head_clusters[dev].store(n + 1, std::memory_order_release);
     return n;
 }
@@ -1206,7 +1223,9 @@ cudaError_t launch_head(const HeadMaps &maps, const HeadParams &p, int grid, cud
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = t_no_pdl ? 1 : 2;
-    return cudaLaunchKernelEx(&cfg, k_head, maps, p);
+    const bool plain = p.from_mask && p.score_canvas && !p.select_band && p.last_pass && p.compact.lazy == 0 &&
+                       !p.norm.sel_list && !p.merge.shard_out;
+    return cudaLaunchKernelEx(&cfg, plain ? k_head<true> : k_head<false>, maps, p);
 }
 
 }  // namespace rpd

@@ -34,7 +34,8 @@ __device__ __forceinline__ int merge_lanes(int splits) {
 // then the lanes combine in a fixed order (the result does not depend on which CTA merges).
 // `sel_list`: compact index of the pass's s-th position (null: s itself); `position`: canvas
 // position of a compact index (only for vocabulary shards).
-template <typename Position>
+// kPlain: no list and no shards.
+template <bool kPlain, typename Position>
 __device__ __forceinline__ void merge_block(const MergeArgs &mg, const PassInfo &pass,
                                             const int32_t *sel_list, int block, int gs,
                                             const int32_t *status, Position position) {
@@ -69,8 +70,8 @@ __device__ __forceinline__ void merge_block(const MergeArgs &mg, const PassInfo 
     if (valid && gl == 0) {
         const int kr = row / pass.sel;
         const int s = row - kr * pass.sel;
-        const int q = sel_list ? sel_list[s] : s;
-        if (mg.shard_out) {
+        const int q = !kPlain && sel_list ? sel_list[s] : s;
+        if (!kPlain && mg.shard_out) {
             mg.shard_out[static_cast<size_t>(pass.layer0 + kr) * mg.shard_stride + position(q)] =
                 make_float4(acc.m, acc.s, acc.t, __int_as_float(acc.a + mg.v_offset));
         } else {

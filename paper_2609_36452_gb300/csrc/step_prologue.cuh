@@ -234,7 +234,8 @@ __device__ __forceinline__ int rows_per_claim(int rows, int warps) {
 
 // Claim and gather rows of the pass until none is left, starting with the claim made before; one
 // warp.  Compact index -> position through `map`, or through the lists in global memory when
-// num_words is 0.  The rows are counted once the warp has no more of them.
+// num_words is 0 (never with kFromMask).  The rows are counted once the warp has no more of them.
+template <bool kFromMask>
 __device__ __forceinline__ void gather_rows(const NormParams &p, const MaskMap &map, int num_words,
                                             int rows, int sel, int layer0, int claim, int per_claim,
                                             int32_t *meta, int lane) {
@@ -243,7 +244,7 @@ __device__ __forceinline__ void gather_rows(const NormParams &p, const MaskMap &
         const int kr = r / sel;
         const int sr = r - kr * sel;
         int pos;
-        if (num_words > 0) {
+        if (kFromMask || num_words > 0) {
             pos = map.position(sr, num_words);
         } else {
             const int q = p.sel_list ? p.sel_list[sr] : sr;

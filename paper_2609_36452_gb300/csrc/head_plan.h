@@ -36,19 +36,21 @@ __host__ __device__ inline float bits_float(unsigned u) {
 #endif
 }
 
-// Smallest (time, g) over split counts g = g0, g0 + step, ... <= gmax of `tiles` x g work
-// units on `slots` persistent pairs: waves x tiles-per-unit x tile_cost, packed so that the
-// smaller key is the smaller time, then the smaller g.
+// Smallest (time, g) over split counts g <= gmax of `tiles` x g work units on `slots` persistent
+// pairs: waves x tiles-per-unit x tile_cost, packed so that the smaller key is the smaller time,
+// then the smaller g.  Of the counts with the same tiles per unit only the smallest can win.
 __host__ __device__ inline unsigned long long best_split_key(float tile_cost, int tiles, int slots,
-                                                             int num_n, int gmax, int g0, int step) {
+                                                             int num_n, int gmax) {
     unsigned long long key = ~0ull;
-    for (int g = g0; g <= gmax; g += step) {
+    for (int g = 1; g <= gmax;) {
         const int per = (num_n + g - 1) / g;
         const int waves = (tiles * g + slots - 1) / slots;
         const float cost = static_cast<float>(waves) * static_cast<float>(per) * tile_cost;
         const unsigned long long k = (static_cast<unsigned long long>(float_bits(cost)) << 20) |
                                      static_cast<unsigned>(g);
         key = k < key ? k : key;
+        if (per == 1) break;
+        g = (num_n + per - 2) / (per - 1);
     }
     return key;
 }
@@ -100,12 +102,12 @@ __host__ __device__ inline HeadPlan plan_head(long long rows, const HeadPlanInpu
     const int tiles2 = static_cast<int>((rows + kPairTileM - 1) / kPairTileM);
     const int gmax2 = in.num_n < in.max_splits ? in.num_n : in.max_splits;
     const unsigned long long key2 =
-        best_split_key(kPairTileCost, tiles2, in.pair_slots, in.num_n, gmax2, 1, 1);
+        best_split_key(kPairTileCost, tiles2, in.pair_slots, in.num_n, gmax2);
     const int gmax3 = in.num_n < in.max_splits / 2 ? in.num_n : in.max_splits / 2;
     const int groups = swap_groups(rows);
     const int ng = swap_group_rows(rows, groups);
     const unsigned long long key3 =
-        gmax3 > 0 ? best_split_key(swap_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax3, 1, 1)
+        gmax3 > 0 ? best_split_key(swap_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax3)
                   : ~0ull;
     return plan_from_keys(in, key2, key3, ng);
 }
@@ -132,12 +134,12 @@ inline HeadPlan regroup_plan(const HeadPlan &plan, long long rows, const HeadPla
         return plan;
     const int tiles2 = static_cast<int>((rows + kPairTileM - 1) / kPairTileM);
     unsigned long long best = best_split_key(1.f, tiles2, in.pair_slots, in.num_n,
-                                             in.num_n < in.max_splits ? in.num_n : in.max_splits, 1, 1);
+                                             in.num_n < in.max_splits ? in.num_n : in.max_splits);
     HeadPlan chosen{kHeadModePair, static_cast<int>(best & 0xFFFFFull), 0, plan.est};
     for (int groups = swap_groups(rows); groups <= kRegroupMaxGroups; ++groups) {
         const int ng = swap_group_rows(rows, groups);
         const unsigned long long key =
-            best_split_key(group_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax, 1, 1);
+            best_split_key(group_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax);
         if (key >> 20 >= best >> 20) continue;
         best = key;
         chosen = HeadPlan{kHeadModeRowsN, 2 * static_cast<int>(key & 0xFFFFFull), ng, plan.est};
@@ -170,9 +172,10 @@ inline HeadPlan split_tail(const HeadPlan &plan, long long rows, const HeadPlanI
 }
 
 // The kernel argument with the plans of every pass of up to kStepPlanRows rows; `plan(rows)`.
+// (rows past max_rows, a multiple of 32, do not occur.)
 template <typename Plan>
-inline void fill_step_plan(StepPlan &p, Plan plan) {
-    for (int i = 0; i < kStepPlanRows / 32; ++i) {
+inline void fill_step_plan(StepPlan &p, int max_rows, Plan plan) {
+    for (int i = 0; i < kStepPlanRows / 32 && 32 * i < max_rows; ++i) {
         const HeadPlan hp = plan(32 * (i + 1));
         p.splits[i] = hp.mode == kHeadModeRowsN ? -hp.splits : hp.splits;
         p.swap_rows[i] = static_cast<uint16_t>(hp.swap_rows);

@@ -193,18 +193,18 @@ int build_plan(rpd_ctx *c) {
     const int gmax2 = std::min(in.num_n, in.max_splits);
     const int gmax3 = std::min(in.num_n, in.max_splits / 2);
     const int entries = plan_entries(c->cap_rows);
-    std::vector<HeadPlan> table(static_cast<size_t>(std::max(entries, kStepPlanRows + 1)));
-    std::vector<unsigned long long> key2(std::max(c->cap_rows, kStepPlanRows) / kPairTileM + 1, 0ull);
+    std::vector<HeadPlan> table(static_cast<size_t>(entries));
+    std::vector<unsigned long long> key2(c->cap_rows / kPairTileM + 1, 0ull);
     std::vector<std::vector<unsigned long long>> key3;  // [groups][ng / step]
     HeadPlan regrouped{};
-    for (int i = 0; i < static_cast<int>(table.size()); ++i) {
+    for (int i = 0; i < entries; ++i) {
         const int r = i <= kPlanRows ? i : kPlanRows + (i - kPlanRows) * kPairTileM;
         if (r == 0 || in.pair_slots <= 0) {
             table[i] = plan_head(r, in);
             continue;
         }
         const int tiles2 = (r + kPairTileM - 1) / kPairTileM;
-        if (!key2[tiles2]) key2[tiles2] = best_split_key(kPairTileCost, tiles2, in.pair_slots, in.num_n, gmax2, 1, 1);
+        if (!key2[tiles2]) key2[tiles2] = best_split_key(kPairTileCost, tiles2, in.pair_slots, in.num_n, gmax2);
         const int groups = swap_groups(r);
         const int ng = swap_group_rows(r, groups);
         unsigned long long k3 = ~0ull;
@@ -213,7 +213,7 @@ int build_plan(rpd_ctx *c) {
             std::vector<unsigned long long> &row = key3[groups];
             const int slot = ng / kSwapRowStep;
             if (static_cast<int>(row.size()) <= slot) row.resize(slot + 1, 0ull);
-            if (!row[slot]) row[slot] = best_split_key(swap_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax3, 1, 1);
+            if (!row[slot]) row[slot] = best_split_key(swap_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax3);
             k3 = row[slot];
         }
         table[i] = plan_from_keys(in, key2[tiles2], k3, ng);
@@ -222,7 +222,7 @@ int build_plan(rpd_ctx *c) {
             table[i] = regrouped;
         }
     }
-    fill_step_plan(c->step_plan, [&](int r) { return table[r]; });
+    fill_step_plan(c->step_plan, c->cap_rows, [&](int r) { return table[r]; });
     cudaError_t e = cudaMemcpy(c->plan, table.data(), static_cast<size_t>(entries) * sizeof(HeadPlan),
                                cudaMemcpyHostToDevice);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(plan table)");

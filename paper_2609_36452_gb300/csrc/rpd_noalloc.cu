@@ -159,7 +159,7 @@ StepPlan step_plan_for(DeviceSetup &dev, const HeadPlanInputs &in, int V, int d)
         if (s.V == V && s.d == d) return s.plan;
     ShapePlan &s = dev.plans[dev.next_plan];
     dev.next_plan = (dev.next_plan + 1) % kShapePlans;
-    fill_step_plan(s.plan, [&](int rows) { return split_tail(regroup_plan(plan_head(rows, in), rows, in), rows, in); });
+    fill_step_plan(s.plan, kNaMaxRows, [&](int rows) { return split_tail(regroup_plan(plan_head(rows, in), rows, in), rows, in); });
     s.V = V;
     s.d = d;
     return s.plan;

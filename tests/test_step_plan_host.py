@@ -1,5 +1,6 @@
 """The plans that a step passes to the head kernel (StepPlan, one entry per 32 rows) are those of
-every row count up to its limit, at the two models' heads, small and ragged ones (no GPU)."""
+every row count up to its limit, and the search over split counts finds what trying each of them
+does, at the two models' heads, small and ragged ones (no GPU)."""
 import os
 import shutil
 import subprocess
@@ -13,6 +14,17 @@ DRIVER = r"""
 #include "head_plan.h"
 #include <cstdio>
 #include <cstdlib>
+// every split count in turn
+static unsigned long long every_key(float cost1, int tiles, int slots, int num_n, int gmax) {
+    unsigned long long key = ~0ull;
+    for (int g = 1; g <= gmax; ++g) {
+        const int per = (num_n + g - 1) / g, waves = (tiles * g + slots - 1) / slots;
+        const float cost = static_cast<float>(waves) * static_cast<float>(per) * cost1;
+        const unsigned long long k = (static_cast<unsigned long long>(rpd::float_bits(cost)) << 20) | unsigned(g);
+        key = k < key ? k : key;
+    }
+    return key;
+}
 int main(int argc, char **argv) {
     const int V = atoi(argv[1]), d = atoi(argv[2]), sms = atoi(argv[3]), force = atoi(argv[4]);
     rpd::HeadPlanInputs in{};
@@ -24,7 +36,7 @@ int main(int argc, char **argv) {
     in.regroup = 1;
     auto plan = [&](int r) { return rpd::regroup_plan(rpd::plan_head(r, in), r, in); };
     rpd::StepPlan sp;
-    rpd::fill_step_plan(sp, plan);
+    rpd::fill_step_plan(sp, rpd::kStepPlanRows, plan);
     int bad = 0;
     for (int r = 1; r <= 4096; ++r) {  // regrouping keeps the plan's rules at every row count
         const rpd::HeadPlan a = plan(r);
@@ -42,6 +54,10 @@ int main(int argc, char **argv) {
         const int mode = sp.splits[i] < 0 ? rpd::kHeadModeRowsN : rpd::kHeadModePair;
         bad += a.mode != mode || a.splits != splits || a.swap_rows != sp.swap_rows[i] || a.est != sp.est[i];
     }
+    for (int tiles = 1; tiles <= 130; ++tiles)
+        for (int gmax = 1; gmax <= in.num_n && gmax <= in.max_splits; gmax = 3 * gmax + 1)
+            bad += every_key(0.914f, tiles, in.pair_slots, in.num_n, gmax) !=
+                   rpd::best_split_key(0.914f, tiles, in.pair_slots, in.num_n, gmax);
     std::printf("%d\n", bad);
     return 0;
 }

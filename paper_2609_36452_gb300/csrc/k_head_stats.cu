@@ -964,9 +964,12 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
     }
     if (!kind.scores()) return;
     int status = RPD_OK, rows_total = pass.rows;
+    if (threadIdx.x == kHeadKernelThreads - 1) {  // a thread with nothing to score on short canvases
+        *reinterpret_cast<volatile int32_t *>(&meta[kMetaClosed]) = 1;
+        __threadfence();  // and the scoring's barriers: before any mask byte changes
+    }
     if (threadIdx.x == 0) {
-        *reinterpret_cast<volatile int32_t *>(&meta[kMetaClosed]) = 1;  // before any mask byte changes
-        status = ld_acquire(&meta[kMetaStatus]);
+        status = *reinterpret_cast<volatile int32_t *>(&meta[kMetaStatus]);
         if (!kind.from_mask()) rows_total = meta[kMetaRowsTotal];
     }
     score_canvas(p.score, 0, p.score.tau, p.score.budget, pass, status, rows_total,

@@ -372,7 +372,6 @@ __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float 
         cnt.x += (f & kFlagCandidate) != 0;
         cnt.y += (f & (kFlagCandidate | kFlagHigh)) == (kFlagCandidate | kFlagHigh);
     }
-    if (threadIdx.x == 0) __threadfence();  // what the caller has stored comes before the commits
     const int4 tot = block_sum4(cnt, sm.sum);
     const int fallback_window = p.block > 0 ? p.block : p.window;
 

@@ -357,7 +357,7 @@ __device__ __forceinline__ int copy_ahead(const HeadParams &p, const HeadSmem &s
             tma_load_2d_pair(dst, w, bar, x, y);
     }
     if (!wait_for_rows(p, sm, rows, 0)) return -1;
-    proxy_fence();
+    proxy_fence_global();
     for (int s = 0; s < ahead; ++s)
         tma_load_2d_pair(sm.ring + s * c.stage_bytes + c.u_off, c.u,
                          full0 + static_cast<uint32_t>(s * sizeof(uint64_t)), s * kTileK, u_row);

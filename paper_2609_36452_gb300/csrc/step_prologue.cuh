@@ -273,7 +273,7 @@ __device__ __forceinline__ void gather_rows(const NormParams &p, const MaskMap &
         claim = __shfl_sync(0xffffffffu, next, 0);
     }
     if (done > 0) {
-        proxy_fence();  // u is read by TMA
+        proxy_fence_global();  // u is read by TMA
         __syncwarp();
         if (lane == 0) counter_add_release(&meta[kMetaRowsDone], done);
     }

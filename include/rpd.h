@@ -301,11 +301,12 @@ int rpd_step_shard_finish(rpd_ctx *ctx, const float *gathered, int P, uint8_t *m
 
 /* Per-kernel timing with CUDA events recorded on the context's stream around every
  * launch while enabled.  rpd_kernel_times synchronises the recorded events and returns,
- * for each of the RPD_NUM_KERNELS kernels (gather/norm, head statistics, merge,
- * score/commit; the compaction kernel is counted with gather/norm, and for a single canvas
- * of at most 2048 positions score/commit runs inside the step's last merge and is counted
- * with it), the summed milliseconds and the launch count since the last reset; reset
- * clears them. */
+ * for each of the RPD_NUM_KERNELS stages (gather/norm, head statistics, merge, score/commit), the
+ * summed milliseconds and the launch count since the last reset; reset clears them.  A head
+ * statistics launch gathers its rows, merges and, for a single canvas, scores and commits as well;
+ * the other stages count the launches that some batches have besides: the compaction (under
+ * gather/norm) and the selection of a second pass's positions (under merge) of batches of more
+ * than 8192 positions, and score/commit of several canvases. */
 #define RPD_NUM_KERNELS 4
 int rpd_profile_enable(rpd_ctx *ctx, int enable);
 int rpd_kernel_times(rpd_ctx *ctx, double *ms /*[RPD_NUM_KERNELS]*/,

@@ -11,18 +11,19 @@
 //   m = max x,  s = sum 2^(x-m),  t = sum 2^(x-m) (x-m),  a = argmax (lowest index).
 // Logits never reach global memory.  Each work unit is (row tile, contiguous range of
 // 256-wide vocabulary tiles); its statistics are written once per row as one partial
-// (float4) that the merge kernel combines.
+// (float4); the rows' partials are merged after the last unit (step_epilogue.cuh).
 //
-// One persistent kernel, launched as clusters of two CTAs (one per SM), serves two tilings;
-// the compaction kernel picks one per projection pass on the device and the kernel reads it
-// from the step's meta words.  Both run on CTA pairs (tcgen05 cta_group::2, M = 256):
+// One persistent kernel, launched as clusters of two CTAs (one per SM), serves two tilings.  Each
+// CTA counts the mask's set bits and looks the pass's plan up by its row count (or, for large
+// batches and second passes, reads both from the step's meta words).  Both tilings run on CTA
+// pairs (tcgen05 cta_group::2, M = 256):
 //   pair tiles:  256 rows (M, 128 per CTA) x 256 vocabulary entries (N);
 //   rows on N:   256 vocabulary entries (M, 128 per CTA) x a group of up to 512 rows (N,
 //                padded to a multiple of 32), so that a pass whose row count is not a multiple
 //                of 256 pads by at most 31 rows per group.
 // Roles: warp 0 TMA producer (one thread), warp 1 TMEM owner (512 columns) and MMA issuer
 // (the whole warp in the even CTA, one elected lane issuing), warps 2-9 epilogue (pair tiles
-// use warps 2-5).  Every wait is
+// use warps 2-5); before the contraction they gather the rows of u (step_prologue.cuh).  Every wait is
 // bounded; a timeout latches RPD_ERR_TIMEOUT in the step's status word and the CTA drains and
 // exits.
 #include <atomic>
@@ -428,8 +429,8 @@ __device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm,
 //
 // Barriers: full[s] lives in the even CTA and receives both CTAs' TMA completions (tx bytes
 // 64 KB per stage); empty[s], acc_full[a] and drain receive multicast commits from the MMA
-// thread in both CTAs; acc_empty[a] lives in the even CTA and counts the 4 epilogue warps
-// of both CTAs (8 arrivals).
+// thread in both CTAs; acc_empty[a] lives in the even CTA and counts two arrivals
+// from each of the 4 epilogue warps of both CTAs (16, as many as with rows on N).
 __device__ __forceinline__ void head_pair(const HeadParams &p, const HeadSmem &sm, const TileWalk &tw,
                                           int rows, int splits, bool tail, int num_kb, uint32_t tmem_base) {
     constexpr int kStageBytes = kPairStageBytesA + kPairStageBytesB;

@@ -38,14 +38,16 @@ UNIT = "commit-steps/s"
 
 # DRAM bytes (read + write) per head-statistics launch from ncu captures, keyed by workload
 # and by a hash of the kernel's sources at capture time; any source change makes it null.
-HEAD_SOURCES = ("paper_2609_36452_gb300/csrc/k_head_stats.cu", "paper_2609_36452_gb300/csrc/ptx.cuh",
-                "paper_2609_36452_gb300/csrc/rpd_internal.h", "paper_2609_36452_gb300/csrc/head_plan.h")
+HEAD_SOURCES = ("paper_2609_36452_gb300/csrc/k_head_stats.cu", "paper_2609_36452_gb300/csrc/step_prologue.cuh",
+                "paper_2609_36452_gb300/csrc/step_epilogue.cuh", "paper_2609_36452_gb300/csrc/step_common.cuh",
+                "paper_2609_36452_gb300/csrc/ptx.cuh", "paper_2609_36452_gb300/csrc/rpd_internal.h",
+                "paper_2609_36452_gb300/csrc/head_plan.h")
 HEAD_TRAFFIC = {
-    ("llada_first_step", "38d1ebfe76e73880"): 1.0519e9,
-    ("llada_tail_70_masked", "38d1ebfe76e73880"): 1.0551e9,
-    ("llada_tail_5_masked", "38d1ebfe76e73880"): 1.0404e9,
-    ("dream_mid_decode", "38d1ebfe76e73880"): 1.1035e9,
-    ("batched_serving", "38d1ebfe76e73880"): 8.8575e9,
+    ("llada_first_step", "78c13a764d5ef6b5"): 1.1114e9,
+    ("llada_tail_70_masked", "78c13a764d5ef6b5"): 1.0433e9,
+    ("llada_tail_5_masked", "78c13a764d5ef6b5"): 1.0395e9,
+    ("dream_mid_decode", "78c13a764d5ef6b5"): 1.1021e9,
+    ("batched_serving", "78c13a764d5ef6b5"): 9.5373e9,
 }
 
 # Nominal dense rates of GB300 (context only; the fractions use the measured peaks).

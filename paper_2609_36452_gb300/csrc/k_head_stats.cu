@@ -181,7 +181,6 @@ struct HeadSmem {
     uint32_t *tmem_slot;
     volatile int *abort_flag;
     volatile int *unit_ring;  // [kUnitRing] claimed unit indices
-    volatile int *stale;      // the canvas was already being scored when the mask was read
     MaskMap map;              // the compaction (and the pass) of this CTA
 };
 
@@ -203,14 +202,13 @@ __device__ __forceinline__ HeadSmem carve_smem(uint8_t *raw) {
     s.tmem_slot = reinterpret_cast<uint32_t *>(s.chunk_free + kTmemCols / 32);
     s.abort_flag = reinterpret_cast<volatile int *>(s.tmem_slot + 1);
     s.unit_ring = s.abort_flag + 1;
-    s.stale = s.unit_ring + kUnitRing;
     s.map.words = reinterpret_cast<uint32_t *>(base + kHeadRegionBytes + kHeadBarrierBytes);
     s.map.before = reinterpret_cast<uint16_t *>(s.map.words + kMaskWords);
     s.map.pass = reinterpret_cast<PassInfo *>(s.map.before + kMaskWords + 8);
     return s;
 }
 
-static_assert((2 * kSwapMaxStages + 6 + 2 * kUnitRing + kTmemCols / 32) * 8 + 12 + 4 * kUnitRing <=
+static_assert((2 * kSwapMaxStages + 6 + 2 * kUnitRing + kTmemCols / 32) * 8 + 8 + 4 * kUnitRing <=
                   kHeadBarrierBytes,
               "barrier region");
 
@@ -238,7 +236,6 @@ __device__ __forceinline__ void init_barriers(const HeadSmem &sm) {
     mbar_init(sm.epi, 32 * kSwapEpiWarps);
     mbar_init(sm.drain, 1);
     *sm.abort_flag = 0;
-    *sm.stale = 0;
     fence_mbar_init();
 }
 
@@ -870,13 +867,12 @@ struct StepKind {
 // is done before the epilogue is); `blocks` if there is nothing to merge.  Only running CTAs hold
 // units, so the wait ends whatever part of the grid is resident.  It also ends when a CTA has
 // given up (the step's outputs are then meaningless), and after the time in which a unit's own
-// waits would have run out.  A CTA that came so late that the canvas was already being scored
-// claims nothing.
+// waits would have run out.
 template <bool kPlain>
 __device__ __forceinline__ int claim_merge(const HeadParams &p, const HeadSmem &sm, const PassInfo &pass,
                                            int blocks) {
     int32_t *meta = p.meta;
-    if (blocks == 0 || *sm.stale) return blocks;
+    if (blocks == 0) return blocks;
     const int block = atomicAdd(&meta[kMetaMergeNext], 1);
     if (block >= blocks) return blocks;
     const bool pair = pass.mode == kHeadModePair;
@@ -919,7 +915,7 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
         if (*sm.abort_flag) atomicExch(&meta[kMetaStatus], RPD_ERR_TIMEOUT);
         share[0] = first;
         // nothing to merge: the first CTA goes on
-        share[1] = blocks == 0 && blockIdx.x == 0 && !*sm.stale && (kPlain || !meta[kMetaScored]);
+        share[1] = blocks == 0 && blockIdx.x == 0 && (kPlain || !meta[kMetaScored]);
     }
     __syncthreads();
     const int num_words = kind.from_mask() ? (p.compact.B * p.compact.N + 31) >> 5 : 0;
@@ -966,8 +962,10 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
     if (!kind.scores()) return;
     int status = RPD_OK, rows_total = pass.rows;
     if (threadIdx.x == kHeadKernelThreads - 1) {  // a thread with nothing to score on short canvases
-        *reinterpret_cast<volatile int32_t *>(&meta[kMetaClosed]) = 1;
-        __threadfence();  // and the scoring's barriers: before any mask byte changes
+        // The scoring's barriers lie between this and the first mask byte that changes.
+        const bool all = !kind.from_mask() || ld_acquire(&meta[kMetaMaskRead]) == static_cast<int>(gridDim.x);
+        share[2] = all;
+        if (!all) meta[kMetaClearLater] = 1;
     }
     if (threadIdx.x == 0) {
         status = *reinterpret_cast<volatile int32_t *>(&meta[kMetaStatus]);
@@ -978,7 +976,8 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
                      if (kind.from_mask()) return sm.map.scored(i) ? sm.map.rank(i) : -1;
                      const int q = p.score.q_of_pos[i];
                      return masked ? q : -1;
-                 });
+                 },
+                 [&] { return share[2] != 0; });
 }
 
 // The head kernel: one launch per projection pass, clusters of two CTAs, one CTA per SM.  It
@@ -1020,10 +1019,10 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     if (kind.from_mask()) {
         const int masked = compact_mask(p.compact, sm.map, reinterpret_cast<int *>(sm.ring));
         num_words = (p.compact.B * p.compact.N + 31) >> 5;
-        if (threadIdx.x == 32) {  // read after the mask
-            __threadfence();
-            *sm.stale = ld_acquire(&p.meta[kMetaClosed]);
-        }
+        // Every CTA of the grid works its pass out of the same mask, also one that starts when the
+        // others are done (kernels of other streams may hold some of the SMs): the canvas is scored
+        // without waiting for it, but no bit is cleared before all have been counted here.
+        if (threadIdx.x == 32) counter_add_release(&p.meta[kMetaMaskRead], 1);
         int lazy = 0;
         if (kind.lazy()) {  // which rows there are may depend on the plan
             if (warp == 0) {
@@ -1118,22 +1117,27 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         tmem_dealloc_pair(tmem_base, kTmemCols);
     }
     // The last CTA of the grid leaves the counters at zero for the next pass.
+    int clear_later = 0;
     if (threadIdx.x == 0) {
         __threadfence();
         if (atomicAdd(&p.meta[kMetaExit], 1) == static_cast<int>(gridDim.x) - 1) {
             __threadfence();
+            if (kind.from_mask() && kind.scores()) clear_later = *reinterpret_cast<volatile int32_t *>(&p.meta[kMetaClearLater]);
             p.meta[kMetaUnitNext] = 0;
             p.meta[kMetaRowNext] = 0;
             p.meta[kMetaMergeNext] = 0;
             p.meta[kMetaMergeDone] = 0;
             p.meta[kMetaRowsDone] = 0;
             p.meta[kMetaUnitsDone] = 0;
-            p.meta[kMetaClosed] = 0;
+            p.meta[kMetaMaskRead] = 0;
+            p.meta[kMetaClearLater] = 0;
             p.meta[kMetaExit] = 0;
             if (!kPlain && p.last_pass) p.meta[kMetaScored] = 0;
             if (kPlain || p.last_pass) p.meta[kMetaStepStatus] = atomicExch(&p.meta[kMetaStatus], RPD_OK);
         }
     }
+    if (kind.from_mask() && kind.scores() && warp == 0 && __shfl_sync(0xffffffffu, clear_later, 0))
+        clear_committed(p.score, lane);
 }
 
 // The tiled copy of the head: thread i writes 16-byte vector i of Wt, which is vector k8 of

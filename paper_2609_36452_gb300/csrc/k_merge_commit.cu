@@ -88,7 +88,8 @@ __global__ void __launch_bounds__(kScoreThreads, 1) k_score_commit(const __grid_
                  [q_of_pos](int i, bool masked) {
                      const int q = q_of_pos[i];  // loaded with the mask byte
                      return masked ? q : -1;
-                 });
+                 },
+                 [] { return true; });
 }
 
 }  // namespace

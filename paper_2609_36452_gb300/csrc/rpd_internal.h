@@ -91,11 +91,13 @@ enum MetaIndex : int {
     kMetaMergeNext = 13, // next block of rows to merge (claimed by the head kernel's CTAs)
     kMetaExit = 14,      // CTAs of the head kernel that are done; the last one zeroes the counters
     kMetaStepStatus = 15,// the step's status, published when its last head kernel ends
-    kMetaClosed = 16,    // the canvas is being scored: the mask no longer describes the pass
+    kMetaClearLater = 16,// the canvas was scored before every CTA had read its mask: the last CTA to
+                         // leave clears the committed bits
     kMetaScored = 17,    // the first of two passes scored the canvas: nothing is left for the second
     // counts that the head kernel's CTAs wait for, on a line of their own
     kMetaRowsDone = 32,  // gathered rows of the pass
     kMetaUnitsDone = 33, // head work units whose partials are written, counted by each epilogue warp
+    kMetaMaskRead = 48,  // CTAs of the head kernel that have read the mask
     kMetaWords = 64
 };
 

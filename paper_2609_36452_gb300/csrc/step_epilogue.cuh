@@ -229,12 +229,12 @@ constexpr int kLayerBatch = 4;  // window layers whose statistics are loaded tog
 //   committed mask bits.  RPD-block skips the budget and takes the fallback over the active
 //   block.
 // `compact_index(i)`: compact index of canvas position i, negative if it is not scored (called
-// with the position's mask byte).  The merged row statistics are read through L2 (ld.cg): other
+// with the position's mask byte).  `clear()`: whether the committed mask bits are cleared here.  The merged row statistics are read through L2 (ld.cg): other
 // CTAs of the same grid may have written them.
-template <typename CompactIndex>
+template <typename CompactIndex, typename Clear>
 __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float tau, float beta,
                                              const PassInfo &pass, int status, int rows_total,
-                                             const ScoreSmem &sm, CompactIndex compact_index) {
+                                             const ScoreSmem &sm, CompactIndex compact_index, Clear clear) {
     const int N = p.N, K = p.K;
     const int nmt = pass.masked;
     const bool lazy_on = pass.lazy != 0;  // earlier layers exist only in the band
@@ -396,6 +396,7 @@ __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float 
     }
 
     // ------------------------------------------------------------------------- outputs
+    const bool clear_now = clear();
 #pragma unroll 1
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         const size_t pos = static_cast<size_t>(b) * N + i;
@@ -403,7 +404,7 @@ __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float 
         p.out_commit[pos] = commit ? 1 : 0;
         if (commit) {
             p.out_token[pos] = sm.y[i];
-            mask[i] = 0;
+            if (clear_now) mask[i] = 0;
         }
     }
     if (threadIdx.x == 0) {
@@ -419,6 +420,13 @@ __device__ __forceinline__ void score_canvas(const ScoreParams &p, int b, float 
         st.n_rows = rows_total;
         p.out_stats[b] = st;
     }
+}
+
+// The mask bits that score_canvas left (of a single canvas); one warp.
+__device__ __forceinline__ void clear_committed(const ScoreParams &p, int lane) {
+#pragma unroll 4
+    for (int i = lane; i < p.N; i += 32)
+        if (__ldcg(p.out_commit + i)) p.mask[i] = 0;
 }
 
 }  // namespace

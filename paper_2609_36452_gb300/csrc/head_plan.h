@@ -8,6 +8,7 @@
 // critical path.
 #pragma once
 
+#include <cmath>
 #include <cstring>
 
 #include "rpd_internal.h"
@@ -37,15 +38,16 @@ __host__ __device__ inline float bits_float(unsigned u) {
 }
 
 // Smallest (time, g) over split counts g <= gmax of `tiles` x g work units on `slots` persistent
-// pairs: waves x tiles-per-unit x tile_cost, packed so that the smaller key is the smaller time,
-// then the smaller g.  Of the counts with the same tiles per unit only the smallest can win.
+// pairs: waves x (tiles-per-unit x tile_cost + unit_cost), packed so that the smaller key is the
+// smaller time, then the smaller g.  Of the counts with the same tiles per unit only the smallest can win.
 __host__ __device__ inline unsigned long long best_split_key(float tile_cost, int tiles, int slots,
-                                                             int num_n, int gmax) {
+                                                             int num_n, int gmax, float unit_cost = 0.f) {
     unsigned long long key = ~0ull;
     for (int g = 1; g <= gmax;) {
         const int per = (num_n + g - 1) / g;
         const int waves = (tiles * g + slots - 1) / slots;
-        const float cost = static_cast<float>(waves) * static_cast<float>(per) * tile_cost;
+        const float cost = static_cast<float>(waves) * static_cast<float>(per) * tile_cost +
+                           static_cast<float>(waves) * unit_cost;
         const unsigned long long k = (static_cast<unsigned long long>(float_bits(cost)) << 20) |
                                      static_cast<unsigned>(g);
         key = k < key ? k : key;
@@ -118,13 +120,27 @@ __host__ __device__ inline HeadPlan plan_head(long long rows, const HeadPlanInpu
 // tiles' time, at groups that share the head's tiles through L2 (measured with 2 to 6 groups of
 // 96 to 512 rows at the LLaDA head, d = 4096; in the power-limited steady state, where the clock
 // follows the work, the differences are larger: 1068 rows 732 us with pair tiles, 704 with groups of 224).
-__host__ __device__ inline float group_tile_cost(int ng) {
+//
+// The table is of d = 4096.  A tile's contraction grows with d, its epilogue does not, and that of a
+// row group (which transposes its logits) costs more than a pair tile's: groups of 224 and 288 rows
+// against pair tiles took 1.49, 1.40, 1.33, 1.22, 1.21, 1.09 times the table at d = 64, 128, 256, 512,
+// 1024, 2048, which 0.08 per halving of d follows.  With the table alone 1088 rows of d = 64 at the
+// LLaDA vocabulary took 122 us in groups, which pair tiles do in 90.
+inline float group_tile_cost(int ng, int d) {
     // groups of 32, 64, ..., 512 rows
     constexpr float kCost[kSwapMaxRows / kSwapRowStep] = {0.70f, 0.70f, 0.72f, 0.74f, 0.79f, 0.85f,
                                                           0.94f, 1.05f, 1.22f, 1.41f, 1.57f, 1.68f,
                                                           1.95f, 2.05f, 2.16f, 2.30f};
-    return kCost[ng / kSwapRowStep - 1];
+    const float shallow = d < 4096 ? 1.f + 0.08f * std::log2(4096.f / static_cast<float>(d)) : 1.f;
+    return kCost[ng / kSwapRowStep - 1] * shallow;
 }
+// What a unit of either tiling costs beside its tiles (the partials, and with row groups the
+// combination of the sub-partitions and its barriers): about 1.2 and 3.2 us whatever the depth, in
+// pair tiles' time, which is 21.5 us at d = 4096 and no less than 2.25 us.  Without it 1216 rows of
+// d = 1024 and 8192 entries took 36.7 us in groups (32.1 in pair tiles), and 1568 rows of d = 256 at the
+// LLaDA vocabulary 189 us in 247 ranges of two pair tiles (136 in 21 ranges).
+inline float unit_cost(float at_4096, int d) { return at_4096 * std::fmin(4096.f / static_cast<float>(d), 9.5f); }
+constexpr float kPairUnitCost = 0.055f, kGroupUnitCost = 0.15f;
 // Up to 2048 rows: with more, pair tiles' padding is under an eighth.
 constexpr int kRegroupMaxGroups = 8;
 
@@ -135,12 +151,14 @@ inline HeadPlan regroup_plan(const HeadPlan &plan, long long rows, const HeadPla
         return plan;
     const int tiles2 = static_cast<int>((rows + kPairTileM - 1) / kPairTileM);
     unsigned long long best = best_split_key(1.f, tiles2, in.pair_slots, in.num_n,
-                                             in.num_n < in.max_splits ? in.num_n : in.max_splits);
+                                             in.num_n < in.max_splits ? in.num_n : in.max_splits,
+                                             unit_cost(kPairUnitCost, in.d));
     HeadPlan chosen{kHeadModePair, static_cast<int>(best & 0xFFFFFull), 0, plan.est};
     for (int groups = swap_groups(rows); groups <= kRegroupMaxGroups; ++groups) {
         const int ng = swap_group_rows(rows, groups);
         const unsigned long long key =
-            best_split_key(group_tile_cost(ng), groups, in.pair_slots, in.num_n, gmax);
+            best_split_key(group_tile_cost(ng, in.d), groups, in.pair_slots, in.num_n, gmax,
+                           unit_cost(kGroupUnitCost, in.d));
         if (key >> 20 >= best >> 20) continue;
         best = key;
         chosen = HeadPlan{kHeadModeRowsN, 2 * static_cast<int>(key & 0xFFFFFull), ng, plan.est};
@@ -185,6 +203,12 @@ inline void fill_step_plan(StepPlan &p, int max_rows, Plan plan) {
         p.swap_rows[i] = static_cast<uint16_t>(hp.swap_rows);
         p.est[i] = hp.est;
     }
+}
+
+// The plan of a pass from plan_head's (a function of the multiple of 32 rows).
+inline HeadPlan refine_plan(const HeadPlan &plan, long long rows, const HeadPlanInputs &in) {
+    if (rows > static_cast<long long>(kRegroupMaxGroups) * kPairTileM) return plan;
+    return split_tail(regroup_plan(plan, rows, in), rows, in);
 }
 
 #ifdef __CUDACC__

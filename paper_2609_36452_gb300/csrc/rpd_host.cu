@@ -175,6 +175,7 @@ HeadPlanInputs plan_inputs(const rpd_ctx *c) {
     in.hbm_tiles = head_stream_in_tiles(c->V, c->d, c->num_sms);
     in.force = c->tiling;
     in.regroup = 1;
+    in.d = c->d;
     return in;
 }
 
@@ -196,7 +197,7 @@ int build_plan(rpd_ctx *c) {
     std::vector<HeadPlan> table(static_cast<size_t>(entries));
     std::vector<unsigned long long> key2(c->cap_rows / kPairTileM + 1, 0ull);
     std::vector<std::vector<unsigned long long>> key3;  // [groups][ng / step]
-    HeadPlan regrouped{};
+    HeadPlan refined{};
     for (int i = 0; i < entries; ++i) {
         const int r = i <= kPlanRows ? i : kPlanRows + (i - kPlanRows) * kPairTileM;
         if (r == 0 || in.pair_slots <= 0) {
@@ -218,8 +219,8 @@ int build_plan(rpd_ctx *c) {
         }
         table[i] = plan_from_keys(in, key2[tiles2], k3, ng);
         if (r <= kRegroupMaxGroups * kPairTileM) {  // a function of the multiple of 32 rows
-            if (r % kSwapRowStep == 1) regrouped = split_tail(regroup_plan(table[i], r, in), r, in);
-            table[i] = regrouped;
+            if (r % kSwapRowStep == 1) refined = refine_plan(table[i], r, in);
+            table[i] = refined;
         }
     }
     fill_step_plan(c->step_plan, c->cap_rows, [&](int r) { return table[r]; });

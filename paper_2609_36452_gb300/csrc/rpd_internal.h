@@ -122,6 +122,7 @@ struct HeadPlanInputs {
     float hbm_tiles;  // time to stream the head once, in tile units
     int force;        // RPD_TILING_*
     int regroup;      // also weigh more, smaller row groups (regroup_plan)
+    int d;            // hidden size
 };
 // Pair tiles whose last, partly filled wave is issued as half tiles (split_tail).
 constexpr int kSplitTail = 1;

@@ -159,7 +159,7 @@ StepPlan step_plan_for(DeviceSetup &dev, const HeadPlanInputs &in, int V, int d)
         if (s.V == V && s.d == d) return s.plan;
     ShapePlan &s = dev.plans[dev.next_plan];
     dev.next_plan = (dev.next_plan + 1) % kShapePlans;
-    fill_step_plan(s.plan, kNaMaxRows, [&](int rows) { return split_tail(regroup_plan(plan_head(rows, in), rows, in), rows, in); });
+    fill_step_plan(s.plan, kNaMaxRows, [&](int rows) { return refine_plan(plan_head(rows, in), rows, in); });
     s.V = V;
     s.d = d;
     return s.plan;
@@ -243,7 +243,7 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
     {
         // the plans of all row counts fit the kernel argument: no table (it would have to be allocated)
         const HeadPlanInputs plan_in{num_n, splits, pair_slots,
-                                     head_stream_in_tiles(V, d, dev->num_sms), RPD_TILING_AUTO, 1};
+                                     head_stream_in_tiles(V, d, dev->num_sms), RPD_TILING_AUTO, 1, d};
         HeadParams hp{};
         hp.compact = CompactParams{mask, q_of_pos, pos_of_q, canvas_off, meta, 1, N, K,
                                    nullptr, 0, rule.block, 0};

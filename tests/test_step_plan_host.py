@@ -34,6 +34,12 @@ int main(int argc, char **argv) {
     in.hbm_tiles = rpd::head_stream_in_tiles(V, d, sms);
     in.force = force;
     in.regroup = 1;
+    in.d = d;
+    if (argc > 5) {  // one pass's plan
+        const rpd::HeadPlan a = rpd::refine_plan(rpd::plan_head(atoi(argv[5]), in), atoi(argv[5]), in);
+        std::printf("%d %d %d\n", a.mode, a.splits, a.swap_rows);
+        return 0;
+    }
     auto plan = [&](int r) { return rpd::regroup_plan(rpd::plan_head(r, in), r, in); };
     rpd::StepPlan sp;
     rpd::fill_step_plan(sp, rpd::kStepPlanRows, plan);
@@ -86,3 +92,26 @@ def driver(tmp_path_factory):
 def test_one_entry_per_32_rows_is_exact(driver, V, d, sms, force):
     out = subprocess.run([driver, str(V), str(d), str(sms), str(force)], capture_output=True, text=True, check=True)
     assert int(out.stdout) == 0
+
+
+# Measured on GB300 (us a pass over every row of the head, in the steady state of a second of them):
+# V, d, rows, in pair tiles, in several row groups.
+MEASURED = [(126464, 64, 1088, 89.5, 121.9), (126464, 256, 1344, 119.8, 149.1), (126464, 512, 672, 82.8, 93.1),
+            (126464, 1024, 1152, 197.2, 224.4), (126464, 3072, 1568, 796.1, 758.1), (126464, 4096, 1088, 741.7, 708.8),
+            (152064, 3584, 896, 647.9, 624.0), (152064, 3584, 1088, 782.9, 754.5), (32000, 128, 1568, 48.6, 58.9),
+            (32000, 512, 1344, 51.6, 59.3), (32000, 1024, 832, 48.2, 54.9), (32000, 2048, 576, 67.1, 62.9),
+            (32000, 4096, 576, 123.7, 111.3), (8192, 128, 1472, 24.5, 34.1), (8192, 512, 1216, 27.9, 33.9),
+            (8192, 1024, 1216, 32.1, 36.7), (8192, 4096, 1152, 68.3, 64.3), (8192, 4096, 1472, 75.4, 80.0)]
+
+
+@pytest.mark.parametrize("V,d,rows,pair,groups", MEASURED)
+def test_row_groups_where_they_were_measured_faster(driver, V, d, rows, pair, groups):
+    out = subprocess.run([driver, str(V), str(d), "152", "0", str(rows)], capture_output=True, text=True, check=True)
+    mode = int(out.stdout.split()[0])
+    assert mode == (3 if groups < pair else 2)
+
+
+def test_ranges_of_two_tiles_are_not_taken_for_a_wave_saved(driver):
+    """1568 rows at V 126464: 247 ranges leave no pair idle, but took 189 us at d = 256 where 21 take 136."""
+    out = subprocess.run([driver, "126464", "256", "152", "0", "1568"], capture_output=True, text=True, check=True)
+    assert out.stdout.split()[:2] == ["2", "21"]

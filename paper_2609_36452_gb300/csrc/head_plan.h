@@ -167,10 +167,17 @@ inline HeadPlan regroup_plan(const HeadPlan &plan, long long rows, const HeadPla
 }
 
 // Pair tiles in whole waves over the CTA pairs and a rest of at most half a wave: the rest runs as
-// half tiles (128 vocabulary entries), two to a tile, in about half a wave.  Each row then has two
-// partials per vocabulary tile, which the scratch must hold.  One of eight slices of the LLaDA
-// head, 748 rows: 186 tiles on 76 pairs took three waves, 74.4 us, and take 73.7; a small head (192
-// rows, 16 tiles) 22.5 and 20.7.
+// half tiles (128 vocabulary entries), two to a tile, in about half a wave.  Every whole tile is then a
+// unit of its own, and each row has two partials per vocabulary tile, which the scratch must hold
+// (heads of up to 38912 entries on 152 SMs) and the merge must read.
+//
+// That pays where nothing but the rest is left to run: 200 rows over 20 and 30 tiles take 33.4 and 25.9
+// us whole, 29.8 and 23.2 halved (d = 4096 and 2048; at d = 128, where a tile is mostly epilogue, 15.2 and
+// 15.3).  After whole waves the units and partials cost most of what half a wave saves, or more:
+//   d = 4096, several row tiles, 2.1 and 2.5 waves: 70.7 -> 68.6, 75.2 -> 74.3 us; 3.4 and 5.3 waves: 90.5 ->
+//   92.4, 141.9 -> 144.8; one row tile (bound by reading the head), 1.4 waves: 53.5 -> 54.4;
+//   d = 2048, 2.5 and 7.4 waves: 45.2 -> 45.8, 98.0 -> 104.4;  d = 512, 2.4 and 4.1: 26.8 -> 29.8, 33.0 -> 38.6;
+//   d = 128, 2.5 and 7.4: 23.2 -> 25.3, 35.9 -> 49.2.
 struct TailSplit {
     int whole, units;  // tiles in whole waves; work units in all
 };
@@ -178,9 +185,7 @@ __host__ __device__ inline TailSplit tail_split(int tiles, int pairs) {
     const int rest = tiles % pairs;
     return TailSplit{tiles - rest, tiles + rest};
 }
-// Half a wave saved of more than eight is under 6 % of the pass, and every row pays for two partials
-// a vocabulary tile in the merge instead of one a split.
-constexpr int kTailMaxWaves = 8;
+constexpr int kTailAfterWavesDepth = 4096;  // from this d on also after up to two whole waves
 
 inline HeadPlan split_tail(const HeadPlan &plan, long long rows, const HeadPlanInputs &in) {
     if (!in.regroup || in.force != RPD_TILING_AUTO || plan.mode != kHeadModePair || in.pair_slots <= 0 ||
@@ -188,8 +193,8 @@ inline HeadPlan split_tail(const HeadPlan &plan, long long rows, const HeadPlanI
         return plan;
     const long long tiles = (rows + kPairTileM - 1) / kPairTileM * in.num_n;
     const int rest = static_cast<int>(tiles % in.pair_slots);
-    if (tiles > static_cast<long long>(kTailMaxWaves) * in.pair_slots || rest == 0 || 2 * rest > in.pair_slots)
-        return plan;
+    const bool after_waves = in.d >= kTailAfterWavesDepth && rows > kPairTileM && tiles < 3ll * in.pair_slots;
+    if (rest == 0 || 2 * rest > in.pair_slots || (tiles >= in.pair_slots && !after_waves)) return plan;
     return HeadPlan{kHeadModePair, 2 * in.num_n, kSplitTail, plan.est};
 }
 

@@ -104,14 +104,21 @@ def test_two_pass_steps_one_after_another(N, projection, tau, prefix):
         runner.close()
 
 
-@pytest.mark.parametrize("V,N", [(4100, 200),    # under half a wave: only half tiles, the last one empty
-                                 (20480, 200),   # one wave and four tiles
-                                 (19713, 300),   # two row tiles, a last half tile of one entry
-                                 (9728, 600)])   # three row tiles of 38: one wave and a half exactly
-def test_pair_tiles_with_a_split_tail(V, N):
+@pytest.mark.parametrize("V,N,d", [(4100, 200, 128),    # under half a wave: only half tiles, the last one empty
+                                   (9728, 200, 128),    # half a wave exactly
+                                   (20480, 200, 128),   # one wave and four tiles: whole tiles only at this depth,
+                                   (19713, 300, 128),   # here too
+                                   (9728, 600, 128),    # and here
+                                   (20480, 400, 4096),  # two waves and eight tiles of two row tiles
+                                   (19713, 500, 4096),  # two waves and four tiles, a last half tile of one entry
+                                   (15872, 748, 4096)]) # three row tiles of 62: two waves and 34 tiles
+def test_pair_tiles_with_a_split_tail(V, N, d):
     """Whole waves of pair tiles and a rest of half tiles, whose rows have two partials per tile."""
-    K, d = 1, 128
-    W, g, hidden = make(800 + N, K, N, d, V)
+    K = 1
+    w_std = 0.08 if d < 1024 else 0.02
+    W, g = WL.make_head(V, d, 800 + N, w_std=w_std)
+    hidden = WL.make_hidden(W, K, N, 1800 + N, WL.u_profile(N, 0.5, 3.0), WL.calibrated_sigma(V, d, w_std, 3.0),
+                            flip_frac=0.1).hidden
     mask = torch.ones(N, dtype=torch.uint8)
     ref = O.rpd_step(bits(hidden), mask.numpy(), bits(g), bits(W), 1e-6, 0.9, 1.0, "llada")
     runner = DeviceRunner(W, g, K)

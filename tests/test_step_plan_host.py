@@ -115,3 +115,18 @@ def test_ranges_of_two_tiles_are_not_taken_for_a_wave_saved(driver):
     """1568 rows at V 126464: 247 ranges leave no pair idle, but took 189 us at d = 256 where 21 take 136."""
     out = subprocess.run([driver, "126464", "256", "152", "0", "1568"], capture_output=True, text=True, check=True)
     assert out.stdout.split()[:2] == ["2", "21"]
+
+
+# The same for the last wave of pair tiles: V, d, rows, us with whole tiles throughout, us with its half tiles.
+TAILS = [(5120, 4096, 200, 33.4, 29.8), (7680, 2048, 200, 25.9, 23.2), (5120, 1024, 200, 20.1, 18.6),
+         (20480, 4096, 400, 70.7, 68.6), (24064, 4096, 400, 74.5, 73.4), (15872, 4096, 748, 75.2, 74.3),
+         (28160, 128, 200, 20.0, 21.0), (28160, 4096, 200, 53.5, 54.4), (20480, 128, 400, 22.8, 24.4),
+         (24064, 1024, 400, 31.1, 32.4), (24064, 2048, 400, 45.2, 45.8), (15872, 128, 748, 23.6, 26.4),
+         (15872, 1024, 748, 31.5, 33.4), (26880, 512, 748, 33.0, 38.6), (35840, 128, 1000, 35.9, 49.2),
+         (35840, 2048, 1000, 98.0, 104.4), (34560, 4096, 748, 141.9, 144.8), (32000, 4096, 480, 90.5, 92.4)]
+
+
+@pytest.mark.parametrize("V,d,rows,whole,halved", TAILS)
+def test_half_tiles_where_they_were_measured_faster(driver, V, d, rows, whole, halved):
+    out = subprocess.run([driver, str(V), str(d), "152", "0", str(rows)], capture_output=True, text=True, check=True)
+    assert (out.stdout.split()[2] == "1") == (halved < whole)

@@ -40,6 +40,7 @@ UNIT = "commit-steps/s"
 # and by a hash of the kernel's sources at capture time; any source change makes it null.
 HEAD_SOURCES = ("paper_2609_36452_gb300/csrc/k_head_stats.cu", "paper_2609_36452_gb300/csrc/step_prologue.cuh",
                 "paper_2609_36452_gb300/csrc/step_epilogue.cuh", "paper_2609_36452_gb300/csrc/step_common.cuh",
+                "paper_2609_36452_gb300/csrc/step_counters.h",
                 "paper_2609_36452_gb300/csrc/ptx.cuh", "paper_2609_36452_gb300/csrc/rpd_internal.h",
                 "paper_2609_36452_gb300/csrc/head_plan.h")
 HEAD_TRAFFIC = {

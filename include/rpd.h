@@ -333,7 +333,8 @@ int rpd_kernel_times(rpd_ctx *ctx, double *ms /*[RPD_NUM_KERNELS]*/,
  * All calls on a device share the one scratch array, which keeps the previous call's
  * contents (the step's count/status words are zero again at the end of every call): calls
  * whose GPU work overlaps - concurrent host threads or different streams - race on it, so
- * order them on one stream.  The first call on each device finds the array's device address
+ * order them on one stream (calls that overlapped all the same have meaningless results; later
+ * ones are not affected).  The first call on each device finds the array's device address
  * (cudaGetSymbolAddress) and caches it; make that first call before any stream capture. */
 int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, int V, int K, float eps,
                      const rpd_rule *rule, const void *hidden, uint8_t *mask, int N, float tau,

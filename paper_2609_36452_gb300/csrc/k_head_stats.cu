@@ -30,6 +30,7 @@
 
 #include "ptx.cuh"
 #include "rpd_internal.h"
+#include "step_counters.h"
 #include "step_epilogue.cuh"
 #include "step_prologue.cuh"
 
@@ -980,6 +981,13 @@ __device__ __forceinline__ void finish_pass(const HeadParams &p, const HeadSmem 
                  [&] { return share[2] != 0; });
 }
 
+// The counters in global memory.
+struct DeviceWords {
+    int32_t *meta;
+    __device__ unsigned inc_wrap(int i, unsigned top) { return atomicInc(reinterpret_cast<unsigned *>(&meta[i]), top); }
+    __device__ void zero(int i) { meta[i] = 0; }
+};
+
 // The head kernel: one launch per projection pass, clusters of two CTAs, one CTA per SM.  It
 // compacts the mask (or reads the pass from the meta words), gathers and normalises the pass's
 // rows, contracts them with the head, merges the splits' statistics and scores a single canvas.
@@ -1120,18 +1128,11 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     int clear_later = 0;
     if (threadIdx.x == 0) {
         __threadfence();
-        if (atomicAdd(&p.meta[kMetaExit], 1) == static_cast<int>(gridDim.x) - 1) {
+        DeviceWords words{p.meta};
+        if (last_to_leave(words, gridDim.x)) {
             __threadfence();
             if (kind.from_mask() && kind.scores()) clear_later = *reinterpret_cast<volatile int32_t *>(&p.meta[kMetaClearLater]);
-            p.meta[kMetaUnitNext] = 0;
-            p.meta[kMetaRowNext] = 0;
-            p.meta[kMetaMergeNext] = 0;
-            p.meta[kMetaMergeDone] = 0;
-            p.meta[kMetaRowsDone] = 0;
-            p.meta[kMetaUnitsDone] = 0;
-            p.meta[kMetaMaskRead] = 0;
-            p.meta[kMetaClearLater] = 0;
-            p.meta[kMetaExit] = 0;
+            zero_counters(words);
             if (!kPlain && p.last_pass) p.meta[kMetaScored] = 0;
             if (kPlain || p.last_pass) p.meta[kMetaStepStatus] = atomicExch(&p.meta[kMetaStatus], RPD_OK);
         }

@@ -21,7 +21,8 @@
 // head tile also reads the rows of the compact head operand past the call's live row count
 // (left over from an earlier call, or zero), and its epilogue discards what those rows
 // produce.  Calls whose work overlaps on the GPU (two host threads, or two streams) race on
-// the arena: serialise them (one stream, or events).
+// the arena: serialise them (one stream, or events).  Such calls' results are meaningless; later ones
+// are not affected (step_counters.h).
 //
 // Set-up: the first call on each device looks up the arena's device address with
 // cudaGetSymbolAddress (the array's name in host code is only a host-side stand-in, not a

@@ -4,7 +4,7 @@
 // head kernel compacts the mask itself (step_prologue.cuh).
 //
 // k_compact (one CTA): order-preserving compaction of mask[B][N] into compact indices
-//   q = 0..NMT-1 (canvas-major, then position), per-canvas offsets, the projected row
+//   q = 0..NMT-1 (canvas-major, then position), the projected row
 //   count R = K*NMT and the head kernel's tiling plan.  Nothing goes back to the host: later
 //   kernels read these words from device memory.
 #include "ptx.cuh"
@@ -17,10 +17,7 @@ namespace {
 constexpr int kCompactThreads = 1024;
 constexpr int kCompactItems = 4;
 
-// At most 48 registers a thread: the CTA then needs 48 K of an SM's 64 K registers, so it can
-// start (launched early, waiting on its predecessor) beside one CTA of the previous step's merge
-// instead of waiting for an SM to empty.
-__global__ void __maxnreg__(48) k_compact(CompactParams p) {
+__global__ void __launch_bounds__(kCompactThreads, 1) k_compact(CompactParams p) {
     __shared__ int warp_sum[32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     __shared__ int block_lo[kMaxBatch];  // RPD-block: first position of each canvas's active block
@@ -66,7 +63,6 @@ __global__ void __maxnreg__(48) k_compact(CompactParams p) {
         for (int j = 0; j < kCompactItems; ++j) {
             const int i = i0 + j;
             if (i < total) {
-                if (i % p.N == 0) p.canvas_off[i / p.N] = excl;
                 p.q_of_pos[i] = f[j] ? excl : -1;
                 if (f[j]) p.pos_of_q[excl] = i;
                 excl += f[j];
@@ -106,7 +102,6 @@ __global__ void __maxnreg__(48) k_compact(CompactParams p) {
     const long long rows = lazy_on ? static_cast<long long>(carry) : all_rows;
     const int mode = plan.mode, splits = plan.splits, swap_rows = plan.swap_rows;
     if (tid == 0) {
-        p.canvas_off[p.B] = carry;
         p.meta[kMetaSwapRows] = swap_rows;
         p.meta[kMetaMasked] = carry;
         p.meta[kMetaRows] = static_cast<int>(rows);

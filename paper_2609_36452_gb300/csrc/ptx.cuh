@@ -299,23 +299,10 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 }
 
 // D (M=256 split over the pair's TMEM) (+)= A (rows split over the pair's shared memory) *
-// B^T (columns split over the pair's shared memory); issued by the even CTA of the pair.
-__device__ __forceinline__ void umma_bf16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
-                                               uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n"
-        " .reg .pred p;\n"
-        " setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same MMA issued from a converged warp: every lane calls it with the same operands and
-// elect.sync picks the issuing lane inside the asm block.  Keeping the whole warp in the
-// issuing loop (rather than one lane under a lane-dependent branch) keeps the operands in
-// uniform registers; measured on GB300, a one-lane loop with a barrier wait per stage took
+// B^T (columns split over the pair's shared memory); issued by the even CTA of the pair from a
+// converged warp: every lane calls it with the same operands and elect.sync picks the issuing
+// lane inside the asm block.  Keeping the whole warp in the issuing loop (rather than one lane
+// under a lane-dependent branch) keeps the operands in uniform registers; measured on GB300, a one-lane loop with a barrier wait per stage took
 // 143 cycles per K-step for N = 32 MMAs and 198 for a 256 + 32 pair, the converged warp 74
 // and 173 (the MMAs' own cost).  elect.sync over the full warp picks the same lane every
 // time, so the commits below track the MMAs issued here.
@@ -332,7 +319,8 @@ __device__ __forceinline__ void umma_bf16_pair_warp(uint32_t d_tmem, uint64_t a_
         : "memory");
 }
 
-// Commit (below) from the elected lane of a converged warp.
+// Arrive once on the mbarrier at the same shared-memory offset in every CTA of `cta_mask` when all
+// tcgen05.mma issued so far by the elected lane have completed; from a converged warp.
 __device__ __forceinline__ void umma_commit_pair_multicast_warp(uint64_t *bar, uint16_t cta_mask) {
     asm volatile(
         "{\n"
@@ -341,16 +329,6 @@ __device__ __forceinline__ void umma_commit_pair_multicast_warp(uint64_t *bar, u
         " @e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
         " [%0], %1;\n"
         "}\n" ::"r"(smem_u32(bar)),
-        "h"(cta_mask)
-        : "memory");
-}
-
-// Arrive once on the mbarrier at the same shared-memory offset in every CTA of `cta_mask`
-// when all tcgen05.mma issued so far by this thread have completed.
-__device__ __forceinline__ void umma_commit_pair_multicast(uint64_t *bar, uint16_t cta_mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
-        " [%0], %1;" ::"r"(smem_u32(bar)),
         "h"(cta_mask)
         : "memory");
 }

@@ -116,7 +116,7 @@ struct rpd_ctx {
     float4 *partials = nullptr;
     int32_t *row_arg = nullptr;
     float *row_pmax = nullptr, *row_H = nullptr;
-    int32_t *q_of_pos = nullptr, *pos_of_q = nullptr, *canvas_off = nullptr, *meta = nullptr;
+    int32_t *q_of_pos = nullptr, *pos_of_q = nullptr, *meta = nullptr;
     HeadPlan *plan = nullptr;  // head-tiling plans by pass row count, rows 0..plan_rows
     int plan_rows = 0;
     StepPlan step_plan{};      // the same for few rows, passed to the head kernel
@@ -151,7 +151,7 @@ struct rpd_ctx {
 
     void free_scratch() {
         void *ptrs[] = {u, inv_rms, partials, row_arg, row_pmax, row_H, q_of_pos, pos_of_q,
-                        canvas_off, meta, sel_q, plan};
+                        meta, sel_q, plan};
         for (void *p : ptrs)
             if (p) cudaFree(p);
         u = nullptr;
@@ -159,7 +159,7 @@ struct rpd_ctx {
         partials = nullptr;
         row_arg = nullptr;
         row_pmax = row_H = nullptr;
-        q_of_pos = pos_of_q = canvas_off = meta = sel_q = nullptr;
+        q_of_pos = pos_of_q = meta = sel_q = nullptr;
         plan = nullptr;
         cap_bn = cap_b = cap_rows = plan_rows = 0;
     }
@@ -260,7 +260,6 @@ int ensure_scratch(rpd_ctx *c, int B, int N) {
         {reinterpret_cast<void **>(&c->q_of_pos), static_cast<size_t>(new_bn) * 4},
         {reinterpret_cast<void **>(&c->pos_of_q), static_cast<size_t>(new_bn) * 4},
         {reinterpret_cast<void **>(&c->sel_q), static_cast<size_t>(new_bn) * 4},
-        {reinterpret_cast<void **>(&c->canvas_off), static_cast<size_t>(new_b + 1) * 4},
         {reinterpret_cast<void **>(&c->meta), kMetaWords * 4},
         {reinterpret_cast<void **>(&c->plan),
          static_cast<size_t>(plan_entries(static_cast<int>(rows))) * sizeof(HeadPlan)},
@@ -377,7 +376,7 @@ BatchScoreParams batch_score_params(const ScoreParams &sp, const float *tau, con
 
 // The compaction of a step's mask; `lazy` as in CompactParams.
 CompactParams compact_params(const rpd_ctx *c, const uint8_t *mask, int B, int N, int lazy) {
-    return CompactParams{mask, c->q_of_pos, c->pos_of_q, c->canvas_off, c->meta, B, N, c->K,
+    return CompactParams{mask, c->q_of_pos, c->pos_of_q, c->meta, B, N, c->K,
                          c->plan, c->plan_rows, c->rule.block, lazy};
 }
 

@@ -144,7 +144,6 @@ struct CompactParams {
     const uint8_t *mask;  // [B*N]
     int32_t *q_of_pos;    // [B*N] compact index or -1
     int32_t *pos_of_q;    // [B*N] flat position b*N+i of compact index q
-    int32_t *canvas_off;  // [B+1]
     int32_t *meta;        // [kMetaWords]
     int B, N, K;
     const HeadPlan *plan; // the context's tables (table_plan)

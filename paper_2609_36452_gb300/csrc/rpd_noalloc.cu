@@ -63,8 +63,7 @@ constexpr size_t kOffRowPmax = kOffRowArg + kNaMaxRows * 4;
 constexpr size_t kOffRowH = kOffRowPmax + kNaMaxRows * 4;
 constexpr size_t kOffQofPos = kOffRowH + kNaMaxRows * 4;
 constexpr size_t kOffPosOfQ = kOffQofPos + kNaMaxN * 4;
-constexpr size_t kOffCanvasOff = kOffPosOfQ + kNaMaxN * 4;
-constexpr size_t kOffMeta = kOffCanvasOff + 256;
+constexpr size_t kOffMeta = kOffPosOfQ + kNaMaxN * 4;
 constexpr size_t kArenaBytes = kOffMeta + 256;
 
 static __device__ __align__(256) uint8_t g_noalloc_arena[kArenaBytes];
@@ -219,7 +218,6 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
     float *row_H = reinterpret_cast<float *>(A + kOffRowH);
     int32_t *q_of_pos = reinterpret_cast<int32_t *>(A + kOffQofPos);
     int32_t *pos_of_q = reinterpret_cast<int32_t *>(A + kOffPosOfQ);
-    int32_t *canvas_off = reinterpret_cast<int32_t *>(A + kOffCanvasOff);
     int32_t *meta = reinterpret_cast<int32_t *>(A + kOffMeta);
 
     // Same head-kernel configuration as rpd_step (tiling chosen on the device).
@@ -246,7 +244,7 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
         const HeadPlanInputs plan_in{num_n, splits, pair_slots,
                                      head_stream_in_tiles(V, d, dev->num_sms), RPD_TILING_AUTO, 1, d};
         HeadParams hp{};
-        hp.compact = CompactParams{mask, q_of_pos, pos_of_q, canvas_off, meta, 1, N, K,
+        hp.compact = CompactParams{mask, q_of_pos, pos_of_q, meta, 1, N, K,
                                    nullptr, 0, rule.block, 0};
         hp.plan = step_plan_for(*dev, plan_in, V, d);
         hp.norm = NormParams{static_cast<const __nv_bfloat16 *>(hidden),

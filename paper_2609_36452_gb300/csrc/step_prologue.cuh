@@ -152,8 +152,7 @@ __device__ __forceinline__ bool choose_lazy(const CompactParams &p, const StepPl
     return e_fin + e_band < e_all;
 }
 
-// What the kernels after this one read of the compaction: the maps, the canvases' offsets and
-// the pass; one warp.
+// What the kernels after this one read of the compaction: the maps and the pass; one warp.
 __device__ __forceinline__ void publish_pass(const CompactParams &p, const MaskMap &map, int lane) {
     const PassInfo &pass = *map.pass;
     const int total = p.B * p.N;
@@ -162,10 +161,8 @@ __device__ __forceinline__ void publish_pass(const CompactParams &p, const MaskM
         const bool on = map.scored(i);
         p.q_of_pos[i] = on ? q : -1;
         if (on) p.pos_of_q[q] = i;
-        if (i % p.N == 0) p.canvas_off[i / p.N] = q;
     }
     if (lane == 0) {
-        p.canvas_off[p.B] = pass.masked;
         p.meta[kMetaMasked] = pass.masked;
         p.meta[kMetaRows] = pass.rows;
         p.meta[kMetaRowsTotal] = pass.rows;

@@ -1075,13 +1075,14 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         } else {
             asm volatile("bar.sync 1, %0;" ::"n"(kHeadKernelThreads) : "memory");
             pass = *sm.map.pass;
-            // for the kernels after this one, by the warp that gathered row 0 (or, without rows,
-            // one of the first CTA)
-            if (kind.publishes() && warp >= 2 &&
-                (pass.rows > 0 ? first_row == 0 : blockIdx.x == 0 && warp == 2)) {
-                publish_pass(p.compact, sm.map, lane);
-                __syncwarp();
-                if (lane == 0) counter_add_release(&p.meta[kMetaUnitsDone], 1);
+            if (kind.publishes() && warp >= 2) {
+                publish_maps(p.compact, sm.map, (blockIdx.x * kSwapEpiWarps + warp - 2) * 32 + lane,
+                             gridDim.x * kSwapEpiWarps * 32);
+                // the pass: by the warp that gathered row 0 (or, without rows, one of the first CTA)
+                if (lane == 0 && (pass.rows > 0 ? first_row == 0 : blockIdx.x == 0 && warp == 2)) {
+                    publish_pass(p.compact, pass);
+                    counter_add_release(&p.meta[kMetaUnitsDone], 1);
+                }
             }
         }
     }

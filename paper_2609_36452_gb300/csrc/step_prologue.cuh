@@ -152,27 +152,30 @@ __device__ __forceinline__ bool choose_lazy(const CompactParams &p, const StepPl
     return e_fin + e_band < e_all;
 }
 
-// What the kernels after this one read of the compaction: the maps and the pass; one warp.
-__device__ __forceinline__ void publish_pass(const CompactParams &p, const MaskMap &map, int lane) {
-    const PassInfo &pass = *map.pass;
+// What the kernels after this one read of the compaction.  The maps: every warp of the grid writes
+// its share (positions first, first + step, ...), and the grid's end is all that their readers wait
+// for.  By one warp, which the merge waited for, the maps of 8192 positions took some 25 us of a step.
+__device__ __forceinline__ void publish_maps(const CompactParams &p, const MaskMap &map, int first, int step) {
     const int total = p.B * p.N;
-    for (int i = lane; i < total; i += 32) {
+    for (int i = first; i < total; i += step) {
         const int q = map.rank(i);
         const bool on = map.scored(i);
         p.q_of_pos[i] = on ? q : -1;
         if (on) p.pos_of_q[q] = i;
     }
-    if (lane == 0) {
-        p.meta[kMetaMasked] = pass.masked;
-        p.meta[kMetaRows] = pass.rows;
-        p.meta[kMetaRowsTotal] = pass.rows;
-        p.meta[kMetaSel] = pass.sel;
-        p.meta[kMetaLayer0] = pass.layer0;
-        p.meta[kMetaLazy] = pass.lazy;
-        p.meta[kMetaHeadMode] = pass.mode;
-        p.meta[kMetaSplits] = pass.splits;
-        p.meta[kMetaSwapRows] = pass.swap_rows;
-    }
+}
+
+// The pass, by one thread of the grid; the second pass's takes its place after the merge.
+__device__ __forceinline__ void publish_pass(const CompactParams &p, const PassInfo &pass) {
+    p.meta[kMetaMasked] = pass.masked;
+    p.meta[kMetaRows] = pass.rows;
+    p.meta[kMetaRowsTotal] = pass.rows;
+    p.meta[kMetaSel] = pass.sel;
+    p.meta[kMetaLayer0] = pass.layer0;
+    p.meta[kMetaLazy] = pass.lazy;
+    p.meta[kMetaHeadMode] = pass.mode;
+    p.meta[kMetaSplits] = pass.splits;
+    p.meta[kMetaSwapRows] = pass.swap_rows;
 }
 
 // bf16(a * b) of both halves, one rounding (the product of two bf16 is exact in fp32).

@@ -130,3 +130,32 @@ def test_pair_tiles_with_a_split_tail(V, N, d):
         runner.close()
     compare_step(ref, got)
     compare_step(ref, whole)
+
+
+def test_maps_of_many_positions_hold_up_no_step():
+    """The compaction's maps (for the kernels after the head kernel) are written by the whole grid:
+    8192 positions cost a step a few us more than 64 with as many masked (25 us by a single warp)."""
+    K, d, V = 1, 64, 1024
+    W, g, _ = make(5, K, 8, d, V)
+    runner = DeviceRunner(W, g, K)
+    runner.ctx.set_vocab_shard(0, V)
+    try:
+        times = []
+        for N in (64, 8192):
+            hidden = torch.zeros(K, N, d, dtype=torch.bfloat16, device="cuda")
+            mask = torch.zeros(N, dtype=torch.uint8, device="cuda")
+            mask[:32] = 1
+            out = torch.zeros(K, N, 4, device="cuda")
+            best = 1e9
+            for _ in range(30):
+                t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                t0.record()
+                for _ in range(20):
+                    runner.ctx.step_shard_partials(hidden, mask, out)
+                t1.record()
+                t1.synchronize()
+                best = min(best, t0.elapsed_time(t1) / 20 * 1e3)
+            times.append(best)
+    finally:
+        runner.close()
+    assert times[1] < times[0] + 12, times

@@ -2,8 +2,8 @@
 // descriptors and the launch sequence of one commit step.
 //
 // Step = k_head (compaction, gather, contraction, merge and, for a single canvas, score and
-// commit), sized from device-resident counts (nothing is read back mid-step).  Several canvases
-// are scored by k_score_commit; batches of more than kFusedMaxPositions positions are compacted
+// commit), sized from device-resident counts (nothing is read back mid-step).  Several canvases, and
+// a long one, are scored by k_score_commit; batches of more than kFusedMaxPositions positions are compacted
 // by k_compact first.  Lazy projection runs a second k_head, over positions that the first one
 // selects (k_band after k_compact).  Scratch is owned by the context and sized for the largest B*N seen.
 #include <cuda.h>
@@ -460,9 +460,9 @@ int run_step(rpd_ctx *c, const void *hidden, uint8_t *mask, int B, int N, const 
     if (e != cudaSuccess) return cuda_fail(e, "compaction launch");
 
     // Scoring, scan and commit: by the step's last head kernel for a single canvas (one launch
-    // fewer), by k_score_commit for several.
+    // fewer), by k_score_commit for several and for long ones.
     const ScoreParams sp = score_params(c, mask, B, N, tau, budget, out_commit, out_token, out_stats);
-    const bool fuse_score = B == 1;
+    const bool fuse_score = B == 1 && N <= kFuseScoreMaxN;
 
     // One projection pass: the head kernel (gather + RMSNorm prologue, head statistics, merge).
     const MergeArgs mg{c->partials, c->max_splits, c->row_arg, c->row_pmax, c->row_H};

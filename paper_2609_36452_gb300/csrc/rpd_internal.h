@@ -70,6 +70,11 @@ constexpr int kMaxBatch = 128;
 constexpr int kMaxCanvas = 8192;
 static_assert(kMaxCanvas <= kFusedMaxPositions, "a single canvas never needs k_compact");
 constexpr int kScoreThreads = 1024;
+// Longest canvas that the head kernel scores itself.  Its 320 threads take 3.2 times as many turns, each
+// a trip to L2 for the rows' statistics, as k_score_commit's 1024, which cost a launch of 1.5 to 2 us:
+// half masked, d = 256, V = 4096, K = 2: 1024 positions 27.8 us here, 27.6 there; 2048: 36.9, 35.2;
+// 4096: 49.9, 46.4; 8192: 91.0, 78.5.  With 5 masked: 1024 20.5, 22.6; 2048 22.4, 22.6; 8192 30.8, 29.0.
+constexpr int kFuseScoreMaxN = 2048;
 constexpr uint64_t kWaitLimitNs = 2000000000ull;  // bounded mbarrier waits: 2 s
 constexpr long long kBandBytes = 32ll << 20;       // u tiles a band of head work units re-reads
 

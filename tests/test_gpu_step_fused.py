@@ -159,3 +159,28 @@ def test_maps_of_many_positions_hold_up_no_step():
     finally:
         runner.close()
     assert times[1] < times[0] + 12, times
+
+
+@pytest.mark.parametrize("B,N,projection,launches", [
+    (1, 256, "all", 1), (1, 2048, "all", 1), (1, 256, "lazy", 2), (1, 256, "auto", 2),  # everything in the head kernel
+    (1, 2049, "all", 2), (1, 8192, "lazy", 3),   # a long canvas, and several, are scored apart
+    (8, 1024, "all", 2), (8, 1024, "lazy", 3),
+    (9, 911, "all", 3), (9, 911, "lazy", 5)])    # more positions than the head kernel compacts: also compaction, band
+def test_kernels_launched_by_a_step(B, N, projection, launches):
+    K, d, V = 2, 64, 512
+    W, g = WL.make_head(V, d, 3, w_std=0.08)
+    gen = torch.Generator().manual_seed(N)
+    hidden = torch.randn(K, B, N, d, generator=gen).to(torch.bfloat16) * 2
+    masks = torch.stack([WL.uniform_fraction_mask(N, 0.3, 20 + b) for b in range(B)])
+    runner = DeviceRunner(W, g, K)
+    try:
+        runner.ctx.set_projection(projection)
+        runner.ctx.profile(True)
+        got = runner.step_batched(hidden, masks, [0.9] * B, [1.5] * B)
+        count = sum(n for _, n in runner.ctx.kernel_times().values())
+    finally:
+        runner.close()
+    assert count == launches
+    for b in {0, B - 1}:
+        ref = O.rpd_step(bits(hidden[:, b].contiguous()), masks[b].numpy(), bits(g), bits(W), 1e-6, 0.9, 1.5, "llada")
+        compare_step(ref, got[b], lazy=projection != "all" and got[b]["stats"]["n_rows"] < K * int(masks.sum()))

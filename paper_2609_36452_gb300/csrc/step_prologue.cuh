@@ -190,40 +190,55 @@ __device__ __forceinline__ float add_squares(uint32_t h, float ss) {
     return fmaf(hi, hi, fmaf(lo, lo, ss));
 }
 
-constexpr int kVecPerLane = 4;  // 16-byte vectors of the row a lane has in registers at a time
+constexpr int kVecPerLane = 4;  // 16-byte vectors of a row a lane has in registers at a time
 
-// Row r of the pass from `src`; one warp.  The row was prefetched into L2 at once and is walked in
-// short steps: this code runs a few times per launch on instructions that the previous step's
-// stream through L2 has evicted, and as one unrolled block (16 KB of them) it took 10 us a row,
-// nearly all of it instruction fetches.
-__device__ __forceinline__ void gather_row(const NormParams &p, int r, const uint4 *__restrict__ src,
+// Rows r .. r + kRows - 1 of the pass from `src` (null: left out, the first is there); one warp.  The
+// rows were prefetched into L2 and are walked in short steps: this code runs a few times per launch on
+// instructions that the previous step's stream through L2 has evicted, and as one unrolled block (16 KB
+// of them) it took 10 us a row, nearly all of it instruction fetches.
+template <int kRows>
+__device__ __forceinline__ void gather_row(const NormParams &p, int r, const uint4 *const (&src)[kRows],
                                            int lane) {
     const int nvec = p.d >> 3;  // 8 bf16 per 16-byte vector
     const uint4 *__restrict__ gvec = reinterpret_cast<const uint4 *>(p.gain);
     uint4 *__restrict__ dst = reinterpret_cast<uint4 *>(p.u + static_cast<size_t>(r) * p.d);
-    float ss = 0.f;
+    float ss[kRows];
+#pragma unroll
+    for (int i = 0; i < kRows; ++i) ss[i] = 0.f;
 #pragma unroll 1
     for (int v0 = lane; v0 < nvec; v0 += 32 * kVecPerLane) {
-        uint4 hv[kVecPerLane], gv[kVecPerLane];
+        uint4 hv[kRows][kVecPerLane], gv[kVecPerLane];
 #pragma unroll
         for (int j = 0; j < kVecPerLane; ++j) {
             const int v = v0 + 32 * j;
-            if (v < nvec) hv[j] = __ldcs(src + v);
+#pragma unroll
+            for (int i = 0; i < kRows; ++i)
+                if (v < nvec && (i == 0 || src[i])) hv[i][j] = __ldcs(src[i] + v);
             if (v < nvec) gv[j] = __ldg(gvec + v);
         }
 #pragma unroll
-        for (int j = 0; j < kVecPerLane; ++j) {
-            const int v = v0 + 32 * j;
-            if (v >= nvec) break;
-            ss = add_squares(hv[j].w, add_squares(hv[j].z, add_squares(hv[j].y, add_squares(hv[j].x, ss))));
-            // g*h of two bf16 values rounded once to bf16 (reading D1)
-            dst[v] = make_uint4(mul_bf16x2(hv[j].x, gv[j].x), mul_bf16x2(hv[j].y, gv[j].y),
-                                mul_bf16x2(hv[j].z, gv[j].z), mul_bf16x2(hv[j].w, gv[j].w));
+        for (int i = 0; i < kRows; ++i) {
+            if (i > 0 && !src[i]) break;
+#pragma unroll
+            for (int j = 0; j < kVecPerLane; ++j) {
+                const int v = v0 + 32 * j;
+                if (v >= nvec) break;
+                const uint4 h = hv[i][j];
+                ss[i] = add_squares(h.w, add_squares(h.z, add_squares(h.y, add_squares(h.x, ss[i]))));
+                // g*h of two bf16 values rounded once to bf16 (reading D1)
+                dst[i * static_cast<size_t>(nvec) + v] =
+                    make_uint4(mul_bf16x2(h.x, gv[j].x), mul_bf16x2(h.y, gv[j].y),
+                               mul_bf16x2(h.z, gv[j].z), mul_bf16x2(h.w, gv[j].w));
+            }
         }
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-    if (lane == 0) p.inv_rms[r] = 1.0f / sqrtf(ss / static_cast<float>(p.d) + p.eps);
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < kRows; ++i) ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], o);
+#pragma unroll
+    for (int i = 0; i < kRows; ++i)
+        if (lane == i && (i == 0 || src[i])) p.inv_rms[r + i] = 1.0f / sqrtf(ss[i] / static_cast<float>(p.d) + p.eps);
 }
 
 // Rows a warp claims at a time: one while every warp of the grid can have its own, several (each
@@ -234,40 +249,64 @@ __device__ __forceinline__ int rows_per_claim(int rows, int warps) {
 
 // Claim and gather rows of the pass until none is left, starting with the claim made before; one
 // warp.  Compact index -> position through `map`, or through the lists in global memory when
-// num_words is 0 (never with kFromMask).  The rows are counted once the warp has no more of them.
-template <bool kFromMask>
+// num_words is 0.  The rows are counted once the warp has no more of them.
+//
+// kPlain: the plain step, of few rows: one at a time.  The general kernel, whose batches have tens of
+// thousands, finds the positions of a claim's rows in as many lanes and keeps two rows in flight: one
+// after another a row took a warp 0.78 us of waiting.
+template <bool kPlain>
 __device__ __forceinline__ void gather_rows(const NormParams &p, const MaskMap &map, int num_words,
                                             int rows, int sel, int layer0, int claim, int per_claim,
                                             int32_t *meta, int lane) {
     const int nvec = p.d >> 3;
-    auto source = [&](int r) -> const uint4 * {  // and its prefetch; null if out of bounds
+    auto source = [&](int r) -> const uint4 * {  // null if out of bounds
         const int kr = r / sel;
         const int sr = r - kr * sel;
         int pos;
-        if (kFromMask || num_words > 0) {
+        if (kPlain || num_words > 0) {
             pos = map.position(sr, num_words);
         } else {
             const int q = p.sel_list ? p.sel_list[sr] : sr;
             pos = rpd_check(q >= 0 && q < p.BN, meta + kMetaStatus) ? p.pos_of_q[q] : -1;
         }
         if (!rpd_check(pos >= 0 && pos < p.BN, meta + kMetaStatus)) return nullptr;
-        const uint4 *src = reinterpret_cast<const uint4 *>(
-            p.hidden + (static_cast<size_t>(layer0 + kr) * p.BN + pos) * p.d);
+        return reinterpret_cast<const uint4 *>(p.hidden + (static_cast<size_t>(layer0 + kr) * p.BN + pos) * p.d);
+    };
+    auto prefetch = [&](const uint4 *src) {
+        if (!src) return;
 #pragma unroll 1
         for (int v = lane * 8; v < nvec; v += 32 * 8) asm volatile("prefetch.global.L2 [%0];" ::"l"(src + v));
-        return src;
     };
     int done = 0;
     while (claim * per_claim < rows) {
         const int r0 = claim * per_claim, r1 = min(rows, r0 + per_claim);
         int next = 0;
         if (lane == 0) next = atomicAdd(&meta[kMetaRowNext], 1);  // its latency hides behind the rows
-        const uint4 *src = source(r0);
+        if (kPlain) {
+            const uint4 *src[1] = {source(r0)};
+            prefetch(src[0]);
 #pragma unroll 1
-        for (int r = r0; r < r1; ++r) {
-            const uint4 *ahead = r + 1 < r1 ? source(r + 1) : nullptr;
-            if (src) gather_row(p, r, src, lane);  // warp-uniform
-            src = ahead;
+            for (int r = r0; r < r1; ++r) {
+                const uint4 *ahead = r + 1 < r1 ? source(r + 1) : nullptr;
+                prefetch(ahead);
+                if (src[0]) gather_row<1>(p, r, src, lane);  // warp-uniform
+                src[0] = ahead;
+            }
+        } else {
+            const uint4 *mine = lane < r1 - r0 ? source(r0 + lane) : nullptr;  // at most 8 rows
+            auto of = [&](int r) {  // of row r, in every lane
+                const unsigned long long a = __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(mine), (r - r0) & 31);
+                return reinterpret_cast<const uint4 *>(r < r1 ? a : 0ull);
+            };
+            prefetch(of(r0));
+            prefetch(of(r0 + 1));
+#pragma unroll 1
+            for (int r = r0; r < r1; r += 2) {
+                const uint4 *src[2] = {of(r), of(r + 1)};
+                prefetch(of(r + 2));
+                prefetch(of(r + 3));
+                if (src[0]) gather_row<2>(p, r, src, lane);
+            }
         }
         done += r1 - r0;
         claim = __shfl_sync(0xffffffffu, next, 0);

@@ -184,3 +184,50 @@ def test_kernels_launched_by_a_step(B, N, projection, launches):
     for b in {0, B - 1}:
         ref = O.rpd_step(bits(hidden[:, b].contiguous()), masks[b].numpy(), bits(g), bits(W), 1e-6, 0.9, 1.5, "llada")
         compare_step(ref, got[b], lazy=projection != "all" and got[b]["stats"]["n_rows"] < K * int(masks.sum()))
+
+
+@pytest.mark.parametrize("K,B,N,d,V", [(3, 4, 1000, 72, 300),     # claims of 4 rows, one trip over a row
+                                       (2, 4, 1900, 1048, 300),   # claims of 6, a second trip of 3 vectors
+                                       (16, 2, 700, 64, 256)])    # claims of 8
+def test_claims_of_several_rows_in_a_batch(K, B, N, d, V):
+    """Batches of more rows than two a warp, gathered two at a time; the last claim is a part one."""
+    W, g = WL.make_head(V, d, 17, w_std=0.08)
+    gen = torch.Generator().manual_seed(N)
+    hidden = torch.randn(K, B, N, d, generator=gen).to(torch.bfloat16) * 2
+    masks = torch.stack([WL.uniform_fraction_mask(N, 0.9, 30 + b) for b in range(B)])
+    runner = DeviceRunner(W, g, K)
+    try:
+        got = runner.step_batched(hidden, masks, [0.9] * B, [1.5] * B)
+    finally:
+        runner.close()
+    for b in (0, B - 1):
+        ref = O.rpd_step(bits(hidden[:, b].contiguous()), masks[b].numpy(), bits(g), bits(W), 1e-6, 0.9, 1.5, "llada")
+        compare_step(ref, got[b])
+
+
+def test_many_rows_of_a_batch_are_in_flight_together():
+    """A further row of a large batch costs under 1.2 ns (1.5 with one row a warp at a time)."""
+    B, N, d, V = 8, 1024, 64, 256
+    W, g, _ = make(5, 1, 8, d, V)
+    times = []
+    for K in (4, 16):
+        runner = DeviceRunner(W, g, K)
+        try:
+            hidden = torch.ones(K, B, N, d, dtype=torch.bfloat16, device="cuda")
+            start = torch.ones(B, N, dtype=torch.uint8, device="cuda")
+            mask = start.clone()
+            commit, token = torch.zeros_like(mask), torch.zeros(B, N, dtype=torch.int32, device="cuda")
+            stats = torch.zeros(B, runner.rpd.STATS_WORDS, dtype=torch.int32, device="cuda")
+            best = 1e9
+            for _ in range(100):
+                mask.copy_(start)
+                t0, t1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                t0.record()
+                runner.ctx.step_batched(hidden, mask, [0.9] * B, [1.0] * B, commit, token, stats)
+                t1.record()
+                t1.synchronize()
+                best = min(best, t0.elapsed_time(t1) * 1e6)
+            times.append(best)
+        finally:
+            runner.close()
+    assert (times[1] - times[0]) / (12 * B * N) < 1.2, times

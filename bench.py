@@ -254,19 +254,6 @@ def run_reference(args):
     print(json.dumps(out))
 
 
-def launches_per_step(case, args) -> int:
-    """Stages of one rpd_step / rpd_step_batched call, the most kernels it can launch: the
-    compaction; per projection pass gather/norm, the contraction and the merge; the band
-    selection before a second (lazy) pass; and score/commit where it is not part of the merge.
-    The library runs most of them inside the head kernel; the launches that it makes are counted
-    by rpd_kernel_times."""
-    B = case.get("B", 1)
-    K, N = case["K"], case["N"]
-    second_pass = args.projection == "lazy" or (args.projection == "auto" and K > 1 and K * B * N > 256)
-    fused_score = B == 1 and N <= 2048
-    return 1 + 3 * (2 if second_pass else 1) + (1 if second_pass else 0) + (0 if fused_score else 1)
-
-
 def config_dict(case, R):
     B = case.get("B", 1)
     rule = case["rule"]
@@ -276,7 +263,7 @@ def config_dict(case, R):
             "signal_kappa": case.get("kappa"),
             "projection": "lazy" if "lazy_rows" in case else "all window layers",
             "rows_projected": case.get("lazy_rows", R),
-            "head_tiling": case.get("tiling", "auto (per pass, on the device)"),
+            "head_tiling": case.get("tiling", "auto (per pass, by its row count)"),
             "head_layout": case.get("head_layout", "tiled (context copy of W in contiguous 128 x 64 blocks)"),
             "l2": f"inputs larger than L2: the {2 * case['V'] * case['d'] / 1e9:.2f} GB head is streamed every step"}
 
@@ -913,7 +900,7 @@ def main():
                     help="how the head kernel reads W: the context's tiled copy (default) or the "
                          "caller's row-major tensor in place")
     ap.add_argument("--tiling", choices=["auto", "pair", "rows_n"], default="auto",
-                    help="head contraction tiling (default: chosen per pass on the device)")
+                    help="head contraction tiling (default: chosen per pass by its row count)")
     ap.add_argument("--cpu-positions", type=int, default=16,
                     help="positions of the oracle sample timed for cpu_baseline")
     ap.add_argument("--vocab-parallel", action="store_true",

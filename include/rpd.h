@@ -263,7 +263,7 @@ int rpd_step_batched(rpd_ctx *ctx, const void *hidden, uint8_t *mask, int B, int
 /* rpd_step with HOST buffers: copies hidden, mask and out_token in, runs the step, copies
  * mask, out_commit, out_token and out_stats back, and returns after the stream has finished.
  * mask and out_token are in/out: out_token (the canvas) changes only at committed positions.
- * hidden in pinned (page-locked) host memory is read in place by the step's gather kernel,
+ * hidden in pinned (page-locked) host memory is read in place by the step's kernels,
  * so only the masked positions' rows cross the host link; hidden in other host memory is
  * copied to the device first.  mask, out_token and the results lie in a pinned staging buffer
  * that the step reads and writes in place.
@@ -303,10 +303,11 @@ int rpd_step_shard_finish(rpd_ctx *ctx, const float *gathered, int P, uint8_t *m
  * launch while enabled.  rpd_kernel_times synchronises the recorded events and returns,
  * for each of the RPD_NUM_KERNELS stages (gather/norm, head statistics, merge, score/commit), the
  * summed milliseconds and the launch count since the last reset; reset clears them.  A head
- * statistics launch gathers its rows, merges and, for a single canvas, scores and commits as well;
+ * statistics launch gathers its rows, merges and, for a single canvas of at most 2048 positions,
+ * scores and commits as well;
  * the other stages count the launches that some batches have besides: the compaction (under
  * gather/norm) and the selection of a second pass's positions (under merge) of batches of more
- * than 8192 positions, and score/commit of several canvases. */
+ * than 8192 positions, and score/commit of several canvases or a longer one. */
 #define RPD_NUM_KERNELS 4
 int rpd_profile_enable(rpd_ctx *ctx, int enable);
 int rpd_kernel_times(rpd_ctx *ctx, double *ms /*[RPD_NUM_KERNELS]*/,

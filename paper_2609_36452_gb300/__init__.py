@@ -282,7 +282,7 @@ class Rpd:
         _check(rpd_set_head_layout(self.handle, HEAD_LAYOUTS[layout]))
 
     def set_head_tiling(self, tiling):
-        """Tiling of the head contraction: "auto" (default, chosen per pass on the device),
+        """Tiling of the head contraction: "auto" (default, chosen per pass by its row count),
         "pair" (256-row x 256-entry tiles on CTA pairs) or "rows_n" (256 entries x row groups
         of up to 512 rows, padded to 32); for tests and measurements."""
         _check(rpd_set_head_tiling(self.handle, HEAD_TILINGS[tiling]))

@@ -1,5 +1,5 @@
 // head_plan.h - the choice of the head kernel's tiling and vocabulary split count for a
-// projection pass of `rows` rows (host and device).  It changes no computed quantity, only
+// projection pass of `rows` rows, and the order of its work units (host and device).  It changes no computed quantity, only
 // how the contraction is laid out on the GPU.
 //
 // It is evaluated on the host: for passes of up to kStepPlanRows rows into an argument of the head
@@ -209,6 +209,51 @@ inline void fill_step_plan(StepPlan &p, int max_rows, Plan plan) {
         p.est[i] = hp.est;
     }
 }
+
+// Work units (row tile m, vocabulary split g) in the order the persistent CTAs take them:
+// row tiles are grouped into bands of `band` tiles; inside a band m runs fastest, then g.
+// The units running at the same time therefore share W tiles (each streamed from HBM once
+// per band) and re-read at most `band` u tiles (kept in L2 while the band runs).  With few
+// row tiles there is a single band and the order is plain (m fastest).
+// With a split tail every unit is one tile, and those after the last whole wave are half tiles.
+struct TileWalk {
+    int num_m, num_n, splits, units, band;
+    int whole;  // units before the half tiles
+    __host__ __device__ __forceinline__ void init(int rows, int tile_rows, int V, int d, int g, bool tail, int pairs) {
+        num_m = (rows + tile_rows - 1) / tile_rows;
+        num_n = (V + kTileN - 1) / kTileN;
+        splits = tail ? num_n : g;
+        units = num_m * splits;
+        whole = units;
+        if (tail) {
+            const TailSplit t = tail_split(units, pairs);
+            whole = t.whole;
+            units = t.units;
+        }
+        band = static_cast<int>(kBandBytes / 2) / tile_rows / d;
+        band = band < num_m ? band : num_m;
+        band = band > 1 ? band : 1;
+    }
+    // A unit's vocabulary range is given in half tiles [v0, v1); an odd one is a half tile.
+    __host__ __device__ __forceinline__ void unit(int u, int &m, int &g, int &v0, int &v1) const {
+        const int half = u - whole;  // of tile whole + half / 2
+        if (half >= 0) u = whole + (half >> 1);
+        const int per_band = band * splits;
+        const int b = u / per_band;
+        const int r = u - b * per_band;
+        const int m0 = b * band;
+        const int in_band = band < num_m - m0 ? band : num_m - m0;
+        m = m0 + r % in_band;
+        g = r / in_band;
+        // at most a few hundred splits of at most 2^23 tiles: the products fit 32 bits
+        v0 = 2 * static_cast<int>(static_cast<unsigned>(g) * num_n / splits);
+        v1 = 2 * static_cast<int>(static_cast<unsigned>(g + 1) * num_n / splits);
+        if (half >= 0) {
+            v0 += half & 1;
+            v1 = v0 + 1;
+        }
+    }
+};
 
 // The plan of a pass from plan_head's (a function of the multiple of 32 rows).
 inline HeadPlan refine_plan(const HeadPlan &plan, long long rows, const HeadPlanInputs &in) {

@@ -40,50 +40,6 @@ namespace {
 constexpr uint32_t kTmemCols = 2 * kTileN;
 constexpr float kLog2e = 1.4426950408889634f;
 
-// Work units (row tile m, vocabulary split g) in the order the persistent CTAs take them:
-// row tiles are grouped into bands of `band` tiles; inside a band m runs fastest, then g.
-// The units running at the same time therefore share W tiles (each streamed from HBM once
-// per band) and re-read at most `band` u tiles (kept in L2 while the band runs).  With few
-// row tiles there is a single band and the order is plain (m fastest).
-// With a split tail every unit is one tile, and those after the last whole wave are half tiles.
-struct TileWalk {
-    int num_m, num_n, splits, units, band;
-    int whole;  // units before the half tiles
-    __device__ __forceinline__ void init(int rows, int tile_rows, int V, int d, int g, bool tail) {
-        num_m = (rows + tile_rows - 1) / tile_rows;
-        num_n = (V + kTileN - 1) / kTileN;
-        splits = tail ? num_n : g;
-        units = num_m * splits;
-        whole = units;
-        if (tail) {
-            const TailSplit t = tail_split(units, gridDim.x / 2);
-            whole = t.whole;
-            units = t.units;
-        }
-        band = static_cast<int>(kBandBytes / 2) / tile_rows / d;
-        band = max(1, min(num_m, band));
-    }
-    // A unit's vocabulary range is given in half tiles [v0, v1); an odd one is a half tile.
-    __device__ __forceinline__ void unit(int u, int &m, int &g, int &v0, int &v1) const {
-        const int half = u - whole;  // of tile whole + half / 2
-        if (half >= 0) u = whole + (half >> 1);
-        const int per_band = band * splits;
-        const int b = u / per_band;
-        const int r = u - b * per_band;
-        const int m0 = b * band;
-        const int in_band = min(band, num_m - m0);
-        m = m0 + r % in_band;
-        g = r / in_band;
-        // at most a few hundred splits of at most 2^23 tiles: the products fit 32 bits
-        v0 = 2 * static_cast<int>(static_cast<unsigned>(g) * num_n / splits);
-        v1 = 2 * static_cast<int>(static_cast<unsigned>(g + 1) * num_n / splits);
-        if (half >= 0) {
-            v0 += half & 1;
-            v1 = v0 + 1;
-        }
-    }
-};
-
 // Work units are claimed at run time from a per-pass counter (meta[kMetaUnitNext]) by the
 // TMA producer, in the walk's order, so the units in flight are always a window of
 // consecutive indices however the CTAs' speeds differ.  The producer passes each claimed
@@ -365,10 +321,10 @@ __device__ __forceinline__ int copy_ahead(const HeadParams &p, const HeadSmem &s
 
 // The TMA producer of one CTA (one thread).
 //
-// With a single row tile every head tile is read once and is dropped from L2 first, which keeps
-// the hidden rows, the partials and the code of the step's other phases there from one step to
-// the next: 171.5 -> 166.4 us at 20 rows (LLaDA head), of which 3 us after the last tile.  Several
-// row tiles re-read a head tile at slightly different times: with that policy, and with an
+// With a single row tile every head tile is read once and is dropped from L2 first, which leaves the
+// hidden rows, the partials and the code of the step's later phases there: at 20 rows (LLaDA head)
+// 181.8 -> 178.6 us where 1 GB of other traffic lies between two steps, as a forward pass would, and
+// 164.2 -> 163.4 where step follows step.  Several row tiles re-read a head tile at slightly different times: with that policy, and with an
 // explicit normal one instead of none, first-step and serving passes were 1.5 % slower.
 __device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm, const Copies &c,
                                         uint32_t rank, const TileWalk &tw, int rows, int num_kb, int first) {
@@ -1094,7 +1050,7 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         const int num_kb = (p.d + kTileK - 1) / kTileK;
         TileWalk tw;
         const bool tail = pair && pass.swap_rows == kSplitTail;
-        tw.init(pass.rows, ng, p.V, p.d, splits, tail);
+        tw.init(pass.rows, ng, p.V, p.d, splits, tail, gridDim.x / 2);
         if (warp == 0) {
             if (lane == 0 && !p.stall) {
                 // this CTA's half of the tile's rows, one copy (rows on N: the map whose box is half

@@ -468,7 +468,6 @@ int run_step(rpd_ctx *c, const void *hidden, uint8_t *mask, int B, int N, const 
     const MergeArgs mg{c->partials, c->max_splits, c->row_arg, c->row_pmax, c->row_H};
     auto pass = [&](const int32_t *sel_list, bool last) -> cudaError_t {
         KernelTimer t(c, 1);
-        // The kernel reads the tiling chosen on the device for this pass.
         HeadParams hp = head_params(c, cp, hidden, sel_list, from_mask && !sel_list, last, mg);
         hp.score = sp;
         hp.score_canvas = fuse_score && (last || from_mask) ? 1 : 0;
@@ -882,7 +881,7 @@ int rpd_step_host(rpd_ctx *c, const void *hidden, uint8_t *mask, int N, float ta
         return fail(RPD_ERR_INVALID_ARGUMENT, "null buffer");
     DeviceGuard dg(c->device);
     if (dg.err != cudaSuccess) return cuda_fail(dg.err, "cudaSetDevice");
-    // Pinned (page-locked, mapped) host memory is read in place by the gather kernel over the
+    // Pinned (page-locked, mapped) host memory is read in place by the head kernel over the
     // host link: only the masked positions' rows cross it, and no copy precedes the step.
     // Any other host memory is copied to the device first.
     const void *in_place = nullptr;

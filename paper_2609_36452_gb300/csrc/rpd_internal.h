@@ -161,9 +161,6 @@ struct CompactParams {
 // first pass (the real band is known only after it).
 constexpr float kLazyBandGuess = 0.25f;
 
-// Second pass of lazy projection: selects the positions whose final confidence lies in the
-// stability band theta_c <= c < tau of their canvas and sets up the pass over their earlier
-// window layers (tiling, split count, row mapping).
 // Where merged per-row statistics go: split partials (log2 units) in, argmax / max
 // probability / entropy per (layer, compact position) out, at layer * NMT + q.
 struct MergeArgs {
@@ -193,6 +190,9 @@ struct ShardMergeParams {
     float *row_H;
 };
 
+// Second pass of lazy projection, of batches that the head kernel does not compact itself: selects the
+// positions whose final confidence lies in the stability band theta_c <= c < tau of their canvas and
+// sets up the pass over their earlier window layers (tiling, split count, row mapping).
 struct BandParams {
     int32_t *meta;
     MergeArgs mg;              // merged first-pass statistics (final-layer confidences)
@@ -360,7 +360,7 @@ inline const char *call_error(const rpd_rule &r, float tau, float budget) {
 }
 
 // Memory the kernels read with TMA (the head, the gain) must be device or managed memory of
-// `device`; memory the gather kernel reads with plain loads (hidden states) may also be
+// `device`; memory the head kernel gathers with plain loads (hidden states) may also be
 // page-locked host memory mapped into the device's address space.  Any other pointer - pageable
 // host memory, another device's memory - would make the kernels fault, so it is refused.
 inline bool pointer_usable(const void *p, int device, bool host_mapped_ok) {
@@ -375,18 +375,18 @@ inline bool pointer_usable(const void *p, int device, bool host_mapped_ok) {
 
 cudaError_t launch_compact(const CompactParams &p, cudaStream_t s);
 // Tensor maps of the head kernel's operands (128-byte swizzling, K boxes of 64): u in boxes of
-// 128 rows (pair tiles) and, for the rows-on-N tiles, in boxes of 16, 32, ..., 128 rows (one
-// per half-group height, so that a stage copies each MMA's share of u with one instruction:
+// 128 rows (pair tiles) and, for the rows-on-N tiles, in boxes of 16, 32, ..., 256 rows (one
+// per half-group height, so that a stage copies a CTA's half of the group with one instruction:
 // the TMA unit's time per copy, not its bytes, bounded a stage built from 16-row boxes); W in
-// boxes of 128 rows.
+// boxes of 128 rows, and of 64 for half tiles.
 constexpr int kUMaps = (kSwapMaxRows / 2) / kUBoxRows;  // box heights kUBoxRows * (1 .. kUMaps)
 struct HeadMaps {
     CUtensorMap u;                // box 64 x 128 rows
     CUtensorMap w128, w64;        // boxes 64 x 128 and 64 x 64 rows of W
     CUtensorMap u_rows[kUMaps];   // u_rows[j]: box 64 x kUBoxRows*(j+1) rows
 };
-// The head kernel (every tiling; the pass's choice is read from the meta words), launched as
-// `grid` CTAs in clusters of two, one per SM.
+// The head kernel (every tiling; the pass's is looked up by its row count, or read from the meta words
+// where another kernel set the pass up), launched as `grid` CTAs in clusters of two, one per SM.
 cudaError_t launch_head(const HeadMaps &maps, const HeadParams &p, int grid, cudaStream_t s);
 // Copy W [V][d] (d % 64 == 0) into blocks of 128 rows x 64 columns, block (t, k) at element
 // ((t * (d / 64) + k) * 128) * 64, rows past V zero; Wt holds ceil(V/128)*128*d elements.

@@ -220,7 +220,7 @@ extern "C" int rpd_step_noalloc(const void *W_head, const void *g_norm, int d, i
     int32_t *pos_of_q = reinterpret_cast<int32_t *>(A + kOffPosOfQ);
     int32_t *meta = reinterpret_cast<int32_t *>(A + kOffMeta);
 
-    // Same head-kernel configuration as rpd_step (tiling chosen on the device).
+    // Same head-kernel configuration as rpd_step.
     const int pair_slots = dev->head_grid / 2;
     HeadMaps maps;
     bool maps_ok = encode_tile_map(&maps.u, u, kNaMaxRows, static_cast<uint64_t>(d), kTileM) &&

@@ -231,3 +231,24 @@ def test_many_rows_of_a_batch_are_in_flight_together():
         finally:
             runner.close()
     assert (times[1] - times[0]) / (12 * B * N) < 1.2, times
+
+
+@pytest.mark.parametrize("N", [2048, 2049, 8192])
+def test_host_buffers_of_long_canvases(N):
+    """rpd_step_host equals rpd_step on both sides of the length up to which the head kernel scores."""
+    K, d, V = 2, 64, 512
+    W, g, hidden = make(30 + N, K, N, d, V)
+    runner = DeviceRunner(W, g, K)
+    try:
+        for count in (N, 700, 1):
+            mask = torch.zeros(N, dtype=torch.uint8)
+            mask[N - count:] = 1
+            want = runner.step(hidden, mask, 0.9, 1.0)
+            m, commit = mask.clone(), torch.full((N,), 7, dtype=torch.uint8)
+            token = torch.full((N,), -5, dtype=torch.int32)
+            stats = torch.zeros(runner.rpd.STATS_WORDS, dtype=torch.int32)
+            runner.ctx.step_host(hidden.pin_memory(), m, 0.9, 1.0, commit, token, stats)
+            assert (commit.numpy() == want["commit"]).all() and (token.numpy() == want["token"]).all()
+            assert (m.numpy() == want["new_mask"]).all() and runner.rpd.stats_dict(stats) == want["stats"]
+    finally:
+        runner.close()

@@ -1,6 +1,7 @@
 """The plans that a step passes to the head kernel (StepPlan, one entry per 32 rows) are those of
-every row count up to its limit, and the search over split counts finds what trying each of them
-does, at the two models' heads, small and ragged ones (no GPU)."""
+every row count up to its limit, the work units of each plan cover its pass exactly once, and the
+search over split counts finds what trying each of them does, at the two models' heads, small and
+ragged ones (no GPU)."""
 import os
 import shutil
 import subprocess
@@ -14,6 +15,7 @@ DRIVER = r"""
 #include "head_plan.h"
 #include <cstdio>
 #include <cstdlib>
+#include <vector>
 // every split count in turn
 static unsigned long long every_key(float cost1, int tiles, int slots, int num_n, int gmax) {
     unsigned long long key = ~0ull;
@@ -40,15 +42,47 @@ int main(int argc, char **argv) {
         std::printf("%d %d %d\n", a.mode, a.splits, a.swap_rows);
         return 0;
     }
-    auto plan = [&](int r) { return rpd::regroup_plan(rpd::plan_head(r, in), r, in); };
+    auto plan = [&](int r) { return rpd::refine_plan(rpd::plan_head(r, in), r, in); };
     rpd::StepPlan sp;
     rpd::fill_step_plan(sp, rpd::kStepPlanRows, plan);
     int bad = 0;
-    for (int r = 1; r <= 4096; ++r) {  // regrouping keeps the plan's rules at every row count
+    int tails = 0;
+    for (int r = 1; r <= 4096; ++r) {  // refining keeps the plan's rules at every row count
+        const rpd::HeadPlan a = plan(r);
+        const bool rows_n = a.mode == rpd::kHeadModeRowsN, tail = !rows_n && a.swap_rows == rpd::kSplitTail;
+        const int splits = rows_n || tail ? a.splits / 2 : a.splits;
+        tails += tail;
+        bad += splits < 1 || splits > in.num_n || a.splits > in.max_splits || a.est != rpd::plan_head(r, in).est;
+        bad += !rows_n && a.swap_rows != (tail ? rpd::kSplitTail : 0);
+        bad += tail && (a.splits != 2 * in.num_n || force != RPD_TILING_AUTO);
+        if (r > 64 && r % 32 > 1) continue;
+        // the units of the pass: every half tile of every row tile once, every partial of a row once
+        const int ng = rows_n ? a.swap_rows : rpd::kPairTileM, tiles = (r + ng - 1) / ng;
+        rpd::TileWalk tw;
+        tw.init(r, ng, V, d, rows_n ? a.splits / 2 : a.splits, tail, in.pair_slots);
+        bad += tw.num_m != tiles;
+        std::vector<int> halves(static_cast<size_t>(tiles) * 2 * in.num_n), slots(static_cast<size_t>(tiles) * a.splits);
+        for (int u = 0; u < tw.units; ++u) {
+            int m, g, v0, v1;
+            tw.unit(u, m, g, v0, v1);
+            if (m < 0 || m >= tiles || v0 < 0 || v1 <= v0 || v1 > 2 * in.num_n) return !std::printf("1\n");
+            bad += v0 + 1 == v1 ? !tail || u < tw.whole : (v0 | v1) & 1;  // half tiles in the tail only
+            for (int v = v0; v < v1; ++v) ++halves[static_cast<size_t>(m) * 2 * in.num_n + v];
+            const int first = rows_n ? 2 * g : tail ? v0 : g, n = rows_n ? 2 : tail ? v1 - v0 : 1;
+            for (int s = first; s < first + n; ++s) {
+                if (s >= a.splits) return !std::printf("1\n");
+                ++slots[static_cast<size_t>(m) * a.splits + s];
+            }
+        }
+        for (int h : halves) bad += h != 1;
+        for (int s : slots) bad += s != 1;
+        const int rest = tiles * in.num_n % in.pair_slots;  // two half tiles to each pair at most
+        bad += tail && (rest == 0 || 2 * rest > in.pair_slots || tw.units - tw.whole != 2 * rest);
+    }
+    bad += (force != RPD_TILING_AUTO || 2 * in.num_n > in.max_splits) && tails > 0;
+    for (int r = 1; r <= 4096; ++r) {
         const rpd::HeadPlan a = plan(r);
         const bool rows_n = a.mode == rpd::kHeadModeRowsN;
-        const int splits = rows_n ? a.splits / 2 : a.splits;
-        bad += splits < 1 || splits > in.num_n || a.splits > in.max_splits || a.est != rpd::plan_head(r, in).est;
         bad += rows_n && (a.swap_rows % 32 || a.swap_rows < 32 || a.swap_rows > 512);
         bad += force == RPD_TILING_PAIR && rows_n;
         bad += force == RPD_TILING_ROWS_N && !rows_n && in.max_splits >= 2;

@@ -946,7 +946,8 @@ struct DeviceWords {
 
 // The head kernel: one launch per projection pass, clusters of two CTAs, one CTA per SM.  It
 // compacts the mask (or reads the pass from the meta words), gathers and normalises the pass's
-// rows, contracts them with the head, merges the splits' statistics and scores a single canvas.
+// rows, contracts them with the head, merges the splits' statistics and scores a single canvas of at
+// most kFuseScoreMaxN positions.
 template <bool kPlain>
 __global__ void __launch_bounds__(kHeadKernelThreads, 1)
     k_head(const __grid_constant__ HeadMaps maps, const __grid_constant__ HeadParams p) {

@@ -1,12 +1,13 @@
 // k_merge_commit.cu - the step's small kernels: the lazy projection's band selection, the scoring
-// of several canvases, the merge of vocabulary shards and the decoding loop's stop test.
+// of several canvases or a long one, the merge of vocabulary shards and the decoding loop's stop test.
 //
 // k_band (one CTA; lazy projection of batches that the head kernel does not compact itself): selects
 //   the positions whose final confidence lies in their canvas's stability band theta_c <= c < tau
 //   (Eq. 5 reads S_i only there) and sets up the second pass over their earlier window layers.
 //
-// k_score_commit (one CTA per canvas): scores and commits several canvases (score_canvas in
-//   step_epilogue.cuh; a single canvas is scored by the head kernel itself).
+// k_score_commit (one CTA per canvas): scores and commits several canvases, or one of more than
+//   kFuseScoreMaxN positions (score_canvas in step_epilogue.cuh; any other single canvas is scored by
+//   the head kernel itself).
 #include "ptx.cuh"
 #include "rpd_internal.h"
 #include "step_common.cuh"

@@ -3,7 +3,7 @@
 // scan and commitment of a canvas (§3).
 //
 // The head kernel runs both after its last tile: its CTAs claim blocks of rows to merge, and the
-// one that completes the merge scores the canvas (a single canvas; several are scored by
+// one that completes the merge scores the canvas (a single one; several, and a long one, are scored by
 // k_score_commit, a CTA each).
 //
 // Both parts are bound by latency: a handful of dependent trips to L2 and, because the head's

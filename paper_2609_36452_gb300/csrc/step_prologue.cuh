@@ -251,9 +251,9 @@ __device__ __forceinline__ int rows_per_claim(int rows, int warps) {
 // warp.  Compact index -> position through `map`, or through the lists in global memory when
 // num_words is 0.  The rows are counted once the warp has no more of them.
 //
-// kPlain: the plain step, of few rows: one at a time.  The general kernel, whose batches have tens of
-// thousands, finds the positions of a claim's rows in as many lanes and keeps two rows in flight: one
-// after another a row took a warp 0.78 us of waiting.
+// kPlain (the plain step), or a row a claim: one at a time.  The general kernel, whose batches have tens
+// of thousands, finds the positions of a claim's rows in as many lanes and keeps two rows in flight: one
+// after another a row took a warp 0.78 us of waiting (131072 rows of d = 64, 256 entries: 201 us, now 123).
 template <bool kPlain>
 __device__ __forceinline__ void gather_rows(const NormParams &p, const MaskMap &map, int num_words,
                                             int rows, int sel, int layer0, int claim, int per_claim,
@@ -282,7 +282,7 @@ __device__ __forceinline__ void gather_rows(const NormParams &p, const MaskMap &
         const int r0 = claim * per_claim, r1 = min(rows, r0 + per_claim);
         int next = 0;
         if (lane == 0) next = atomicAdd(&meta[kMetaRowNext], 1);  // its latency hides behind the rows
-        if (kPlain) {
+        if (kPlain || per_claim == 1) {
             const uint4 *src[1] = {source(r0)};
             prefetch(src[0]);
 #pragma unroll 1

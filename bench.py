@@ -44,11 +44,11 @@ HEAD_SOURCES = ("paper_2609_36452_gb300/csrc/k_head_stats.cu", "paper_2609_36452
                 "paper_2609_36452_gb300/csrc/ptx.cuh", "paper_2609_36452_gb300/csrc/rpd_internal.h",
                 "paper_2609_36452_gb300/csrc/head_plan.h")
 HEAD_TRAFFIC = {
-    ("llada_first_step", "23a00819a2c32d97"): 1.0996e9,
-    ("llada_tail_70_masked", "23a00819a2c32d97"): 1.0434e9,
-    ("llada_tail_5_masked", "23a00819a2c32d97"): 1.0396e9,
-    ("dream_mid_decode", "23a00819a2c32d97"): 1.1024e9,
-    ("batched_serving", "23a00819a2c32d97"): 9.5494e9,
+    ("llada_first_step", "e0020a2e9beee1d6"): 1.0996e9,
+    ("llada_tail_70_masked", "e0020a2e9beee1d6"): 1.0434e9,
+    ("llada_tail_5_masked", "e0020a2e9beee1d6"): 1.0396e9,
+    ("dream_mid_decode", "e0020a2e9beee1d6"): 1.1024e9,
+    ("batched_serving", "e0020a2e9beee1d6"): 9.5494e9,
 }
 
 # Nominal dense rates of GB300 (context only; the fractions use the measured peaks).

@@ -324,8 +324,9 @@ __device__ __forceinline__ int copy_ahead(const HeadParams &p, const HeadSmem &s
 // With a single row tile every head tile is read once and is dropped from L2 first, which leaves the
 // hidden rows, the partials and the code of the step's later phases there: at 20 rows (LLaDA head)
 // 181.8 -> 178.6 us where 1 GB of other traffic lies between two steps, as a forward pass would, and
-// 164.2 -> 163.4 where step follows step.  Several row tiles re-read a head tile at slightly different times: with that policy, and with an
-// explicit normal one instead of none, first-step and serving passes were 1.5 % slower.
+// 164.2 -> 163.4 where step follows step.  Several row tiles re-read a head tile at slightly different
+// times: with that policy, and with an explicit normal one instead of none, first-step and serving
+// passes were 1.5 % slower.
 __device__ __forceinline__ void produce(const HeadParams &p, const HeadSmem &sm, const Copies &c,
                                         uint32_t rank, const TileWalk &tw, int rows, int num_kb, int first) {
     const uint32_t full0 = mapa_shared(smem_u32(&sm.full[0]), 0);
@@ -1089,7 +1090,8 @@ __global__ void __launch_bounds__(kHeadKernelThreads, 1)
         DeviceWords words{p.meta};
         if (last_to_leave(words, gridDim.x)) {
             __threadfence();
-            if (kind.from_mask() && kind.scores()) clear_later = *reinterpret_cast<volatile int32_t *>(&p.meta[kMetaClearLater]);
+            if (kind.from_mask() && kind.scores())
+                clear_later = *reinterpret_cast<volatile int32_t *>(&p.meta[kMetaClearLater]);
             zero_counters(words);
             if (!kPlain && p.last_pass) p.meta[kMetaScored] = 0;
             if (kPlain || p.last_pass) p.meta[kMetaStepStatus] = atomicExch(&p.meta[kMetaStatus], RPD_OK);

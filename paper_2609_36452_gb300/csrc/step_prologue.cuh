@@ -295,7 +295,8 @@ __device__ __forceinline__ void gather_rows(const NormParams &p, const MaskMap &
         } else {
             const uint4 *mine = lane < r1 - r0 ? source(r0 + lane) : nullptr;  // at most 8 rows
             auto of = [&](int r) {  // of row r, in every lane
-                const unsigned long long a = __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(mine), (r - r0) & 31);
+                const unsigned long long a =
+                    __shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(mine), (r - r0) & 31);
                 return reinterpret_cast<const uint4 *>(r < r1 ? a : 0ull);
             };
             prefetch(of(r0));
